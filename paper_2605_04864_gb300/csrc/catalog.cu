@@ -369,126 +369,270 @@ __global__ void k_scatter(const P* __restrict__ pos, const P* __restrict__ w, in
   }
 }
 
-// Per-axis taps of one phase: up to 3 (TSC) or 2 (CIC) tile cells with weights, from the
-// stored fraction and decision bits.
-template <int ASSIGN, typename T>
-__device__ __forceinline__ void axis_taps(T frac, uint32_t m8, int phase, int* idx, T* wt) {
+// Per-axis taps of one phase: up to 3 (TSC) or 2 (CIC) cells with weights, from the stored fraction
+// and decision bits.  Returns the first tap's tile index; the others follow it.  The rounding of the
+// middle float weight 3/4 - d^2 is spelled out (FUSED: the square is not rounded by itself), so that
+// the mesh does not depend on which products the compiler fuses.
+__device__ __forceinline__ float middle_weight(float d, bool fused) {
+  return fused ? fmaf(-d, d, 0.75f) : __fsub_rn(0.75f, __fmul_rn(d, d));
+}
+__device__ __forceinline__ double middle_weight(double d, bool) { return 0.75 - d * d; }
+
+template <int ASSIGN, typename T, bool FUSED = true>
+__device__ __forceinline__ int axis_taps(T frac, uint32_t m8, int phase, T* wt) {
   const int local = (int)(m8 & 31u);
   const int off = phase ? (int)((m8 >> 6) & 3u) : (int)((m8 >> 5) & 1u);
   // d = s - centre (phase a) or (s + 1/2) - centre (phase b)
   const T d = frac + (phase ? T(0.5) : T(0)) - T(off);
   const int rel = local + off + 1;   // tile index of the centre (tile starts one cell below the brick)
   if (ASSIGN == 2) {
-    idx[0] = rel; wt[0] = T(1) - d;
-    idx[1] = rel + 1; wt[1] = d;
-  } else {
-    const T a = T(0.5) - d, b = T(0.5) + d;
-    idx[0] = rel - 1; wt[0] = T(0.5) * a * a;
-    idx[1] = rel; wt[1] = T(0.75) - d * d;
-    idx[2] = rel + 1; wt[2] = T(0.5) * b * b;
+    wt[0] = T(1) - d;
+    wt[1] = d;
+    return rel;
   }
+  const T a = T(0.5) - d, b = T(0.5) + d;
+  wt[0] = T(0.5) * a * a;
+  wt[1] = middle_weight(d, FUSED);
+  wt[2] = T(0.5) * b * b;
+  return rel - 1;
 }
 
-// Round to the nearest 64-bit integer (ties to even).  The float path takes |v| < 2^43 (the tile
-// kernel's scale guarantees it) and needs no conversion instruction: hi = rn(v / 2^22) and the exact
-// remainder lo = v - 2^22 hi, both of magnitude <= 2^21, are rounded to integers by adding 1.5 * 2^23
-// (the float add rounds to nearest even, and the integer sits in the low mantissa bits); since
-// 2^22 hi is an even integer, 2^22 hi + rn(lo) = rn(v).
-template <typename T> __device__ __forceinline__ long long to_fixed(T v);
-template <> __device__ __forceinline__ long long to_fixed<float>(float v) {
-  const float magic = 12582912.0f;                         // 1.5 * 2^23
-  const float th = v * 2.384185791015625e-07f + magic;     // rn(v 2^-22) + magic
-  const float hf = th - magic;                             // exact
-  const float lf = fmaf(hf, -4194304.0f, v);               // v - 2^22 hi, exact
-  const float tl = lf + magic;
-  const int hi = __float_as_int(th) - 0x4B400000;
-  const int lo = __float_as_int(tl) - 0x4B400000;
-  return (long long)hi * 4194304LL + (long long)lo;
+// Pairs of floats in one 64-bit register: the packed add, multiply and fused multiply-add of this
+// architecture round each half as the scalar instruction does and issue once for both.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
 }
-template <> __device__ __forceinline__ long long to_fixed<double>(double v) { return __double2ll_rn(v); }
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// Two float tap values as integer parts: |v| < 2^43 (the tile kernel's scale guarantees it),
+// rn(v) = 2^22 h + l with |h|, |l| <= 2^21, without a conversion instruction: h = rn(v / 2^22) and the
+// exact remainder v - 2^22 h are rounded to integers by adding 1.5 * 2^23 (the float add rounds to
+// nearest even, and the integer sits in the low mantissa bits); since 2^22 h is an even integer,
+// 2^22 h + rn(remainder) = rn(v).
+__device__ __forceinline__ void fixed_parts2(f32x2 v, int (&h)[2], int (&l)[2]) {
+  const f32x2 magic = pack2(12582912.0f, 12582912.0f);                                       // 1.5 * 2^23
+  const f32x2 th = fma2(v, pack2(2.384185791015625e-07f, 2.384185791015625e-07f), magic);   // rn(v 2^-22) + magic
+  const f32x2 hf = add2(th, pack2(-12582912.0f, -12582912.0f));                              // exact
+  const f32x2 tl = add2(fma2(hf, pack2(-4194304.0f, -4194304.0f), v), magic);                // (v - 2^22 h) + magic
+  float a, b;
+  unpack2(th, a, b);
+  h[0] = __float_as_int(a) - 0x4B400000;
+  h[1] = __float_as_int(b) - 0x4B400000;
+  unpack2(tl, a, b);
+  l[0] = __float_as_int(a) - 0x4B400000;
+  l[1] = __float_as_int(b) - 0x4B400000;
+}
 
 // 64-bit fixed point back to T times 2^-e; the float path uses two 32-bit conversions.
-template <typename T> __device__ __forceinline__ T from_fixed(long long q, T inv);
-template <> __device__ __forceinline__ float from_fixed<float>(long long q, float inv) {
+__device__ __forceinline__ float from_fixed(long long q, float inv) {
   const int hi = (int)(q >> 32);
   const unsigned lo = (unsigned)(q & 0xffffffffull);
   return fmaf((float)hi, 4294967296.0f, (float)lo) * inv;
 }
-template <> __device__ __forceinline__ double from_fixed<double>(long long q, double inv) { return (double)q * inv; }
+__device__ __forceinline__ double from_fixed(long long q, double inv) { return (double)q * inv; }
 
-// One CTA per (brick, phase): fixed-point accumulation of all taps in a (bs+4)^3 tile.
-template <int ASSIGN, typename R, typename T>
-__global__ void __launch_bounds__(512)
-k_paint_brick(const typename RecOf<R>::type* __restrict__ rec, const uint32_t* __restrict__ meta,
-              const int* __restrict__ start, const int* __restrict__ count, PaintGeo g, int nphase,
-              const double* __restrict__ sc, int maxw_slot, T* __restrict__ tiles) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  long long* acc = reinterpret_cast<long long*>(smem_raw);
-  const int ts3 = g.ts * g.ts * g.ts;
-  const int b = blockIdx.x / nphase, ph = blockIdx.x % nphase;
-  for (int i = threadIdx.x; i < ts3; i += blockDim.x) acc[i] = 0;
-  const int cnt = count[b];
-  // fixed-point scale 2^e with cnt * max|w| * 2^e < 2^61 (no overflow of the tile sums)
-  const double bound = (double)cnt * sc[maxw_slot];
-  int ex = 0;
-  if (bound > 0) frexp(bound, &ex);
-  int e = 61 - ex;
-  if constexpr (sizeof(T) == 4) {
-    // and every tap |w W| 2^e < 2^43, the range of the float conversion
-    int exw = 0;
-    if (sc[maxw_slot] > 0) frexp(sc[maxw_slot], &exw);
-    e = min(e, 43 - exw);
+// The tile sums are 64-bit integers, but shared memory has no native 64-bit atomic add (it runs as a
+// compare-and-swap loop: 21 cycles per warp instruction measured here), so every sum is kept as two
+// 32-bit words with native adds:
+//   float, at most NARROW_MAX objects in the brick: sums of the h and of the l parts, two adds without
+//     a return value; no word can overflow (1023 * 2^21 < 2^31).  10 cycles at 671 objects.
+//   float, more objects: the adds return the old word, so that an overflow of l is carried into h
+//     (2^32 = 1024 * 2^22) and one of h into the cell's signed byte of a third array (the whole sum is
+//     below 2^60, so h overflows at most 2^38 / 2^32 = 64 times either way).  9 cycles at 20,000
+//     objects, where the tile's clearing and writing no longer count.
+//   double: low and high halves of the 64-bit integer, the high add taking the carry of the low one.
+constexpr int NARROW_MAX = 1023;
+__device__ __forceinline__ bool add_overflows(int old, int q) {
+  const int now = (int)((unsigned)old + (unsigned)q);
+  return ((old ^ now) & (q ^ now)) < 0;
+}
+template <bool WIDE>
+__device__ __forceinline__ void tile_add(int* lo, int* hi, unsigned* top, int idx, int h, int l) {
+  if constexpr (!WIDE) {
+    atomicAdd(lo + idx, l);
+    atomicAdd(hi + idx, h);
+  } else {
+    if (add_overflows(atomicAdd(lo + idx, l), l)) h += l < 0 ? -1024 : 1024;
+    if (add_overflows(atomicAdd(hi + idx, h), h)) atomicAdd(top + (idx >> 2), (h < 0 ? 0xffffffffu : 1u) << (8 * (idx & 3)));
   }
-  const T scale = (T)ldexp(1.0, e);
-  __syncthreads();
-  const int beg = start[b];
+}
+__device__ __forceinline__ void tile_add(int* lo, int* hi, int idx, double v) {
+  const long long q = __double2ll_rn(v);
+  const unsigned ql = (unsigned)q;
+  const unsigned old = atomicAdd(reinterpret_cast<unsigned*>(lo) + idx, ql);
+  const int h = (int)(q >> 32) + (old + ql < old ? 1 : 0);
+  if (h != 0) atomicAdd(hi + idx, h);
+}
+
+// Sum of cell idx from its words.  The bytes of `top` hold signed digits that borrowed from their
+// upper neighbours: digit d is the sign-extended low byte once the digits below it are taken out.
+template <typename T>
+__device__ __forceinline__ long long tile_sum(int lo, int hi, unsigned topw, int digit) {
+  if constexpr (sizeof(T) == 8) return ((long long)hi << 32) | (unsigned)lo;
+  int d = 0;
+  if (topw != 0u) {
+    for (int k = 0; k <= digit; ++k) {
+      d = (int)(signed char)(topw & 0xffu);
+      topw = (topw - (unsigned)d) >> 8;
+    }
+  }
+  return (((long long)d << 32) + hi) * 4194304LL + lo;
+}
+
+// Every tap of the brick's objects into the tile words.
+template <int ASSIGN, typename T, int BS, bool WIDE>
+__device__ __forceinline__ void tile_taps(const typename RecOf<T>::type* __restrict__ rec,
+                                          const uint32_t* __restrict__ meta, int cnt, int ph, T scale, int* lo, int* hi,
+                                          unsigned* top) {
+  constexpr int TS = BS + 4;
   constexpr int NT = ASSIGN == 2 ? 2 : 3;
   // NT adjacent lanes share one object, lane xt taking its x tap: the atomics of one instruction
-  // then hit runs of NT neighbouring cells instead of 32 scattered ones (fewer bank wavefronts)
+  // then hit runs of NT neighbouring cells instead of 32 scattered ones (fewer bank wavefronts; nine
+  // lanes per object, x and y, measured 1.6 times slower: three times the record decoding per tap)
   constexpr int OPW = 32 / NT;   // objects per warp and pass
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   const int xt = lane % NT, slot = lane / NT;
   for (int k0 = warp * OPW; k0 < cnt; k0 += nwarp * OPW) {
     const int k = k0 + slot;
     if (slot >= OPW || k >= cnt) continue;
-    const typename RecOf<R>::type r = rec[beg + k];
-    int ix[NT], iy[NT], iz[NT];
+    const typename RecOf<T>::type r = rec[k];
     T wx[NT], wy[NT], wz[NT];
-    if constexpr (sizeof(R) == 4) {
+    int ix, iy, iz;
+    if constexpr (sizeof(T) == 4) {
       const uint32_t ux = __float_as_uint(r.x), uy = __float_as_uint(r.y), uz = __float_as_uint(r.z);
       const float sc24 = 5.9604644775390625e-8f;   // 2^-24
-      axis_taps<ASSIGN, T>((T)((float)(ux & 0xffffffu) * sc24), ux >> 24, ph, ix, wx);
-      axis_taps<ASSIGN, T>((T)((float)(uy & 0xffffffu) * sc24), uy >> 24, ph, iy, wy);
-      axis_taps<ASSIGN, T>((T)((float)(uz & 0xffffffu) * sc24), uz >> 24, ph, iz, wz);
+      ix = axis_taps<ASSIGN, T>((float)(ux & 0xffffffu) * sc24, ux >> 24, ph, wx);
+      iy = axis_taps<ASSIGN, T>((float)(uy & 0xffffffu) * sc24, uy >> 24, ph, wy);
+      iz = axis_taps<ASSIGN, T, false>((float)(uz & 0xffffffu) * sc24, uz >> 24, ph, wz);
     } else {
-      const uint32_t m = meta[beg + k];
-      axis_taps<ASSIGN, T>((T)r.x, m & 255u, ph, ix, wx);
-      axis_taps<ASSIGN, T>((T)r.y, (m >> 8) & 255u, ph, iy, wy);
-      axis_taps<ASSIGN, T>((T)r.z, (m >> 16) & 255u, ph, iz, wz);
+      const uint32_t m = meta[k];
+      ix = axis_taps<ASSIGN, T>(r.x, m & 255u, ph, wx);
+      iy = axis_taps<ASSIGN, T>(r.y, (m >> 8) & 255u, ph, wy);
+      iz = axis_taps<ASSIGN, T, false>(r.z, (m >> 16) & 255u, ph, wz);
     }
+    // the taps of a brick's object lie inside its tile by construction; the test only protects shared memory
+    if (max(max(ix, iy), iz) > TS - NT) continue;
     T wxs = wx[0];
-    int ixs = ix[0];
 #pragma unroll
     for (int a = 1; a < NT; ++a)
-      if (xt == a) { wxs = wx[a]; ixs = ix[a]; }
-    const T wgt = (T)r.w * scale * wxs;
+      if (xt == a) wxs = wx[a];
+    const T wgt = r.w * scale * wxs;
+    const int base = (iz * TS + iy) * TS + ix + xt;
+    // tap values (w 2^e W_x) W_z W_y, formed once per tap in a fixed order
+    if constexpr (sizeof(T) == 4) {
+      int h[2], l[2];
+      float wc[NT];
 #pragma unroll
-    for (int c = 0; c < NT; ++c) {
+      for (int c = 0; c < NT; ++c) {
+        wc[c] = wgt * wz[c];
+        fixed_parts2(mul2(pack2(wc[c], wc[c]), pack2(wy[0], wy[1])), h, l);
+        tile_add<WIDE>(lo, hi, top, base + c * TS * TS, h[0], l[0]);
+        tile_add<WIDE>(lo, hi, top, base + (c * TS + 1) * TS, h[1], l[1]);
+      }
+      if constexpr (NT == 3) {
+        fixed_parts2(mul2(pack2(wc[0], wc[1]), pack2(wy[2], wy[2])), h, l);
+        tile_add<WIDE>(lo, hi, top, base + 2 * TS, h[0], l[0]);
+        tile_add<WIDE>(lo, hi, top, base + (TS + 2) * TS, h[1], l[1]);
+        fixed_parts2(mul2(pack2(wc[2], 0.0f), pack2(wy[2], 0.0f)), h, l);
+        tile_add<WIDE>(lo, hi, top, base + (2 * TS + 2) * TS, h[0], l[0]);
+      }
+    } else {
 #pragma unroll
-      for (int bb = 0; bb < NT; ++bb) {
-        // tap value (w 2^e W_x) W_z W_y, formed once per tap in a fixed order
-        const long long q = to_fixed<T>(wgt * wz[c] * wy[bb]);
-        // taps stay inside the tile by construction; the guard only protects shared memory
-        if ((unsigned)iz[c] < (unsigned)g.ts && (unsigned)iy[bb] < (unsigned)g.ts && (unsigned)ixs < (unsigned)g.ts)
-          atomicAdd(reinterpret_cast<unsigned long long*>(acc + (iz[c] * g.ts + iy[bb]) * g.ts + ixs),
-                    static_cast<unsigned long long>(q));
+      for (int c = 0; c < NT; ++c) {
+#pragma unroll
+        for (int bb = 0; bb < NT; ++bb) tile_add(lo, hi, base + (c * TS + bb) * TS, wgt * wz[c] * wy[bb]);
       }
     }
   }
+}
+
+template <typename T, int BS> constexpr size_t tile_smem() {
+  return (sizeof(T) == 4 ? 9 : 8) * (size_t)(BS + 4) * (BS + 4) * (BS + 4);
+}
+
+// One CTA per (brick, phase): fixed-point accumulation of all taps in a (BS+4)^3 tile.  Bound by the
+// shared-memory atomics and the instructions that form a tap's integer parts (27 taps per object and
+// phase for TSC, 8 for CIC); 72 KB of tile words, three CTAs of 512 threads per SM.
+template <int ASSIGN, typename T, int BS>
+__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 3 : 2)
+k_paint_brick(const typename RecOf<T>::type* __restrict__ rec, const uint32_t* __restrict__ meta,
+              const int* __restrict__ start, const int* __restrict__ count, int nphase,
+              const double* __restrict__ sc, int maxw_slot, T* __restrict__ tiles) {
+  constexpr int TS = BS + 4, TS3 = TS * TS * TS;
+  static_assert(TS3 % 16 == 0, "the tile words are cleared and read in 16-byte steps");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int* lo = reinterpret_cast<int*>(smem_raw);
+  int* hi = lo + TS3;
+  unsigned* top = reinterpret_cast<unsigned*>(hi + TS3);   // one signed byte per cell (float tiles)
+  __shared__ int s_exp;
+  const int b = blockIdx.x / nphase, ph = blockIdx.x % nphase;
+  const int cnt = count[b], beg = start[b];
+  for (int i = threadIdx.x; i < (int)(tile_smem<T, BS>() / 16); i += blockDim.x)
+    reinterpret_cast<int4*>(smem_raw)[i] = make_int4(0, 0, 0, 0);
+  if (threadIdx.x == 0) {
+    // fixed-point scale 2^e with cnt * max|w| * 2^e < 2^61 (no overflow of the tile sums)
+    const double bound = (double)cnt * sc[maxw_slot];
+    int ex = 0;
+    if (bound > 0) frexp(bound, &ex);
+    int e = 61 - ex;
+    if constexpr (sizeof(T) == 4) {
+      // float: below 2^60 (the words' range) and every tap |w W| 2^e < 2^43 (that of fixed_parts)
+      int exw = 0;
+      if (sc[maxw_slot] > 0) frexp(sc[maxw_slot], &exw);
+      e = max(-126, min(126, min(e - 1, 43 - exw)));
+    }
+    s_exp = e;
+  }
   __syncthreads();
-  const T inv = (T)ldexp(1.0, -e);
-  T* out = tiles + ((size_t)b * nphase + ph) * ts3;
-  for (int i = threadIdx.x; i < ts3; i += blockDim.x) out[i] = from_fixed<T>(acc[i], inv);
+  const int e = s_exp;
+  T scale, inv;   // 2^e and 2^-e
+  if constexpr (sizeof(T) == 4) {
+    scale = __int_as_float((127 + e) << 23);
+    inv = __int_as_float((127 - e) << 23);
+  } else {
+    scale = ldexp(1.0, e);
+    inv = ldexp(1.0, -e);
+  }
+  const uint32_t* bmeta = sizeof(T) == 8 ? meta + beg : nullptr;
+  if (cnt <= NARROW_MAX)
+    tile_taps<ASSIGN, T, BS, false>(rec + beg, bmeta, cnt, ph, scale, lo, hi, top);
+  else
+    tile_taps<ASSIGN, T, BS, true>(rec + beg, bmeta, cnt, ph, scale, lo, hi, top);
+  __syncthreads();
+  T* out = tiles + ((size_t)b * nphase + ph) * TS3;
+  for (int i = threadIdx.x; i < TS3 / 4; i += blockDim.x) {
+    const int4 l = reinterpret_cast<const int4*>(lo)[i];
+    const int4 h = reinterpret_cast<const int4*>(hi)[i];
+    const unsigned t = sizeof(T) == 4 ? top[i] : 0u;
+    const T v0 = from_fixed(tile_sum<T>(l.x, h.x, t, 0), inv), v1 = from_fixed(tile_sum<T>(l.y, h.y, t, 1), inv);
+    const T v2 = from_fixed(tile_sum<T>(l.z, h.z, t, 2), inv), v3 = from_fixed(tile_sum<T>(l.w, h.w, t, 3), inv);
+    if constexpr (sizeof(T) == 4) {
+      reinterpret_cast<float4*>(out)[i] = make_float4(v0, v1, v2, v3);
+    } else {
+      reinterpret_cast<double2*>(out)[2 * i] = make_double2(v0, v1);
+      reinterpret_cast<double2*>(out)[2 * i + 1] = make_double2(v2, v3);
+    }
+  }
 }
 
 // Each cell sums the tiles covering it, in a fixed order (brick offset -1, 0, +1 per axis, z
@@ -613,7 +757,19 @@ npc_status launch_fold(npc_ctx* ctx, const void* tiles, const PaintGeo& g, int n
   return NPC_OK;
 }
 
-template <int ASSIGN, typename R, typename T>
+template <int ASSIGN, typename T, int BS>
+npc_status launch_tiles(npc_ctx* ctx, const void* rec, const uint32_t* meta, const int* start, const int* count,
+                        int nbricks, int nphase, const double* sc, int slot, void* tiles) {
+  const size_t smem = tile_smem<T, BS>();
+  auto kern = k_paint_brick<ASSIGN, T, BS>;
+  NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  kern<<<nbricks * nphase, 512, smem, ctx->stream>>>((const typename RecOf<T>::type*)rec, meta, start, count, nphase, sc,
+                                                     slot, (T*)tiles);
+  NPC_LAUNCH(ctx);
+  return NPC_OK;
+}
+
+template <int ASSIGN, typename T>
 npc_status paint_impl(npc_ctx* ctx, const DevCatalog& d, const DevCatalog* r, const npc_mesh_spec& m,
                       int weight_power, const double* sc, void* mesh_a, void* mesh_b) {
   PaintGeo g;
@@ -645,7 +801,7 @@ npc_status paint_impl(npc_ctx* ctx, const DevCatalog& d, const DevCatalog* r, co
   NPC_TRY(ws_get(ctx, "paint.brick", sizeof(int) * std::max<int64_t>(ntot, 1), (void**)&brick));
   NPC_TRY(ws_get(ctx, "paint.rank", sizeof(int) * std::max<int64_t>(ntot, 1), (void**)&rank));
   NPC_TRY(ws_get(ctx, "paint.meta", sizeof(uint32_t) * std::max<int64_t>(ntot, 1), (void**)&meta));
-  NPC_TRY(ws_get(ctx, "paint.rec", sizeof(typename RecOf<R>::type) * std::max<int64_t>(ntot, 1), &rec));
+  NPC_TRY(ws_get(ctx, "paint.rec", sizeof(typename RecOf<T>::type) * std::max<int64_t>(ntot, 1), &rec));
   NPC_TRY(ws_get(ctx, "paint.tiles", sizeof(T) * ts3 * nbricks * nphase, &tiles));
   NPC_CUDA(ctx, cudaMemsetAsync(count, 0, sizeof(int) * nbricks, ctx->stream));
   // counting: data then randoms share the brick counters (ranks continue)
@@ -658,19 +814,18 @@ npc_status paint_impl(npc_ctx* ctx, const DevCatalog& d, const DevCatalog* r, co
   k_scan<<<1, 1024, 0, ctx->stream>>>(count, nbricks, start);
   NPC_LAUNCH(ctx);
   NPC_TRY(stage_mark(ctx, "paint_count"));
-  NPC_TRY((scatter_cat<ASSIGN, R>(ctx, d, weight_power, 0, sc, g, brick, rank, start, rec, meta)));
+  NPC_TRY((scatter_cat<ASSIGN, T>(ctx, d, weight_power, 0, sc, g, brick, rank, start, rec, meta)));
   if (r) {
     const int kind = weight_power == 1 ? 1 : 2;
-    NPC_TRY((scatter_cat<ASSIGN, R>(ctx, *r, weight_power, kind, sc, g, brick + d.n, rank + d.n, start, rec, meta)));
+    NPC_TRY((scatter_cat<ASSIGN, T>(ctx, *r, weight_power, kind, sc, g, brick + d.n, rank + d.n, start, rec, meta)));
   }
   NPC_TRY(stage_mark(ctx, "paint_scatter"));
-  const size_t smem = sizeof(long long) * ts3;
   const int slot = weight_power == 1 ? SC_MAXW_F : SC_MAXW_N;
-  auto kern = k_paint_brick<ASSIGN, R, T>;
-  NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<nbricks * nphase, 512, smem, ctx->stream>>>((const typename RecOf<R>::type*)rec, meta, start, count, g,
-                                                     nphase, sc, slot, (T*)tiles);
-  NPC_LAUNCH(ctx);
+  switch (g.bs) {
+    case 4: NPC_TRY((launch_tiles<ASSIGN, T, 4>(ctx, rec, meta, start, count, nbricks, nphase, sc, slot, tiles))); break;
+    case 8: NPC_TRY((launch_tiles<ASSIGN, T, 8>(ctx, rec, meta, start, count, nbricks, nphase, sc, slot, tiles))); break;
+    default: NPC_TRY((launch_tiles<ASSIGN, T, 16>(ctx, rec, meta, start, count, nbricks, nphase, sc, slot, tiles)));
+  }
   NPC_TRY(stage_mark(ctx, "paint_tiles"));
   const int sub = (m.periodic && weight_power == 1) ? 1 : 0;
   return launch_fold<T>(ctx, tiles, g, nphase, sc, sub, mesh_a, mesh_b);
@@ -745,13 +900,13 @@ npc_status launch_paint(npc_ctx* ctx, const DevCatalog& d, const DevCatalog* r, 
                         int weight_power, int prec, const double* dev_scalars, void* mesh_a, void* mesh_b) {
   const bool any_double = d.dtype == 1 || (r && r->dtype == 1);
   if (prec == NPC_PREC_FP64) {
-    if (m.assign == 2) return paint_impl<2, double, double>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b);
-    return paint_impl<3, double, double>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b);
+    if (m.assign == 2) return paint_impl<2, double>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b);
+    return paint_impl<3, double>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b);
   }
   // records keep the fraction s - floor(s) (< 1) in float32 in the mixed path
   (void)any_double;
-  if (m.assign == 2) return paint_impl<2, float, float>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b);
-  return paint_impl<3, float, float>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b);
+  if (m.assign == 2) return paint_impl<2, float>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b);
+  return paint_impl<3, float>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b);
 }
 
 // ---------------------------------------------------------------------------------------------
