@@ -150,77 +150,159 @@ __global__ void k_cat_final(const double* __restrict__ pd, const double* __restr
 // ---------------------------------------------------------------------------------------------
 struct PaintGeo {
   int n, bs, nb, ts;     // mesh cells, brick size, bricks per side, tile side (bs + 4)
+  int bshift;            // log2(bs)
   double o[3];           // origin
   double inv_h;          // n / box
   float o_hi[3], o_lo[3];      // origin and n / box as float pairs (hi + lo) for the scatter's
   float ih_hi, ih_lo;          // float fast path
 };
 
-__device__ __forceinline__ long long wrapi(long long i, int n) {
-  long long r = i % n;
-  return r < 0 ? r + n : r;
+// i modulo n; the integer division only outside the box
+__device__ __forceinline__ int wrapi(long long i, int n) {
+  if (i >= 0 && i < n) return (int)i;
+  const long long r = i % n;
+  return (int)(r < 0 ? r + n : r);
 }
 
+// One or two catalogues of the same type sorted together: object i is the first's for i < n0, else the
+// second's (randoms).
+template <typename P> struct CatPair {
+  const P* pos[2];
+  const P* w[2];
+  int64_t n0, n;
+};
+
+// Brick of an object, -1 when its position is not finite (or absurdly far).
 template <typename P>
-__global__ void k_brick_count(const P* __restrict__ pos, int64_t n, PaintGeo g, int* __restrict__ count,
-                              int* __restrict__ brick, int* __restrict__ rank) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    int bidx[3];
-    bool ok = true;
+__device__ __forceinline__ int brick_of(const P* __restrict__ pos, int64_t i, const PaintGeo& g) {
+  int bidx[3];
+  bool ok = true;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      // floor(s) decided in float when s is farther from an integer than a bound on the float
-      // rounding error (three roundings of relative size 2^-24 on |x| n/box, |origin| n/box and
-      // |s|, with a factor 8 of margin), otherwise in float64 exactly as everywhere else
-      const P pa = pos[3 * i + a];
-      long long f;
-      if (sizeof(P) == 4) {
-        const float ih = (float)g.inv_h;
-        const float sf = ((float)pa - (float)g.o[a]) * ih;
-        const float ff = floorf(sf);
-        const float fr = sf - ff;
-        const float tol = 1.0e-6f * ((fabsf((float)pa) + fabsf((float)g.o[a])) * ih + fabsf(sf)) + 1.0e-6f;
-        if (fabsf(sf) < 1.0e6f && fr > tol && fr < 1.0f - tol) {
-          f = (long long)ff;
-        } else {
-          const double s = ((double)pa - g.o[a]) * g.inv_h;
-          if (!(fabs(s) < 1e15)) { ok = false; bidx[a] = 0; continue; }
-          f = (long long)floor(s);
-        }
-      } else {
-        const double s = ((double)pa - g.o[a]) * g.inv_h;
-        if (!(fabs(s) < 1e15)) { ok = false; bidx[a] = 0; continue; }
-        f = (long long)floor(s);
+  for (int a = 0; a < 3; ++a) {
+    // floor(s) decided in float when s is farther from an integer than a bound on the float
+    // rounding error (three roundings of relative size 2^-24 on |x| n/box, |origin| n/box and
+    // |s|, with a factor 8 of margin), otherwise in float64 exactly as everywhere else
+    const P pa = pos[3 * i + a];
+    if (sizeof(P) == 4) {
+      const float ih = (float)g.inv_h;
+      const float sf = ((float)pa - (float)g.o[a]) * ih;
+      const float ff = floorf(sf);
+      const float fr = sf - ff;
+      const float tol = 1.0e-6f * ((fabsf((float)pa) + fabsf((float)g.o[a])) * ih + fabsf(sf)) + 1.0e-6f;
+      if (fabsf(sf) < 1.0e6f && fr > tol && fr < 1.0f - tol) {
+        bidx[a] = wrapi((int)ff, g.n) >> g.bshift;
+        continue;
       }
-      bidx[a] = (int)(wrapi(f, g.n) / g.bs);
     }
-    if (!ok) { brick[i] = -1; rank[i] = 0; continue; }
-    const int b = (bidx[2] * g.nb + bidx[1]) * g.nb + bidx[0];
-    brick[i] = b;
-    rank[i] = atomicAdd(&count[b], 1);
+    const double s = ((double)pa - g.o[a]) * g.inv_h;
+    if (!(fabs(s) < 1e15)) {
+      ok = false;
+      bidx[a] = 0;
+      continue;
+    }
+    bidx[a] = wrapi((long long)floor(s), g.n) >> g.bshift;
+  }
+  return ok ? (bidx[2] * g.nb + bidx[1]) * g.nb + bidx[0] : -1;
+}
+
+// Brick and in-brick rank of every object, and the objects per brick.  Up to COUNT_SHARED_MAX bricks the
+// CTA counts its COUNT_CHUNK objects in shared memory and takes one range per brick from the global
+// counter: a global counter then sees one add per CTA instead of one per object (the adds that return
+// a rank serialise per 32-byte sector at about 10 ns each: 189 us for 1.4 M objects in 512 bricks, 10 ms
+// of a batch's 34 ms; for the same reason every counter has a sector of its own).  Above it the counters
+// are too many for that to help (less than one object per CTA and brick) and each object adds to its own.
+constexpr int COUNT_THREADS = 512, COUNT_ITEMS = 8;
+constexpr int COUNT_SHARED_MAX = 8192;
+constexpr int COUNT_STRIDE = 8;   // ints between the counters of consecutive bricks
+template <typename P, bool SHARED>
+__global__ void __launch_bounds__(COUNT_THREADS)
+k_brick_count(const CatPair<P> c, PaintGeo g, int nbricks, int* __restrict__ count, int* __restrict__ brick,
+              int* __restrict__ rank) {
+  extern __shared__ int s_hist[];
+  const int64_t beg = blockIdx.x * (int64_t)(COUNT_THREADS * COUNT_ITEMS);
+  if constexpr (SHARED) {
+    for (int b = threadIdx.x; b < nbricks; b += COUNT_THREADS) s_hist[b] = 0;
+    __syncthreads();
+  }
+  int br[COUNT_ITEMS], rk[COUNT_ITEMS];
+#pragma unroll
+  for (int k = 0; k < COUNT_ITEMS; ++k) {
+    const int64_t i = beg + k * COUNT_THREADS + threadIdx.x;
+    br[k] = -1;
+    rk[k] = 0;
+    if (i >= c.n) continue;
+    br[k] = i < c.n0 ? brick_of<P>(c.pos[0], i, g) : brick_of<P>(c.pos[1], i - c.n0, g);
+    if (br[k] >= 0) rk[k] = atomicAdd(SHARED ? s_hist + br[k] : count + (size_t)br[k] * COUNT_STRIDE, 1);
+  }
+  if constexpr (SHARED) {
+    __syncthreads();
+    for (int b = threadIdx.x; b < nbricks; b += COUNT_THREADS) {
+      const int m = s_hist[b];
+      if (m > 0) s_hist[b] = atomicAdd(count + (size_t)b * COUNT_STRIDE, m);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int k = 0; k < COUNT_ITEMS; ++k) {
+    const int64_t i = beg + k * COUNT_THREADS + threadIdx.x;
+    if (i >= c.n) continue;
+    brick[i] = br[k];
+    rank[i] = br[k] < 0 ? 0 : (SHARED ? s_hist[br[k]] + rk[k] : rk[k]);
   }
 }
 
-// exclusive scan of count[0..m) into start[0..m), single block
-__global__ void __launch_bounds__(1024) k_scan(const int* __restrict__ count, int m, int* __restrict__ start) {
-  __shared__ int sh[1024];
-  const int per = (m + blockDim.x - 1) / blockDim.x;
-  const int beg = threadIdx.x * per;
-  int s = 0;
-  for (int i = beg; i < min(m, beg + per); ++i) s += count[i];
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int off = 1; off < blockDim.x; off <<= 1) {
-    int v = threadIdx.x >= off ? sh[threadIdx.x - off] : 0;
-    __syncthreads();
-    sh[threadIdx.x] += v;
-    __syncthreads();
+// Exclusive scan of the m brick counts into start[0..m), the total into start[m]: one CTA per SCAN_CHUNK entries writes its chunk's scan
+// and total; with more than one chunk k_scan_add adds the totals of the chunks before (one CTA over
+// everything took 428 us for the 262,144 bricks of a 1024^3 mesh).
+constexpr int SCAN_THREADS = 1024, SCAN_PER = 8, SCAN_CHUNK = SCAN_THREADS * SCAN_PER;
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan(const int* __restrict__ count, int m, int* __restrict__ start,
+                                                       int* __restrict__ total) {
+  __shared__ int s_warp[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int beg = blockIdx.x * SCAN_CHUNK + threadIdx.x * SCAN_PER;
+  int v[SCAN_PER], sum = 0;
+#pragma unroll
+  for (int k = 0; k < SCAN_PER; ++k) {
+    v[k] = beg + k < m ? count[(size_t)(beg + k) * COUNT_STRIDE] : 0;
+    sum += v[k];
   }
-  int run = sh[threadIdx.x] - s;
-  for (int i = beg; i < min(m, beg + per); ++i) {
-    start[i] = run;
-    run += count[i];
+  int inc = sum;   // inclusive over the warp's threads
+  for (int off = 1; off < 32; off <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, inc, off);
+    if (lane >= off) inc += o;
+  }
+  if (lane == 31) s_warp[warp] = inc;
+  __syncthreads();
+  if (warp == 0) {
+    int w = s_warp[lane];
+    for (int off = 1; off < 32; off <<= 1) {
+      const int o = __shfl_up_sync(0xffffffffu, w, off);
+      if (lane >= off) w += o;
+    }
+    s_warp[lane] = w;
+  }
+  __syncthreads();
+  int run = inc - sum + (warp > 0 ? s_warp[warp - 1] : 0);
+#pragma unroll
+  for (int k = 0; k < SCAN_PER; ++k) {
+    if (beg + k <= m) start[beg + k] = run;
+    run += v[k];
+  }
+  if (threadIdx.x == SCAN_THREADS - 1) total[blockIdx.x] = run;
+}
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_add(const int* __restrict__ total, int m,
+                                                           int* __restrict__ start) {
+  __shared__ int s_before;
+  if (threadIdx.x < 32) {
+    int v = 0;
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += 32) v += total[b];
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if (threadIdx.x == 0) s_before = v;
+  }
+  __syncthreads();
+  for (int k = 0; k < SCAN_PER; ++k) {
+    const int i = blockIdx.x * SCAN_CHUNK + k * SCAN_THREADS + threadIdx.x;
+    if (i <= m) start[i] += s_before;
   }
 }
 
@@ -248,7 +330,7 @@ __device__ __forceinline__ uint32_t axis_meta(double s, int n, int bs, double* f
     ib = (long long)floor(sb + 0.5);
   }
   *frac = s - f;
-  const uint32_t local = (uint32_t)(wrapi(fb, n) % bs);
+  const uint32_t local = (uint32_t)(wrapi(fb, n) & (bs - 1));
   return local | ((uint32_t)(ia - fb) << 5) | ((uint32_t)(ib - fb) << 6);
 }
 
@@ -284,28 +366,30 @@ __device__ __forceinline__ bool axis_meta_fast(float x, float o_hi, float o_lo, 
   if (fr < tol || fr > 1.0f - tol || fabsf(fr - 0.5f) < tol) return false;
   const int fb = (int)f;
   const uint32_t half = fr >= 0.5f ? 1u : 0u;
-  const uint32_t local = (uint32_t)((((fb % n) + n) % n) % bs);
+  const uint32_t local = (uint32_t)(wrapi(fb, n) & (bs - 1));
   const uint32_t da = ASSIGN == 2 ? 0u : half, db = ASSIGN == 2 ? half : 1u;
   *meta = local | (da << 5) | (db << 6);
   *frac = fr;
   return true;
 }
 
-// coefficient * w^power per particle; coef_kind: 0 -> 1, 1 -> -alpha, 2 -> +alpha^2
+// coefficient * w^power per object: 1 for the first catalogue, -alpha (power 1) or alpha^2 for the randoms
 template <int ASSIGN, typename P, typename R>
-__global__ void k_scatter(const P* __restrict__ pos, const P* __restrict__ w, int64_t n, int power,
-                          int coef_kind, const double* __restrict__ sc, PaintGeo g, const int* __restrict__ brick,
-                          const int* __restrict__ rank, const int* __restrict__ start,
+__global__ void k_scatter(const CatPair<P> c, int power, bool randoms_first, const double* __restrict__ sc, PaintGeo g,
+                          const int* __restrict__ brick, const int* __restrict__ rank, const int* __restrict__ start,
                           typename RecOf<R>::type* __restrict__ rec, uint32_t* __restrict__ meta) {
-  double coef = 1.0;
-  if (coef_kind == 1) coef = -sc[SC_ALPHA];
-  if (coef_kind == 2) coef = sc[SC_ALPHA] * sc[SC_ALPHA];
-  const float coef_f = (float)coef;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int b = brick[i];
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < c.n;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int b = brick[t];
     if (b < 0) continue;
-    const int dst = start[b] + rank[i];
+    const int dst = start[b] + rank[t];
+    const bool second = t >= c.n0;
+    const P* __restrict__ pos = second ? c.pos[1] : c.pos[0];
+    const P* __restrict__ w = second ? c.w[1] : c.w[0];
+    const int64_t i = second ? t - c.n0 : t;
+    double coef = 1.0;
+    if (second || randoms_first) coef = power == 2 ? sc[SC_ALPHA] * sc[SC_ALPHA] : -sc[SC_ALPHA];
+    const float coef_f = (float)coef;
     if constexpr (sizeof(R) == 4 && sizeof(P) == 4) {
       // float records from float positions: the float pair path, float64 only near a decision
       uint32_t u[3];
@@ -576,8 +660,8 @@ template <typename T, int BS> constexpr size_t tile_smem() {
 template <int ASSIGN, typename T, int BS>
 __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 3 : 2)
 k_paint_brick(const typename RecOf<T>::type* __restrict__ rec, const uint32_t* __restrict__ meta,
-              const int* __restrict__ start, const int* __restrict__ count, int nphase,
-              const double* __restrict__ sc, int maxw_slot, T* __restrict__ tiles) {
+              const int* __restrict__ start, int nphase, const double* __restrict__ sc, int maxw_slot,
+              T* __restrict__ tiles) {
   constexpr int TS = BS + 4, TS3 = TS * TS * TS;
   static_assert(TS3 % 16 == 0, "the tile words are cleared and read in 16-byte steps");
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -586,7 +670,7 @@ k_paint_brick(const typename RecOf<T>::type* __restrict__ rec, const uint32_t* _
   unsigned* top = reinterpret_cast<unsigned*>(hi + TS3);   // one signed byte per cell (float tiles)
   __shared__ int s_exp;
   const int b = blockIdx.x / nphase, ph = blockIdx.x % nphase;
-  const int cnt = count[b], beg = start[b];
+  const int beg = start[b], cnt = start[b + 1] - beg;
   for (int i = threadIdx.x; i < (int)(tile_smem<T, BS>() / 16); i += blockDim.x)
     reinterpret_cast<int4*>(smem_raw)[i] = make_int4(0, 0, 0, 0);
   if (threadIdx.x == 0) {
@@ -714,34 +798,46 @@ k_fold(const T* __restrict__ tiles, PaintGeo g, int nphase, const double* __rest
   }
 }
 
+// A catalogue and its randoms (r may be null) as one object list; of one type only.
 template <typename P>
-npc_status paint_count(npc_ctx* ctx, const DevCatalog& c, const PaintGeo& g, int* count, int* brick,
+CatPair<P> cat_pair(const DevCatalog* d, const DevCatalog* r) {
+  CatPair<P> c{};
+  c.pos[0] = (const P*)d->pos;
+  c.w[0] = (const P*)d->w;
+  c.n0 = c.n = d->n;
+  if (r) {
+    c.pos[1] = (const P*)r->pos;
+    c.w[1] = (const P*)r->w;
+    c.n += r->n;
+  }
+  return c;
+}
+
+template <typename P>
+npc_status paint_count(npc_ctx* ctx, const CatPair<P>& c, const PaintGeo& g, int nbricks, int* count, int* brick,
                        int* rank) {
   if (c.n == 0) return NPC_OK;
-  const int blocks = (int)std::min<int64_t>((c.n + 255) / 256, (int64_t)1 << 20);   // one object per thread
-  k_brick_count<P><<<blocks, 256, 0, ctx->stream>>>((const P*)c.pos, c.n, g, count, brick, rank);
+  const int chunk = COUNT_THREADS * COUNT_ITEMS;
+  const unsigned blocks = (unsigned)((c.n + chunk - 1) / chunk);
+  if (nbricks <= COUNT_SHARED_MAX)
+    k_brick_count<P, true><<<blocks, COUNT_THREADS, sizeof(int) * nbricks, ctx->stream>>>(c, g, nbricks, count, brick,
+                                                                                          rank);
+  else
+    k_brick_count<P, false><<<blocks, COUNT_THREADS, 0, ctx->stream>>>(c, g, nbricks, count, brick, rank);
   NPC_LAUNCH(ctx);
   return NPC_OK;
 }
 
 template <int ASSIGN, typename P, typename R>
-npc_status paint_scatter(npc_ctx* ctx, const DevCatalog& c, int power, int coef_kind, const double* sc,
+npc_status paint_scatter(npc_ctx* ctx, const CatPair<P>& c, int power, bool randoms_first, const double* sc,
                          const PaintGeo& g, const int* brick, const int* rank, const int* start, void* rec,
                          uint32_t* meta) {
   if (c.n == 0) return NPC_OK;
   const int blocks = (int)std::min<int64_t>((c.n + 255) / 256, (int64_t)1 << 20);   // one object per thread
-  k_scatter<ASSIGN, P, R><<<blocks, 256, 0, ctx->stream>>>((const P*)c.pos, (const P*)c.w, c.n, power, coef_kind,
-                                                           sc, g, brick, rank, start,
+  k_scatter<ASSIGN, P, R><<<blocks, 256, 0, ctx->stream>>>(c, power, randoms_first, sc, g, brick, rank, start,
                                                            (typename RecOf<R>::type*)rec, meta);
   NPC_LAUNCH(ctx);
   return NPC_OK;
-}
-
-template <int ASSIGN, typename R>
-npc_status scatter_cat(npc_ctx* ctx, const DevCatalog& c, int power, int kind, const double* sc, const PaintGeo& g,
-                       const int* brick, const int* rank, const int* start, void* rec, uint32_t* meta) {
-  if (c.dtype == 1) return paint_scatter<ASSIGN, double, R>(ctx, c, power, kind, sc, g, brick, rank, start, rec, meta);
-  return paint_scatter<ASSIGN, float, R>(ctx, c, power, kind, sc, g, brick, rank, start, rec, meta);
 }
 
 template <typename T>
@@ -758,12 +854,12 @@ npc_status launch_fold(npc_ctx* ctx, const void* tiles, const PaintGeo& g, int n
 }
 
 template <int ASSIGN, typename T, int BS>
-npc_status launch_tiles(npc_ctx* ctx, const void* rec, const uint32_t* meta, const int* start, const int* count,
-                        int nbricks, int nphase, const double* sc, int slot, void* tiles) {
+npc_status launch_tiles(npc_ctx* ctx, const void* rec, const uint32_t* meta, const int* start, int nbricks,
+                        int nphase, const double* sc, int slot, void* tiles) {
   const size_t smem = tile_smem<T, BS>();
   auto kern = k_paint_brick<ASSIGN, T, BS>;
   NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<nbricks * nphase, 512, smem, ctx->stream>>>((const typename RecOf<T>::type*)rec, meta, start, count, nphase, sc,
+  kern<<<nbricks * nphase, 512, smem, ctx->stream>>>((const typename RecOf<T>::type*)rec, meta, start, nphase, sc,
                                                      slot, (T*)tiles);
   NPC_LAUNCH(ctx);
   return NPC_OK;
@@ -775,6 +871,7 @@ npc_status paint_impl(npc_ctx* ctx, const DevCatalog& d, const DevCatalog* r, co
   PaintGeo g;
   g.n = m.n;
   g.bs = (m.n >= 48 && m.n % 16 == 0) ? 16 : m.n / 4;   // 16 for every size >= 48; 4, 8 at n = 16, 32
+  g.bshift = g.bs == 16 ? 4 : (g.bs == 8 ? 3 : 2);
   g.nb = m.n / g.bs;
   g.ts = g.bs + 4;
   for (int a = 0; a < 3; ++a) g.o[a] = m.origin[a];
@@ -796,35 +893,48 @@ npc_status paint_impl(npc_ctx* ctx, const DevCatalog& d, const DevCatalog* r, co
   void* rec;
   void* tiles;
   const size_t ts3 = (size_t)g.ts * g.ts * g.ts;
-  NPC_TRY(ws_get(ctx, "paint.count", sizeof(int) * nbricks, (void**)&count));
-  NPC_TRY(ws_get(ctx, "paint.start", sizeof(int) * nbricks, (void**)&start));
+  NPC_TRY(ws_get(ctx, "paint.count", sizeof(int) * nbricks * COUNT_STRIDE, (void**)&count));
+  NPC_TRY(ws_get(ctx, "paint.start", sizeof(int) * (nbricks + 1), (void**)&start));
   NPC_TRY(ws_get(ctx, "paint.brick", sizeof(int) * std::max<int64_t>(ntot, 1), (void**)&brick));
   NPC_TRY(ws_get(ctx, "paint.rank", sizeof(int) * std::max<int64_t>(ntot, 1), (void**)&rank));
   NPC_TRY(ws_get(ctx, "paint.meta", sizeof(uint32_t) * std::max<int64_t>(ntot, 1), (void**)&meta));
   NPC_TRY(ws_get(ctx, "paint.rec", sizeof(typename RecOf<T>::type) * std::max<int64_t>(ntot, 1), &rec));
   NPC_TRY(ws_get(ctx, "paint.tiles", sizeof(T) * ts3 * nbricks * nphase, &tiles));
-  NPC_CUDA(ctx, cudaMemsetAsync(count, 0, sizeof(int) * nbricks, ctx->stream));
-  // counting: data then randoms share the brick counters (ranks continue)
-  if (d.dtype == 1) NPC_TRY(paint_count<double>(ctx, d, g, count, brick, rank));
-  else NPC_TRY(paint_count<float>(ctx, d, g, count, brick, rank));
-  if (r) {
-    if (r->dtype == 1) NPC_TRY(paint_count<double>(ctx, *r, g, count, brick + d.n, rank + d.n));
-    else NPC_TRY(paint_count<float>(ctx, *r, g, count, brick + d.n, rank + d.n));
-  }
-  k_scan<<<1, 1024, 0, ctx->stream>>>(count, nbricks, start);
+  NPC_CUDA(ctx, cudaMemsetAsync(count, 0, sizeof(int) * nbricks * COUNT_STRIDE, ctx->stream));
+  // data and randoms share the brick counters (ranks continue): one launch each for counting and for
+  // scattering when both catalogues have one type
+  const bool joint = r && r->dtype == d.dtype;
+  auto each = [&](auto&& run) -> npc_status {   // run(catalogue pair's parts, offset, randoms first)
+    NPC_TRY(run(&d, joint ? r : nullptr, (int64_t)0, false));
+    if (r && !joint) NPC_TRY(run(r, (const DevCatalog*)nullptr, d.n, true));
+    return NPC_OK;
+  };
+  NPC_TRY(each([&](const DevCatalog* a, const DevCatalog* b, int64_t off, bool) {
+    return a->dtype == 1 ? paint_count<double>(ctx, cat_pair<double>(a, b), g, nbricks, count, brick + off, rank + off)
+                         : paint_count<float>(ctx, cat_pair<float>(a, b), g, nbricks, count, brick + off, rank + off);
+  }));
+  const int chunks = nbricks / SCAN_CHUNK + 1;   // of the nbricks + 1 entries
+  int* total;
+  NPC_TRY(ws_get(ctx, "paint.total", sizeof(int) * chunks, (void**)&total));
+  k_scan<<<chunks, SCAN_THREADS, 0, ctx->stream>>>(count, nbricks, start, total);
   NPC_LAUNCH(ctx);
-  NPC_TRY(stage_mark(ctx, "paint_count"));
-  NPC_TRY((scatter_cat<ASSIGN, T>(ctx, d, weight_power, 0, sc, g, brick, rank, start, rec, meta)));
-  if (r) {
-    const int kind = weight_power == 1 ? 1 : 2;
-    NPC_TRY((scatter_cat<ASSIGN, T>(ctx, *r, weight_power, kind, sc, g, brick + d.n, rank + d.n, start, rec, meta)));
+  if (chunks > 1) {
+    k_scan_add<<<chunks, SCAN_THREADS, 0, ctx->stream>>>(total, nbricks, start);
+    NPC_LAUNCH(ctx);
   }
+  NPC_TRY(stage_mark(ctx, "paint_count"));
+  NPC_TRY(each([&](const DevCatalog* a, const DevCatalog* b, int64_t off, bool rf) {
+    return a->dtype == 1 ? paint_scatter<ASSIGN, double, T>(ctx, cat_pair<double>(a, b), weight_power, rf, sc, g,
+                                                            brick + off, rank + off, start, rec, meta)
+                         : paint_scatter<ASSIGN, float, T>(ctx, cat_pair<float>(a, b), weight_power, rf, sc, g,
+                                                           brick + off, rank + off, start, rec, meta);
+  }));
   NPC_TRY(stage_mark(ctx, "paint_scatter"));
   const int slot = weight_power == 1 ? SC_MAXW_F : SC_MAXW_N;
   switch (g.bs) {
-    case 4: NPC_TRY((launch_tiles<ASSIGN, T, 4>(ctx, rec, meta, start, count, nbricks, nphase, sc, slot, tiles))); break;
-    case 8: NPC_TRY((launch_tiles<ASSIGN, T, 8>(ctx, rec, meta, start, count, nbricks, nphase, sc, slot, tiles))); break;
-    default: NPC_TRY((launch_tiles<ASSIGN, T, 16>(ctx, rec, meta, start, count, nbricks, nphase, sc, slot, tiles)));
+    case 4: NPC_TRY((launch_tiles<ASSIGN, T, 4>(ctx, rec, meta, start, nbricks, nphase, sc, slot, tiles))); break;
+    case 8: NPC_TRY((launch_tiles<ASSIGN, T, 8>(ctx, rec, meta, start, nbricks, nphase, sc, slot, tiles))); break;
+    default: NPC_TRY((launch_tiles<ASSIGN, T, 16>(ctx, rec, meta, start, nbricks, nphase, sc, slot, tiles)));
   }
   NPC_TRY(stage_mark(ctx, "paint_tiles"));
   const int sub = (m.periodic && weight_power == 1) ? 1 : 0;

@@ -41,3 +41,57 @@ def test_tile_words_carry(nobj, assign, sign):
     if sign != "positive":
         w *= np.where((rng.random(nobj) < 0.5) | (sign == "negative"), -1, 1).astype(np.float32)
     _check(pos, w, 32, 32.0, assign, float(np.abs(w).sum()))
+
+
+@pytest.mark.parametrize("n", [16, 32, 96, 256])
+@pytest.mark.parametrize("nobj", [1, 4095, 4096, 4097, 30_011])
+def test_brick_sort_and_wrap(n, nobj):
+    """Object numbers around the counting chunk, positions in cell order and up to two boxes outside:
+    every object must reach its cells (4, 4, 6 and 16 bricks a side)."""
+    rng = np.random.default_rng(n + nobj)
+    pos = ((rng.random((nobj, 3)) * 5 - 2) * n).astype(np.float32)
+    pos[: nobj // 2] = pos[np.lexsort(np.floor(pos[: nobj // 2]).T)]
+    w = (rng.random(nobj) + 0.5).astype(np.float32)
+    # reach of a cell: all objects within 3 cells of it, bounded by the densest 5^3 block
+    cells = np.floor(pos.astype(np.float64)).astype(np.int64) % n
+    dense = np.bincount((cells // 4) @ np.array([1, n, n * n]), weights=w).max()
+    _check(pos, w, n, float(n), 3, 8.0 * dense)
+
+
+def test_more_bricks_than_shared_counters():
+    """512^3 has 32,768 bricks: per-object counters and a scan over several chunks.  Each of 5,003
+    objects sits alone on a grid point, so its cell holds its weight and its neighbours known taps."""
+    n, nobj = 512, 5_003
+    rng = np.random.default_rng(5)
+    cells = np.unique(rng.integers(0, 128, (nobj, 3)) * 4, axis=0)
+    w = (rng.random(len(cells)) + 0.5).astype(np.float32)
+    got = _paint(cells.astype(np.float32), w, n, float(n), 2)
+    mean = float(w.astype(np.float64).sum()) / n**3
+    at = got[cells[:, 0], cells[:, 1], cells[:, 2]]
+    assert np.all(np.abs(at - (w - mean)) <= 6 * EPS * w)
+    got[cells[:, 0], cells[:, 1], cells[:, 2]] = -mean
+    assert np.all(np.abs(got + mean) <= 6 * EPS)
+
+
+@pytest.mark.parametrize("swap", [False, True])
+def test_catalogues_of_two_types(swap):
+    """Data and randoms of different float types are sorted by two launches, of one type by one: the
+    same positions give the same multipoles (to the rounding of the fractions and weights, 2^-20 of the
+    monopole's scale)."""
+    from types import SimpleNamespace
+
+    from paper_2605_04864_gb300 import api
+
+    rng = np.random.default_rng(3)
+    def cat(m):
+        return SimpleNamespace(pos=(rng.random((m, 3)) * 64 + 100).astype(np.float32), w=np.ones(m, np.float32),
+                               nbar=np.full(m, 1e-2, np.float32))
+    def wide(c):
+        return SimpleNamespace(pos=c.pos.astype(np.float64), w=c.w.astype(np.float64), nbar=c.nbar.astype(np.float64))
+    g, r = cat(2_000), cat(20_001)
+    kw = dict(n=32, box=64.0, origin=(100.0,) * 3, kbins=(0.05, 0.1, 12))
+    one = api.power_multipoles(g, r, **kw)
+    two = api.power_multipoles(wide(g) if swap else g, r if swap else wide(r), **kw)
+    scale = np.abs(one["P"][0]) + one["scalars"]["N0"]
+    for ell in (0, 2, 4):
+        assert np.all(np.abs(one["P"][ell] - two["P"][ell]) <= 2.0**-20 * scale)
