@@ -14,21 +14,22 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "npc_internal.cuh"
 
 namespace {
 
 constexpr int RED_THREADS = 256;
-constexpr int RED_BLOCKS = 1024;
+constexpr int RED_CHUNK = 4096;   // objects per block, until the blocks number four per SM
 constexpr int NSUM = 6;  // sum w, w^2, w^3, nbar w^2, nbar^2 w^3, max |w|
 
 template <typename T>
-__global__ void __launch_bounds__(RED_THREADS)
-k_cat_partials(const T* __restrict__ w, const T* __restrict__ nbar, int64_t n, double* part) {
+__device__ __forceinline__ void cat_partial(const T* __restrict__ w, const T* __restrict__ nbar, int64_t n,
+                                            int nblk, int blk, double* __restrict__ part) {
   __shared__ double sh[NSUM][RED_THREADS];
-  const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
-  const int64_t beg = (int64_t)blockIdx.x * chunk;
+  const int64_t chunk = (n + nblk - 1) / nblk;
+  const int64_t beg = (int64_t)blk * chunk;
   const int64_t end = min(n, beg + chunk);
   double a[NSUM] = {0, 0, 0, 0, 0, 0};
   if constexpr (sizeof(T) == 4) {
@@ -45,9 +46,7 @@ k_cat_partials(const T* __restrict__ w, const T* __restrict__ nbar, int64_t n, d
       hs[k] = __fadd_rn(s, e);
       ls[k] = __fsub_rn(e, __fsub_rn(hs[k], s));
     };
-    for (int64_t i = beg + threadIdx.x; i < end; i += blockDim.x) {
-      const float wi = w ? (float)w[i] : 1.0f;
-      const float nb = nbar ? (float)nbar[i] : 0.0f;
+    auto add = [&](float wi, float nb) {
       const float p2 = __fmul_rn(wi, wi), e2 = fmaf(wi, wi, -p2);             // w^2
       const float p3 = __fmul_rn(p2, wi), e3 = fmaf(p2, wi, -p3) + e2 * wi;   // w^3
       const float p4 = __fmul_rn(nb, p2), e4 = fmaf(nb, p2, -p4) + nb * e2;   // nbar w^2
@@ -59,7 +58,20 @@ k_cat_partials(const T* __restrict__ w, const T* __restrict__ nbar, int64_t n, d
       acc(3, p4, e4);
       acc(4, p5, e5);
       wmax = fmaxf(wmax, fabsf(wi));
+    };
+    // four objects' loads in flight per thread
+    int64_t i = beg + threadIdx.x;
+    for (; i + 3 * RED_THREADS < end; i += 4 * RED_THREADS) {
+      float wv[4], nv[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        wv[k] = w ? (float)w[i + k * RED_THREADS] : 1.0f;
+        nv[k] = nbar ? (float)nbar[i + k * RED_THREADS] : 0.0f;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) add(wv[k], nv[k]);
     }
+    for (; i < end; i += RED_THREADS) add(w ? (float)w[i] : 1.0f, nbar ? (float)nbar[i] : 0.0f);
 #pragma unroll
     for (int k = 0; k < NSUM - 1; ++k) a[k] = (double)hs[k] + (double)ls[k];
     a[NSUM - 1] = (double)wmax;
@@ -79,41 +91,53 @@ k_cat_partials(const T* __restrict__ w, const T* __restrict__ nbar, int64_t n, d
 #pragma unroll
   for (int k = 0; k < NSUM; ++k) sh[k][threadIdx.x] = a[k];
   __syncthreads();
-  for (int off = RED_THREADS / 2; off > 0; off >>= 1) {
-    if (threadIdx.x < off) {
+  // warp k reduces sum k over the block in a fixed tree: float64 adds are scarce on this part (16 cycles
+  // per warp instruction), so they are spread over the warps, with one barrier
+  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+  if (k >= NSUM) return;
+  auto comb = [&](double x, double y) { return k == NSUM - 1 ? fmax(x, y) : x + y; };
+  double v[RED_THREADS / 32];
 #pragma unroll
-      for (int k = 0; k < NSUM - 1; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + off];
-      sh[NSUM - 1][threadIdx.x] = fmax(sh[NSUM - 1][threadIdx.x], sh[NSUM - 1][threadIdx.x + off]);
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x < NSUM) part[blockIdx.x * NSUM + threadIdx.x] = sh[threadIdx.x][0];
+  for (int j = 0; j < RED_THREADS / 32; ++j) v[j] = sh[k][lane + 32 * j];
+#pragma unroll
+  for (int off = RED_THREADS / 64; off > 0; off >>= 1)
+#pragma unroll
+    for (int j = 0; j < off; ++j) v[j] = comb(v[j], v[j + off]);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v[0] = comb(v[0], __shfl_down_sync(0xffffffffu, v[0], off));
+  if (lane == 0) part[blk * NSUM + k] = v[0];
 }
 
-// One warp: lane l sums the partials of blocks l, l+32, ... in order, then a fixed shuffle tree;
-// the reduction order depends only on nblk (bitwise reproducible).
-__global__ void k_cat_final(const double* __restrict__ pd, const double* __restrict__ pr, int nblk,
-                            int have_randoms, double box, double* __restrict__ sc) {
-  const int lane = threadIdx.x & 31;
-  if (threadIdx.x >= 32) return;
-  double g[NSUM] = {0, 0, 0, 0, 0, 0}, r[NSUM] = {0, 0, 0, 0, 0, 0};
-  for (int b = lane; b < nblk; b += 32) {
-    for (int k = 0; k < NSUM - 1; ++k) g[k] += pd[b * NSUM + k];
-    g[NSUM - 1] = fmax(g[NSUM - 1], pd[b * NSUM + NSUM - 1]);
-    if (have_randoms) {
-      for (int k = 0; k < NSUM - 1; ++k) r[k] += pr[b * NSUM + k];
-      r[NSUM - 1] = fmax(r[NSUM - 1], pr[b * NSUM + NSUM - 1]);
-    }
+// grid (blocks, 1 or 2): per-block partial sums of the data (y = 0) and of the randoms (y = 1)
+template <typename T, typename U>
+__global__ void __launch_bounds__(RED_THREADS)
+k_cat_partials(const T* __restrict__ wd, const T* __restrict__ nd, int64_t n_d, const U* __restrict__ wr,
+               const U* __restrict__ nr, int64_t n_r, double* __restrict__ pd, double* __restrict__ pr) {
+  if (blockIdx.y == 0) cat_partial<T>(wd, nd, n_d, gridDim.x, blockIdx.x, pd);
+  else cat_partial<U>(wr, nr, n_r, gridDim.x, blockIdx.x, pr);
+}
+
+// Warp w sums sum w % NSUM of catalogue w / NSUM: lane l takes the partials of blocks l, l+32, ... in
+// order, then a fixed shuffle tree; the order depends only on nblk (bitwise reproducible).  One warp for
+// all twelve took 25 us over 1024 blocks.
+__global__ void __launch_bounds__(2 * NSUM * 32)
+k_cat_final(const double* __restrict__ pd, const double* __restrict__ pr, int nblk, int have_randoms, double box,
+            double* __restrict__ sc) {
+  __shared__ double s_sum[2 * NSUM];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = warp % NSUM;
+  double v = 0.0;
+  if (warp < NSUM || have_randoms) {
+    const double* __restrict__ p = warp < NSUM ? pd : pr;
+    for (int b = lane; b < nblk; b += 32) v = k == NSUM - 1 ? fmax(v, p[b * NSUM + k]) : v + p[b * NSUM + k];
   }
   for (int off = 16; off > 0; off >>= 1) {
-    for (int k = 0; k < NSUM - 1; ++k) {
-      g[k] += __shfl_down_sync(0xffffffffu, g[k], off);
-      r[k] += __shfl_down_sync(0xffffffffu, r[k], off);
-    }
-    g[NSUM - 1] = fmax(g[NSUM - 1], __shfl_down_sync(0xffffffffu, g[NSUM - 1], off));
-    r[NSUM - 1] = fmax(r[NSUM - 1], __shfl_down_sync(0xffffffffu, r[NSUM - 1], off));
+    const double o = __shfl_down_sync(0xffffffffu, v, off);
+    v = k == NSUM - 1 ? fmax(v, o) : v + o;
   }
-  if (lane != 0) return;
+  if (lane == 0) s_sum[warp] = v;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  const double *g = s_sum, *r = s_sum + NSUM;
   for (int k = 0; k < SC_COUNT; ++k) sc[k] = 0.0;
   if (have_randoms) {
     const double alpha = g[0] / r[0];
@@ -941,6 +965,21 @@ npc_status paint_impl(npc_ctx* ctx, const DevCatalog& d, const DevCatalog* r, co
   return launch_fold<T>(ctx, tiles, g, nphase, sc, sub, mesh_a, mesh_b);
 }
 
+// Partial sums of one or two catalogues (types 0 float, 1 double) in one launch.
+void launch_cat_partials(const void* wd, const void* nd, int64_t n_d, int type_d, const void* wr, const void* nr,
+                         int64_t n_r, int type_r, int ncat, int nblk, double* pd, double* pr, cudaStream_t st) {
+  auto run = [&](auto* t, auto* u) {
+    using T = std::remove_pointer_t<decltype(t)>;
+    using U = std::remove_pointer_t<decltype(u)>;
+    k_cat_partials<T, U><<<dim3(nblk, ncat), RED_THREADS, 0, st>>>((const T*)wd, (const T*)nd, n_d, (const U*)wr,
+                                                                   (const U*)nr, n_r, pd, pr);
+  };
+  float* f = nullptr;
+  double* d = nullptr;
+  if (type_d == 1) type_r == 1 ? run(d, d) : run(d, f);
+  else type_r == 1 ? run(f, d) : run(f, f);
+}
+
 // Scalars of a cross spectrum from those of tracers A and B: the normalisation sqrt(I22^A I22^B)
 // in the I22 slot, no shot noise, and the tracers' own values for the output (layout in npc.h).
 __global__ void k_cross_scalars(const double* __restrict__ sa, const double* __restrict__ sb, double* __restrict__ sx) {
@@ -983,25 +1022,15 @@ npc_status launch_cross_scalars(npc_ctx* ctx, const double* sa, const double* sb
 
 npc_status launch_catalog_scalars(npc_ctx* ctx, const DevCatalog& d, const DevCatalog* r, double box,
                                   double* dev_scalars) {
+  const int64_t nmax = std::max<int64_t>(d.n, r ? r->n : 0);
+  const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((nmax + RED_CHUNK - 1) / RED_CHUNK, 4 * ctx->num_sms));
   double* part;
-  NPC_TRY(ws_get(ctx, "scalars.part", sizeof(double) * NSUM * RED_BLOCKS * 2, (void**)&part));
-  if (d.dtype == 1)
-    k_cat_partials<double><<<RED_BLOCKS, RED_THREADS, 0, ctx->stream>>>((const double*)d.w, (const double*)d.nbar,
-                                                                         d.n, part);
-  else
-    k_cat_partials<float><<<RED_BLOCKS, RED_THREADS, 0, ctx->stream>>>((const float*)d.w, (const float*)d.nbar,
-                                                                        d.n, part);
+  NPC_TRY(ws_get(ctx, "scalars.part", sizeof(double) * NSUM * 4 * ctx->num_sms * 2, (void**)&part));
+  double* part_r = part + (size_t)NSUM * nblk;
+  launch_cat_partials(d.w, d.nbar, d.n, d.dtype, r ? r->w : nullptr, r ? r->nbar : nullptr, r ? r->n : 0,
+                      r ? r->dtype : d.dtype, r ? 2 : 1, nblk, part, part_r, ctx->stream);
   NPC_LAUNCH(ctx);
-  if (r) {
-    if (r->dtype == 1)
-      k_cat_partials<double><<<RED_BLOCKS, RED_THREADS, 0, ctx->stream>>>(
-          (const double*)r->w, (const double*)r->nbar, r->n, part + NSUM * RED_BLOCKS);
-    else
-      k_cat_partials<float><<<RED_BLOCKS, RED_THREADS, 0, ctx->stream>>>(
-          (const float*)r->w, (const float*)r->nbar, r->n, part + NSUM * RED_BLOCKS);
-    NPC_LAUNCH(ctx);
-  }
-  k_cat_final<<<1, 32, 0, ctx->stream>>>(part, part + NSUM * RED_BLOCKS, RED_BLOCKS, r ? 1 : 0, box, dev_scalars);
+  k_cat_final<<<1, 2 * NSUM * 32, 0, ctx->stream>>>(part, part_r, nblk, r ? 1 : 0, box, dev_scalars);
   NPC_LAUNCH(ctx);
   return NPC_OK;
 }
@@ -1145,16 +1174,10 @@ extern "C" npc_status npc_catalog_scalars_noalloc(const npc_catalog* data, const
   double* sc = scratch + 2 * NOALLOC_PART;
   // every partial that k_cat_final reads is written by this call's k_cat_partials (blocks past the
   // end of a catalogue write zeros), so nothing needs clearing first
-  for (int c = 0; c < 2; ++c) {
-    const npc_catalog* k = cats[c];
-    if (!k) continue;
-    double* part = c == 0 ? part_d : part_r;
-    if (k->dtype == 1)
-      k_cat_partials<double><<<nblk, RED_THREADS, 0, st>>>((const double*)k->w, (const double*)k->nbar, k->n, part);
-    else
-      k_cat_partials<float><<<nblk, RED_THREADS, 0, st>>>((const float*)k->w, (const float*)k->nbar, k->n, part);
-  }
-  k_cat_final<<<1, 32, 0, st>>>(part_d, part_r, nblk, randoms ? 1 : 0, box, sc);
+  launch_cat_partials(data->w, data->nbar, data->n, data->dtype, randoms ? randoms->w : nullptr,
+                      randoms ? randoms->nbar : nullptr, randoms ? randoms->n : 0,
+                      randoms ? randoms->dtype : data->dtype, randoms ? 2 : 1, nblk, part_d, part_r, st);
+  k_cat_final<<<1, 2 * NSUM * 32, 0, st>>>(part_d, part_r, nblk, randoms ? 1 : 0, box, sc);
   // peek, not get: an error that the caller's earlier asynchronous work left pending is reported
   // as this call's failure but stays pending for the caller to read
   cudaError_t e = cudaPeekAtLastError();
