@@ -106,14 +106,27 @@ npc_status get_twiddles(npc_ctx* ctx, int n, int prec, const void** out) {
     *out = p;
     return NPC_OK;
   }
+  // exponent j of entry i: natural for composite lengths, stage by stage for powers of two (twiddle_offset)
+  std::vector<int> expo(n, 0);
+  if (n & (n - 1)) {
+    for (int j = 0; j < n; ++j) expo[j] = j;
+  } else {
+    int i = 0;
+    for (int span = 8; span < n; span *= 8) {
+      const int radix = std::min(8, n / span);
+      for (int r = 1; r < radix; ++r)
+        for (int k = 0; k < span; ++k) expo[i++] = r * k * (n / (span * radix));
+    }
+  }
   if (prec == NPC_PREC_FP64) {
     std::vector<double2> h(n);
-    for (int j = 0; j < n; ++j) h[j] = make_double2(std::cos(2.0 * M_PI * j / n), -std::sin(2.0 * M_PI * j / n));
+    for (int i = 0; i < n; ++i)
+      h[i] = make_double2(std::cos(2.0 * M_PI * expo[i] / n), -std::sin(2.0 * M_PI * expo[i] / n));
     NPC_TRY(ws_table(ctx, name, key, h.data(), sizeof(double2) * n, &p));
   } else {
     std::vector<float2> h(n);
-    for (int j = 0; j < n; ++j)
-      h[j] = make_float2((float)std::cos(2.0 * M_PI * j / n), (float)-std::sin(2.0 * M_PI * j / n));
+    for (int i = 0; i < n; ++i)
+      h[i] = make_float2((float)std::cos(2.0 * M_PI * expo[i] / n), (float)-std::sin(2.0 * M_PI * expo[i] / n));
     NPC_TRY(ws_table(ctx, name, key, h.data(), sizeof(float2) * n, &p));
   }
   *out = p;

@@ -59,19 +59,31 @@ __device__ __forceinline__ void dft8(C (&v)[8]) {
 }
 
 // Shared-memory views used for the inter-stage exchange.  sub(off) is the view of the elements
-// from `off` on (off a multiple of 8), used by the sub-transforms of a composite length.
+// from `off` on (off a multiple of 8), used by the sub-transforms of a composite length.  The exchange
+// after the stage with span Ns writes and reads through put<Ns> / get<Ns>.
 template <typename C> struct ColView {  // element n of column at p[n*stride]
   C* p;
   int stride;
   __device__ __forceinline__ void st(int n, C v) const { p[n * stride] = v; }
   __device__ __forceinline__ C ld(int n) const { return p[n * stride]; }
+  template <int Ns> __device__ __forceinline__ void put(int n, C v) const { st(n, v); }
+  template <int Ns> __device__ __forceinline__ C get(int n) const { return ld(n); }
   __device__ __forceinline__ ColView sub(int off) const { return ColView{p + off * stride, stride}; }
 };
-template <typename C> struct RowView {  // element n at p[n + n/8] (one pad slot per 8)
+// Element n at p[n + n/8] (one pad slot per 8).  The exchanges pad for their own pattern, so that the 16
+// lanes of an 8-byte access meet distinct banks both ways: after span 1 thread b writes 8 b + r (one slot
+// per 16), after span 8 it writes 64 (b div 8) + (b mod 8) + 8 r (eight slots per 64), later spans write
+// runs of 64; all read runs t, t + 1, ...  (With one slot per 8 throughout every read took two passes.)
+template <typename C> struct RowView {
   C* p;
   __device__ __forceinline__ static int idx(int n) { return n + (n >> 3); }
+  template <int Ns> __device__ __forceinline__ static int pos(int n) {
+    return Ns == 1 ? n + (n >> 4) : (Ns == 8 ? n + ((n >> 6) << 3) : n);
+  }
   __device__ __forceinline__ void st(int n, C v) const { p[idx(n)] = v; }
   __device__ __forceinline__ C ld(int n) const { return p[idx(n)]; }
+  template <int Ns> __device__ __forceinline__ void put(int n, C v) const { p[pos<Ns>(n)] = v; }
+  template <int Ns> __device__ __forceinline__ C get(int n) const { return p[pos<Ns>(n)]; }
   __device__ __forceinline__ RowView sub(int off) const { return RowView{p + idx(off)}; }
 };
 template <int N> __host__ __device__ constexpr int row_pad_len() { return N + N / 8; }
@@ -109,11 +121,20 @@ struct SyncNamed {
   }
 };
 
-// All threads that share `buf` must call this the same number of times (it contains barriers).
-// TS: stride into the twiddle table (a length-N/TS sub-transform reads every TS-th twiddle of N).
-template <int N, int DIR, int Ns, int TS = 1, typename C, typename View, typename Sync = SyncBlock>
-__device__ __forceinline__ void fft_stages(C (&v)[8], const int t, const C* __restrict__ tw,
-                                           const View& buf, const Sync& sync = Sync()) {
+// Twiddle tables.  Powers of two: stage by stage, for the stage with span Ns > 1 and radix R the factors
+// w^(r k), w = exp(-2 pi i/(Ns R)), at twiddle_offset(N, Ns) + (r - 1) Ns + k, so that the lanes of one
+// access (consecutive k) read consecutive entries (from the natural order w_N^j they meet strides of
+// r N/(Ns R), up to eight lanes on one bank).  At most N entries.  Composite lengths: w_N^j, j < N.
+__host__ __device__ constexpr int twiddle_offset(int n, int span) {
+  int off = 0;
+  for (int s = 8; s < span; s *= 8) off += ((n / s >= 8 ? 8 : n / s) - 1) * s;
+  return off;
+}
+
+// Butterflies of the stage with span Ns on the thread's elements.  TS: stride into the natural twiddle
+// table (a length-N/TS sub-transform reads every TS-th twiddle of N); 1: the stage-by-stage table.
+template <int N, int DIR, int Ns, int TS, typename C>
+__device__ __forceinline__ void fft_butterflies(C (&v)[8], const int t, const C* __restrict__ tw) {
   constexpr int TPF = N / 8;
   constexpr int REM = N / Ns;
   constexpr int R = (REM >= 8) ? 8 : REM;
@@ -126,8 +147,8 @@ __device__ __forceinline__ void fft_stages(C (&v)[8], const int t, const C* __re
       const int k = b & (Ns - 1);
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        const int j = r * k * (N / (Ns * R));
-        v[s + r * BPT] = cmul(v[s + r * BPT], twiddle<C, DIR>(tw, j * TS));
+        const int j = TS == 1 ? twiddle_offset(N, Ns) + (r - 1) * Ns + k : r * k * (N / (Ns * R)) * TS;
+        v[s + r * BPT] = cmul(v[s + r * BPT], twiddle<C, DIR>(tw, j));
       }
     }
     if constexpr (R == 8) {
@@ -138,19 +159,60 @@ __device__ __forceinline__ void fft_stages(C (&v)[8], const int t, const C* __re
       bfly2(v[s], v[s + BPT]);
     }
   }
+}
+
+// All threads that share `buf` must call this the same number of times (it contains barriers).
+template <int N, int DIR, int Ns, int TS = 1, typename C, typename View, typename Sync = SyncBlock>
+__device__ __forceinline__ void fft_stages(C (&v)[8], const int t, const C* __restrict__ tw,
+                                           const View& buf, const Sync& sync = Sync()) {
+  constexpr int TPF = N / 8;
+  constexpr int REM = N / Ns;
+  constexpr int R = (REM >= 8) ? 8 : REM;
+  constexpr int BPT = 8 / R;
+  fft_butterflies<N, DIR, Ns, TS>(v, t, tw);
   if constexpr (Ns * R < N) {
 #pragma unroll
     for (int s = 0; s < BPT; ++s) {
       const int b = t + s * TPF;
       const int base = (b / Ns) * Ns * R + (b & (Ns - 1));
 #pragma unroll
-      for (int r = 0; r < R; ++r) buf.st(base + r * Ns, v[s + r * BPT]);
+      for (int r = 0; r < R; ++r) buf.template put<Ns>(base + r * Ns, v[s + r * BPT]);
     }
     sync();
 #pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = buf.ld(t + q * TPF);
+    for (int q = 0; q < 8; ++q) v[q] = buf.template get<Ns>(t + q * TPF);
     sync();
     fft_stages<N, DIR, Ns * R, TS>(v, t, tw, buf, sync);
+  }
+}
+
+// The same stages with the exchanges alternating between two buffers: a buffer is written again only
+// after the barrier of the exchange through the other one, so one barrier per exchange is enough.  A
+// caller that transforms row after row swaps the two when fft_exchanges<N>() is odd.
+template <int N> constexpr int fft_exchanges(int span = 1) {
+  return N / span <= 8 ? 0 : 1 + fft_exchanges<N>(span * 8);
+}
+template <int N, int DIR, int Ns = 1, typename C, typename View, typename Sync>
+__device__ __forceinline__ void fft_block_alternate(C (&v)[8], const int t, const C* __restrict__ tw, const View& buf,
+                                                    const View& other, const Sync& sync) {
+  static_assert(FftLen<N>::pow2, "alternating exchanges are for powers of two");
+  constexpr int TPF = N / 8;
+  constexpr int REM = N / Ns;
+  constexpr int R = (REM >= 8) ? 8 : REM;
+  constexpr int BPT = 8 / R;
+  fft_butterflies<N, DIR, Ns, 1>(v, t, tw);
+  if constexpr (Ns * R < N) {
+#pragma unroll
+    for (int s = 0; s < BPT; ++s) {
+      const int b = t + s * TPF;
+      const int base = (b / Ns) * Ns * R + (b & (Ns - 1));
+#pragma unroll
+      for (int r = 0; r < R; ++r) buf.template put<Ns>(base + r * Ns, v[s + r * BPT]);
+    }
+    sync();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = buf.template get<Ns>(t + q * TPF);
+    fft_block_alternate<N, DIR, Ns * R>(v, t, tw, other, buf, sync);
   }
 }
 

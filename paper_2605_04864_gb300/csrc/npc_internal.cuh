@@ -325,7 +325,7 @@ npc_status run_power_contract(npc_ctx* ctx, int prec, const PowerPlan& plan, con
 // bin table: int16 per integer |k|^2 in [0, 3 (n/2)^2]
 // slots: 0 power spectrum, 2-3 bispectrum, 4 mesh-level adjoint (tables stay cached per slot)
 npc_status get_bin_table(npc_ctx* ctx, int n, double box, const npc_kbins& kb, const int16_t** out, int slot = 0);
-// twiddle table exp(-2 pi i j / n), j < n, as cplx<T>
+// twiddle table of length-n transforms (n entries, laid out as fft_core.cuh describes), as cplx<T>
 npc_status get_twiddles(npc_ctx* ctx, int n, int prec, const void** out);
 
 // ---------------------------------------------------------------------------------------------

@@ -30,7 +30,8 @@
 namespace {
 
 constexpr int CONTRACT_THREADS = 256;
-constexpr int MAX_SUMS = 10;
+constexpr int MAX_PRODS = 8;              // P_0 .. P_4 and P_22, P_42, P_44
+constexpr int MAX_SUMS = MAX_PRODS + 2;   // and the modes and their |k|
 
 template <int N> struct ColCfg {
   static constexpr int TX = N >= 1024 ? 4 : (N >= 512 ? 8 : 16);  // TX <= N
@@ -492,51 +493,42 @@ k_fft_cols(cplx<T>* __restrict__ data, size_t plane_stride, int row_stride, cons
   }
 }
 
-// Per stored real field: which F_l it feeds, its mesh phase and its k-space coefficient
-// scale * (ReY or ImY)(khat) from the row's Y table (scale = 4 pi/(2l+1) * (m > 0 ? 2 : 1)).
-struct FieldCoef {
-  int8_t acc;    // 0, 1, 2 for F_0, F_2, F_4
-  int8_t phase;  // 0 or 1
-  int8_t yidx;   // row Y-table index, -1 for PART_ONE
-  int8_t part;   // PART_RE / PART_IM / PART_ONE
+// One step of the x pass: a stored real field, its k-space coefficient scale * part of Q_lm(uz)
+// (ux + i uy)^m (scale = 4 pi/(2l+1) * (m > 0 ? 2 : 1) * the norm of Y_lm), and what follows it.
+struct FieldStep {
+  int8_t field;  // index into the half-spectrum buffer
+  int8_t weight; // 2 (l(l+1)/2 + m) + (1 for the imaginary part); 0: no weight (F_0, global line of sight)
+  int8_t acc;    // accumulator of the step's multipole
+  int8_t flags;  // STEP_ROTATE, STEP_STORE
   float scale_f;
   double scale_d;
 };
-template <typename T> __device__ __forceinline__ T coef_scale(const FieldCoef& c);
-template <> __device__ __forceinline__ float coef_scale<float>(const FieldCoef& c) { return c.scale_f; }
-template <> __device__ __forceinline__ double coef_scale<double>(const FieldCoef& c) { return c.scale_d; }
+// the accumulator holds phase b only so far: apply the interlacing phase e^{i pi (i + j + l)/N}
+constexpr int8_t STEP_ROTATE = 1;
+// the accumulator's last field: apply the window factor and store F_l
+constexpr int8_t STEP_STORE = 2;
+template <typename T> __device__ __forceinline__ T step_scale(const FieldStep& c);
+template <> __device__ __forceinline__ float step_scale<float>(const FieldStep& c) { return c.scale_f; }
+template <> __device__ __forceinline__ double step_scale<double>(const FieldStep& c) { return c.scale_d; }
 
-// Row Y table: Y_lm(khat) in the fixed order (2,0) (2,1) (2,2) (4,0) .. (4,4) (1,0) (1,1) (3,0) .. (3,3).
-constexpr int MAX_YTAB = 14;
-__host__ __device__ constexpr int ytab_index(int l, int m) {
-  return l == 2 ? m : (l == 4 ? 3 + m : (l == 1 ? 8 + m : 10 + m));
-}
-// Field slots of the x pass: slot[r * G + g] is the field row group g transforms in round r.
-constexpr int MAX_SLOTS = 256;
+// A binned sum: Re (Im, when one of the two l is odd) of F_lx F_ly^*, and the accumulators that hold them
+// (F_0's for every l with a global line of sight).
+struct SumDesc {
+  int8_t lx, ly, acc_x, acc_y;
+};
 
 struct ContractParams {
-  int nf;
-  FieldCoef fc[NPC_MAX_FIELDS];
-  int ny;                       // Y table rows: 0, 3 (l = 2) or 8 (l = 2 and 4)
-  int nacc;                     // F accumulators: nacc_b of F_0, F_2, F_4, then F_0^A if cross
-  int nacc_b;
-  int acc_a;                    // accumulator of F_0^A (cross spectra), -1 otherwise
+  int nsteps;
+  FieldStep step[NPC_MAX_FIELDS];   // grouped by accumulator, phase b before phase a
+  int nacc;                     // F accumulators: of F_0, F_1, ... of tracer B, then F_0^A if cross
   int nphase;
-  int nrounds;                  // rounds of G field rows
-  int phase_pure;               // 1: every group sees one mesh phase only (group parity when nphase = 2)
-  int8_t slot[MAX_SLOTS];       // field per (round, group), -1 for none
+  int pair_rows;                // rows ky and -ky are binned together
+  int shared_part;              // the warps' partial sums are kept in shared memory
   int nbins, nsum;
   int row_n2max;                // rows (ky, kz) with ky^2 + kz^2 above this hold no binned mode
   int KZ;                       // planes kz < KZ stored per field by the forward passes
-  int nell;
-  int ell_list[5];
-  int nll;
-  int lla[3], llb[3];
-  int need2, need4;
-  int need_mask;                // multipoles l whose F_l the binning forms (bit l)
-  int acc_of[5];                // accumulator of F_l (tracer B), -1 if none
-  int ymask;                    // Y table groups evaluated per row: bit l for l = 1 .. 4
-  int even_layout;              // acc_of = {0, -1, 1 or -1, -1, 2 or -1}: the fixed even-l layout
+  int nprod;                    // product sums; then the modes and their |k| are summed
+  SumDesc sum[MAX_PRODS];
   int global_los;
   double los[3];
   int assign;
@@ -554,281 +546,313 @@ __device__ __forceinline__ T sinc_pow(T a, int p) {
 __device__ __forceinline__ void sincospi_t(float x, float* s, float* c) { sincospif(x, s, c); }
 __device__ __forceinline__ void sincospi_t(double x, double* s, double* c) { sincospi(x, s, c); }
 
-template <int N> struct XCfg {
+// L_l(mu), l <= 4, as polynomials (uniform l, no division)
+template <typename T> __device__ __forceinline__ T legendre_0to4(int l, T mu) {
+  const T m2 = mu * mu;
+  switch (l) {
+    case 0: return T(1);
+    case 1: return mu;
+    case 2: return T(1.5) * m2 - T(0.5);
+    case 3: return mu * (T(2.5) * m2 - T(1.5));
+  }
+  return (T(4.375) * m2 - T(3.75)) * m2 + T(0.375);
+}
+
+// Threads of a CTA that meet at one barrier in the x pass: the warps of one row where a row takes whole
+// warps, one warp holding several rows where rows pack into a warp, else (lengths 3 * 2^k) the block.
+template <int N> struct XTeam {
   static constexpr int TPF = N / 8;
-  static constexpr int G = RowGroups<N, CONTRACT_THREADS>::G;        // rows in flight
-  static constexpr int NBUF = RowGroups<N, CONTRACT_THREADS>::NBUF;  // exchange buffers
+  static constexpr bool BLOCK = !(TPF % 32 == 0 || 32 % TPF == 0);
+  static constexpr int SIZE = TPF > 32 ? TPF : 32;   // of a team, unless BLOCK
+  // exchange buffers per row: two where every exchange of the transform writes the other one, which
+  // leaves one barrier per exchange
+  static constexpr int XBUF = BLOCK ? 1 : 2;
+  // slots per row: the buffers, and for rows of fewer than 16 threads an offset that puts the rows of one
+  // 16-lane access on different banks
+  static constexpr int ROW = XBUF * row_pad_len<N>() + (TPF < 16 ? TPF : 0);
+  // threads per CTA: whole warps of whole rows for the lengths 3 * 2^k
+  static constexpr int THREADS = BLOCK ? 96 : CONTRACT_THREADS;
 };
 
-// Last pass.  For one (ky, kz) row: every field row is transformed along x and added, with its
-// coefficient, into per-group F_l accumulators (F_l is linear in the fields, so the 30 rows never
-// need to be resident together); then per mode the products Re[F_0 F_l^*], Re[F_l F_l'^*] are
-// binned.  Groups own their accumulators and threads own their modes, so no shared-memory
-// atomics are needed, and the group sum runs in a fixed order.
-template <typename T, int N>
-__global__ void __launch_bounds__(CONTRACT_THREADS, 2)
-k_fft_x_contract(const cplx<T>* __restrict__ half, const ContractParams P, const YNorm nrm,
+// v[q] (mode kx = t + q TPF) times scale * the part of Q_LM(uz) (ux + i uy)^M, added to acc.
+template <typename T, int N, int L, int M, int IM>
+__device__ __forceinline__ void add_weighted(cplx<T> (&acc)[8], const cplx<T> (&v)[8], const T (&inv)[8], T scale,
+                                             int t, T fj, T fk) {
+  constexpr int TPF = N / 8;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    T iv = inv[q];
+    keep_here(iv);   // the weights of the other fields must not be formed beside this one's
+    const T ux = T(t + (q < 4 ? q : q - 8) * TPF) * iv, uy = fj * iv;
+    T pr = T(1), pi = T(0);
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+      const T nr = pr * ux - pi * uy;
+      pi = pr * uy + pi * ux;
+      pr = nr;
+    }
+    const T w = scale * (ylm_q<T, L, M>(fk * iv) * (IM ? pi : pr));
+    acc[q] = cmk(acc[q].x + w * v[q].x, acc[q].y + w * v[q].y);
+  }
+}
+
+// Last pass.  A group of N/8 threads owns a row (ky, kz): it transforms the row of every field along x,
+// one after the other, and adds it with its coefficient to one F_l accumulator in registers (F_l is
+// linear in the fields, and they come grouped by multipole, so one accumulator is live at a time); the
+// finished F_l go to the group's shared memory, from which the team's threads form the products
+// Re[F_0 F_l^*], Re[F_l F_l'^*] per pair of mirror modes and bin them.  Groups of one or more warps never
+// wait for each other.  The modes (kx, ky) with either sign of each have one |k|, hence one bin: all four
+// (the two signs of kx where rows are not paired) are added before the warp-segmented scan.
+template <typename T, int N, int MINB>
+__global__ void __launch_bounds__(CONTRACT_THREADS, MINB)
+k_fft_x_contract(const cplx<T>* __restrict__ half, const __grid_constant__ ContractParams P,
                  const int16_t* __restrict__ bintab, const cplx<T>* __restrict__ tw_g, double* __restrict__ part) {
   using C = cplx<T>;
-  constexpr int TPF = XCfg<N>::TPF;
-  constexpr int G = XCfg<N>::G;
+  using Team = XTeam<N>;
+  constexpr int TPF = Team::TPF;
   constexpr int NP = row_pad_len<N>();
-  constexpr int NW = CONTRACT_THREADS / 32;
+  const int G = blockDim.x / TPF;             // rows in flight
+  const int nw = blockDim.x >> 5;
+  const int nbuf = G + (Team::BLOCK && blockDim.x % TPF ? 1 : 0);   // threads left over transform zeros
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
-  C* ytab = tw + N;                         // [ny][N]
-  C* facc = ytab + (size_t)P.ny * N;        // [G][nacc][N]
-  C* rowbuf = facc + (size_t)G * P.nacc * N;  // [G][NP]
-  C* fb = rowbuf + (size_t)XCfg<N>::NBUF * NP;  // phase-b factor per kx: fa e^{i pi (i+j+l)/N}
-  T* winv = reinterpret_cast<T*>(fb + N);   // 1/sinc^p, a = 0..N/2
-  T* fa = winv + (N / 2 + 2);               // phase-a factor per kx
-  const int tid = threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
+  C* phs = tw + N;                            // e^{i pi m/N}, m = -N .. N-1
+  C* rowbuf = phs + 2 * N;                    // [nbuf][ROW]
+  C* fsm = rowbuf + (size_t)nbuf * Team::ROW;   // [G][1 or 2 rows][nacc][N]
+  const int nslot = P.pair_rows ? 2 : 1;
+  T* winv = reinterpret_cast<T*>(fsm + (size_t)G * nslot * P.nacc * N);   // 1/sinc^p, a = 0..N/2
+  double* spart = reinterpret_cast<double*>(smem_raw + (((reinterpret_cast<unsigned char*>(winv + N / 2 + 2) - smem_raw) + 15) & ~(size_t)15));
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nent = P.nbins * P.nsum;
   for (int i = tid; i < N; i += blockDim.x) tw[i] = tw_g[i];
   for (int i = tid; i <= N / 2; i += blockDim.x) winv[i] = T(1) / sinc_pow<T>(T(M_PI) * T(i) / T(N), P.assign);
+  for (int i = tid; i < 2 * N; i += blockDim.x) {
+    T sn, cs;
+    sincospi_t(T(i - N) / T(N), &sn, &cs);
+    phs[i] = cmk(cs, sn);
+  }
+  if (P.shared_part)
+    for (int i = tid; i < nw * nent; i += blockDim.x) spart[i] = 0.0;
   __syncthreads();
-  double* mypart = part + ((size_t)blockIdx.x * NW + warp) * P.nbins * P.nsum;
-  const int nrows = P.KZ * N;
+  double* mypart = P.shared_part ? spart + (size_t)warp * nent : part + ((size_t)blockIdx.x * nw + warp) * nent;
   const int g = tid / TPF, t = tid % TPF;
   const bool ingroup = g < G;
+  const size_t fstride = (size_t)P.KZ * N * N;
   const T half_or_one = P.nphase == 2 ? T(0.5) : T(1);
-  for (int r = blockIdx.x; r < nrows; r += gridDim.x) {
-    const int kz = r / N, ky = r % N;
-    const int jy = ky < N / 2 ? ky : ky - N;
-    if (jy * jy + kz * kz > P.row_n2max) continue;   // block-uniform: the whole row is outside the bins
-    // per-mode window/interlace factor and Y_lm(khat) table; clear the accumulators
-    for (int kx = tid; kx < N; kx += blockDim.x) {
-      const int i = kx < N / 2 ? kx : kx - N;
-      const int ai = i < 0 ? -i : i, aj = jy < 0 ? -jy : jy;
-      fa[kx] = half_or_one * winv[ai] * winv[aj] * winv[kz];
-      {
-        // interlacing phase e^{i pi (i + j + l)/N}, the argument reduced to (-1, 1] half turns
-        int m = i + jy + kz;
-        m = ((m % (2 * N)) + 2 * N) % (2 * N);
-        if (m > N) m -= 2 * N;
-        T sn, cs;
-        sincospi_t(T(m) / T(N), &sn, &cs);
-        fb[kx] = cmk(cs * fa[kx], sn * fa[kx]);
+  // items (kz, |ky|), ky >= 0 before -ky
+  const int nitems = P.KZ * (N / 2), istep = gridDim.x * G;
+  auto in_bins = [&](int item) {
+    const int kz = item / (N / 2), ay = item % (N / 2);
+    return item < nitems && kz * kz + ay * ay <= P.row_n2max;
+  };
+  // first item at or after `item` (steps of istep) with modes in the bins
+  auto seek = [&](int item) {
+    while (item < nitems && !in_bins(item)) item += istep;
+    return item;
+  };
+  auto row_of = [&](int item, int sgn) {
+    const int kz = item / (N / 2), ay = item % (N / 2);
+    return half + ((size_t)kz * N + (sgn && ay ? N - ay : ay)) * N;
+  };
+  // team-uniform loop: a team's groups (rows of one warp, or of the block) go on until none has an item
+  int item = ingroup ? blockIdx.x * G + g : nitems;
+  if (!Team::BLOCK) item = seek(item);
+  int pass = 0, flip = 0;
+  C* bufs = rowbuf + (size_t)(ingroup ? g : G) * Team::ROW;
+  C v[8], vn[8];
+  if (in_bins(item)) {
+    const C* src = row_of(item, 0) + (size_t)P.step[0].field * fstride;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = src[t + q * TPF];
+  }
+  auto team_sync = [&]() {
+    if constexpr (Team::BLOCK) __syncthreads();
+    else if constexpr (TPF <= 32) __syncwarp();
+    else SyncNamed{1 + g, TPF}();
+  };
+  auto team_any = [&](bool p) -> bool {
+    if constexpr (Team::BLOCK) return __syncthreads_or(p);
+    else if constexpr (TPF < 32) return __any_sync(0xffffffffu, p);
+    else return p;
+  };
+  while (team_any(item < nitems)) {
+    const bool live0 = in_bins(item);
+    const int next = Team::BLOCK ? item + istep : seek(item + istep);
+    // (a group without an item transforms zeros with its team: its table look-ups stay in range)
+    const int kz = live0 ? item / (N / 2) : 0, ay = live0 ? item % (N / 2) : 0;
+    if (!Team::BLOCK || team_any(live0)) {
+#pragma unroll 1
+      for (int sgn = 0; sgn < 2; ++sgn) {
+        const bool live = live0 && (sgn == 0 || ay > 0);
+        const int jy = sgn ? -ay : ay;
+        // |k| of the thread's modes, and the row's factor of the window
+        T inv[8];
+        C racc[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const T fi = T(t + (q < 4 ? q : q - 8) * TPF), fj = T(jy), fk = T(kz);
+          const T r2 = fi * fi + fj * fj + fk * fk;
+          inv[q] = r2 > T(0) ? rsqrt(r2) : T(0);
+          racc[q] = cmk(T(0), T(0));
+        }
+        if (team_any(live)) {
+#pragma unroll 1
+          for (int st = 0; st < P.nsteps; ++st) {
+            const FieldStep c = P.step[st];
+            {
+              // the row that comes next: this row's next field, else the first field of the next row
+              const bool more = st + 1 < P.nsteps;
+              const int nsgn = more ? sgn : (sgn == 0 && ay > 0 ? 1 : 0);
+              const int nitem = more || nsgn > sgn ? item : next;
+              if (more ? live : in_bins(nitem)) {
+                const C* src = row_of(nitem, nsgn) + (size_t)P.step[more ? st + 1 : 0].field * fstride;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) vn[q] = src[t + q * TPF];
+              }
+            }
+            if (!live) {
+#pragma unroll
+              for (int q = 0; q < 8; ++q) v[q] = cmk(T(0), T(0));
+            }
+            if constexpr (Team::BLOCK) {
+              fft_block<N, -1>(v, t, tw, RowView<C>{bufs}, SyncBlock{});
+            } else {
+              const RowView<C> b0{bufs + flip * NP}, b1{bufs + (flip ^ 1) * NP};
+              if constexpr (TPF <= 32) fft_block_alternate<N, -1>(v, t, tw, b0, b1, SyncWarp{});
+              else fft_block_alternate<N, -1>(v, t, tw, b0, b1, SyncNamed{1 + g, TPF});
+              flip ^= fft_exchanges<N>() & 1;
+            }
+            const T sc = step_scale<T>(c), fj = T(jy), fk = T(kz);
+#define NPC_W(L, M, IM) \
+  case 2 * (L * (L + 1) / 2 + M) + IM: add_weighted<T, N, L, M, IM>(racc, v, inv, sc, t, fj, fk); break;
+            switch (c.weight) {
+              NPC_W(1, 0, 0) NPC_W(1, 1, 0) NPC_W(1, 1, 1)
+              NPC_W(2, 0, 0) NPC_W(2, 1, 0) NPC_W(2, 1, 1) NPC_W(2, 2, 0) NPC_W(2, 2, 1)
+              NPC_W(3, 0, 0) NPC_W(3, 1, 0) NPC_W(3, 1, 1) NPC_W(3, 2, 0) NPC_W(3, 2, 1) NPC_W(3, 3, 0) NPC_W(3, 3, 1)
+              NPC_W(4, 0, 0) NPC_W(4, 1, 0) NPC_W(4, 1, 1) NPC_W(4, 2, 0) NPC_W(4, 2, 1) NPC_W(4, 3, 0) NPC_W(4, 3, 1)
+              NPC_W(4, 4, 0) NPC_W(4, 4, 1)
+              default:
+#pragma unroll
+                for (int q = 0; q < 8; ++q) racc[q] = cadd(racc[q], v[q]);
+            }
+#undef NPC_W
+            if (c.flags & STEP_ROTATE) {
+#pragma unroll
+              for (int q = 0; q < 8; ++q) {
+                int m = t + (q < 4 ? q : q - 8) * TPF + jy + kz;   // in (-N, 3N/2)
+                if (m >= N) m -= 2 * N;
+                racc[q] = cmul(racc[q], phs[m + N]);
+              }
+            }
+            if (c.flags & STEP_STORE) {
+              C* f = fsm + (((size_t)(ingroup ? g : 0) * nslot + (P.pair_rows ? sgn : 0)) * P.nacc + c.acc) * N;
+              const T wr = half_or_one * winv[ay] * winv[kz];
+#pragma unroll
+              for (int q = 0; q < 8; ++q) {
+                const int ai = q < 4 ? t + q * TPF : (8 - q) * TPF - t;
+                if (ingroup) f[t + q * TPF] = cscale(racc[q], wr * winv[ai]);
+                racc[q] = cmk(T(0), T(0));
+              }
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = vn[q];
+          }
+        }
+        if (P.pair_rows && sgn == 0) continue;
+        team_sync();
+        // bin the team's rows: tasks (row, chunk of 32 modes kx = jp >= 0 with their mirror modes)
+        constexpr int NJ = N / 2, CH = (NJ + 31) / 32;
+        const int trows = Team::BLOCK ? G : (TPF < 32 ? 32 / TPF : 1);
+        const int twarps = Team::BLOCK ? nw : (TPF > 32 ? TPF / 32 : 1);
+        const int twarp = Team::BLOCK ? warp : warp % twarps;
+        for (int task = twarp; task < trows * CH; task += twarps) {
+          const int tr = task / CH, jp = (task % CH) * 32 + lane;
+          const int gr = Team::BLOCK ? tr : (TPF < 32 ? warp * trows + tr : g);   // the task's group
+          int titem = item;
+          if constexpr (Team::BLOCK) titem = blockIdx.x * G + gr + pass * istep;
+          else if constexpr (TPF < 32) titem = __shfl_sync(0xffffffffu, item, tr * TPF);
+          if (!in_bins(titem)) continue;   // warp-uniform
+          const int tkz = titem / (N / 2), tay = titem % (N / 2);
+          int bin = -1;
+          T vals[MAX_SUMS];
+#pragma unroll
+          for (int e = 0; e < MAX_SUMS; ++e) vals[e] = T(0);
+          const int n2 = jp * jp + tay * tay + tkz * tkz;
+          if (jp < NJ && n2 > 0) bin = bintab[n2];
+          if (bin >= 0) {
+            const T wgt = tkz > 0 ? T(2) : T(1), fkz = T(tkz);
+            const T kk = sqrt(T(n2));
+            T modes = T(0);
+#pragma unroll 1
+            for (int m = 0; m < 4; ++m) {   // kx = jp, -jp at ky of either sign
+              const int ms = P.pair_rows ? m >> 1 : sgn;
+              if ((m & 1) && jp == 0) continue;
+              if ((m >> 1) && (!P.pair_rows || tay == 0)) continue;
+              if (ms && tay == 0) continue;
+              const int i = (m & 1) ? -jp : jp, j = (m & 1) ? N - jp : jp;
+              const C* f = fsm + ((size_t)gr * nslot + (P.pair_rows ? ms : 0)) * P.nacc * N + j;
+              T mu = T(0);
+              if (P.global_los)
+                mu = (T(i) * T(P.los[0]) + T(ms ? -tay : tay) * T(P.los[1]) + fkz * T(P.los[2])) / kk;
+              modes += T(1);
+#pragma unroll
+              for (int e = 0; e < MAX_PRODS; ++e) {
+                if (e >= P.nprod) break;
+                const SumDesc sd = P.sum[e];
+                const C x = f[(size_t)sd.acc_x * N], y = f[(size_t)sd.acc_y * N];
+                // Re x y^*; with one odd l Im x y^* (Sec. 2.1, odd multipoles)
+                T p = wgt * (((sd.lx + sd.ly) & 1) ? (x.y * y.x - x.x * y.y) : (x.x * y.x + x.y * y.y));
+                if (P.global_los) p *= legendre_0to4<T>(sd.lx, mu) * legendre_0to4<T>(sd.ly, mu);
+                vals[e] += p;
+              }
+            }
+            modes *= wgt;
+            vals[MAX_SUMS - 2] = modes;
+            vals[MAX_SUMS - 1] = modes * (T(P.kf) * kk);
+          }
+          // warp-segmented inclusive scan over the runs of consecutive lanes with equal bin (bins rise
+          // with kx, so a bin has one run)
+          const int pb = __shfl_up_sync(0xffffffffu, bin, 1);
+          const bool head = (lane == 0) || (pb != bin);
+          const unsigned heads = __ballot_sync(0xffffffffu, head);
+          const int first = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));   // lane of the run's head
+          const bool last = (lane == 31) || ((heads >> (lane + 1)) & 1u);
+          // run sums over at most 32 lanes stay in T; only run ends convert to float64
+#pragma unroll
+          for (int e = 0; e < MAX_SUMS; ++e) {
+            if (e < MAX_PRODS && e >= P.nprod) continue;
+            T x = vals[e];
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+              const T y = __shfl_up_sync(0xffffffffu, x, off);
+              if (lane - off >= first) x += y;
+            }
+            if (last && bin >= 0) {
+              double* dst = mypart + (size_t)bin * P.nsum + (e < MAX_PRODS ? e : P.nprod + e - MAX_PRODS);
+              if (P.shared_part) *dst += (double)x;
+              else atomicAdd(dst, (double)x);
+            }
+          }
+          if (P.shared_part) __syncwarp();
+        }
+        if constexpr (Team::BLOCK) __syncthreads();
       }
-      if (P.ny > 0) {
-        const T fi = T(i), fj = T(jy), fk = T(kz);
-        const T r2 = fi * fi + fj * fj + fk * fk;
-        const T inv = r2 > T(0) ? rsqrt(r2) : T(0);
-        const T ux = fi * inv, uy = fj * inv, uz = r2 > T(0) ? fk * inv : T(1);
-        T re, im;
-        if (P.ymask & 2) {
-          ylm_ct<T, 1, 0>(ux, uy, uz, nrm, re, im); ytab[8 * N + kx] = cmk(re, im);
-          ylm_ct<T, 1, 1>(ux, uy, uz, nrm, re, im); ytab[9 * N + kx] = cmk(re, im);
-        }
-        if (P.ymask & 8) {
-          ylm_ct<T, 3, 0>(ux, uy, uz, nrm, re, im); ytab[10 * N + kx] = cmk(re, im);
-          ylm_ct<T, 3, 1>(ux, uy, uz, nrm, re, im); ytab[11 * N + kx] = cmk(re, im);
-          ylm_ct<T, 3, 2>(ux, uy, uz, nrm, re, im); ytab[12 * N + kx] = cmk(re, im);
-          ylm_ct<T, 3, 3>(ux, uy, uz, nrm, re, im); ytab[13 * N + kx] = cmk(re, im);
-        }
-        ylm_ct<T, 2, 0>(ux, uy, uz, nrm, re, im); ytab[0 * N + kx] = cmk(re, im);
-        ylm_ct<T, 2, 1>(ux, uy, uz, nrm, re, im); ytab[1 * N + kx] = cmk(re, im);
-        ylm_ct<T, 2, 2>(ux, uy, uz, nrm, re, im); ytab[2 * N + kx] = cmk(re, im);
-        if (P.ymask & 16) {
-          ylm_ct<T, 4, 0>(ux, uy, uz, nrm, re, im); ytab[3 * N + kx] = cmk(re, im);
-          ylm_ct<T, 4, 1>(ux, uy, uz, nrm, re, im); ytab[4 * N + kx] = cmk(re, im);
-          ylm_ct<T, 4, 2>(ux, uy, uz, nrm, re, im); ytab[5 * N + kx] = cmk(re, im);
-          ylm_ct<T, 4, 3>(ux, uy, uz, nrm, re, im); ytab[6 * N + kx] = cmk(re, im);
-          ylm_ct<T, 4, 4>(ux, uy, uz, nrm, re, im); ytab[7 * N + kx] = cmk(re, im);
-        }
-      }
-      for (int q = 0; q < G * P.nacc; ++q) facc[(size_t)q * N + kx] = cmk(T(0), T(0));
     }
-    __syncthreads();
-    C v[8], vn[8], racc[8];
-    int cur = -1;   // accumulator held in racc
-    const size_t fstride = (size_t)P.KZ * N * N;
-    const size_t roff = ((size_t)kz * N + ky) * N;
-    int f = ingroup ? P.slot[g] : -1;
-    if (f >= 0) {
-      const C* src = half + (size_t)f * fstride + roff;
+    else if (in_bins(next)) {   // nothing to do in this pass of the block: the next pass's first row
+      const C* src = row_of(next, 0) + (size_t)P.step[0].field * fstride;
 #pragma unroll
       for (int q = 0; q < 8; ++q) v[q] = src[t + q * TPF];
     }
-    for (int rd = 0; rd < P.nrounds; ++rd) {
-      const bool live = f >= 0;
-      const int fn = (ingroup && rd + 1 < P.nrounds) ? P.slot[(rd + 1) * G + g] : -1;
-      if (fn >= 0) {
-        const C* src = half + (size_t)fn * fstride + roff;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) vn[q] = src[t + q * TPF];
-      }
-      if (!live) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = cmk(T(0), T(0));
-      }
-      fft_block<N, -1>(v, t, tw, RowView<C>{rowbuf + (size_t)(ingroup ? g : G) * NP},
-                       RowSync<N, CONTRACT_THREADS>::make(g));
-      if (live) {
-        const FieldCoef c = P.fc[f];
-        if (c.acc != cur) {   // a group's fields come in accumulator order: flush once per change
-          if (cur >= 0) {
-            C* acc = facc + ((size_t)g * P.nacc + cur) * N;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) acc[t + q * TPF] = cadd(acc[t + q * TPF], racc[q]);
-          }
-          cur = c.acc;
-#pragma unroll
-          for (int q = 0; q < 8; ++q) racc[q] = cmk(T(0), T(0));
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int kx = t + q * TPF;
-          T w = coef_scale<T>(c);
-          if (c.yidx >= 0) {
-            const C y = ytab[(size_t)c.yidx * N + kx];
-            w *= (c.part == PART_RE ? y.x : y.y);
-          }
-          // phase-pure groups apply the window and interlacing factors once per mode, at binning
-          const C a = P.phase_pure ? cscale(v[q], w)
-                                   : (c.phase ? cmul(v[q], cscale(fb[kx], w)) : cscale(v[q], w * fa[kx]));
-          racc[q] = cadd(racc[q], a);
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = vn[q];
-      f = fn;
-    }
-    if (cur >= 0) {
-      C* acc = facc + ((size_t)g * P.nacc + cur) * N;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) acc[t + q * TPF] = cadd(acc[t + q * TPF], racc[q]);
-    }
+    item = next;
+    if constexpr (Team::BLOCK) ++pass;
+  }
+  if (P.shared_part) {   // the CTA's sums, warps in order
     __syncthreads();
-    const T fjy = T(jy), fkz = T(kz);
-    // modes kx = jp and kx = -jp (index N - jp) have the same |k|, hence the same bin: where a thread
-    // would bin two or more modes, it adds the mirror pair before the warp-segmented scan (one scan
-    // and one set of run-end atomics per pair); smaller rows keep one mode per thread
-    constexpr bool MIRROR = N >= 2 * CONTRACT_THREADS;
-    constexpr int NJ = MIRROR ? N / 2 : N;
-    for (int jb = warp * 32; jb < NJ; jb += blockDim.x) {
-      const int jp = jb + lane;
-      int bin = -1;
-      T vals[MAX_SUMS];
-#pragma unroll
-      for (int s = 0; s < MAX_SUMS; ++s) vals[s] = T(0);
-#pragma unroll 1
-      for (int mir = 0; mir < (MIRROR ? 2 : 1); ++mir) {
-        const int j = MIRROR ? (mir ? N - jp : jp) : jp;
-        const int i = MIRROR ? (mir ? -jp : jp) : (jp < N / 2 ? jp : jp - N);
-        const bool in_row = MIRROR ? (jp < N / 2 && (mir == 0 || jp > 0)) : (jp < N && i != -N / 2);
-        int mbin = -1;
-        if (in_row && jy != -N / 2 && (i != 0 || jy != 0 || kz != 0)) mbin = bintab[i * i + jy * jy + kz * kz];
-        if (mbin >= 0) {
-          bin = mbin;
-          const T wgt = kz > 0 ? T(2) : T(1);
-          // accumulators summed over the groups: phase a (even g, or all with one phase) and phase b
-          C Aa[6], Ab[6];
-#pragma unroll
-          for (int a = 0; a < 6; ++a) Aa[a] = Ab[a] = cmk(T(0), T(0));
-          auto gsum = [&](int g0, int gstep, C (&acc)[6]) {
-            for (int gg = g0; gg < G; gg += gstep) {
-              const C* fg = facc + (size_t)gg * P.nacc * N + j;
-#pragma unroll
-              for (int a = 0; a < 6; ++a)
-                if (a < P.nacc) acc[a] = cadd(acc[a], fg[(size_t)a * N]);
-            }
-          };
-          if (P.phase_pure) {
-            gsum(0, P.nphase == 2 ? 2 : 1, Aa);
-            const T faj = fa[j];
-#pragma unroll
-            for (int a = 0; a < 6; ++a) Aa[a] = cscale(Aa[a], faj);
-            if (P.nphase == 2) {
-              gsum(1, 2, Ab);
-              const C fbj = fb[j];
-#pragma unroll
-              for (int a = 0; a < 6; ++a) Aa[a] = cadd(Aa[a], cmul(Ab[a], fbj));
-            }
-          } else {
-            gsum(0, 1, Aa);
-          }
-          auto pick = [&](int k) {   // accumulator k (runtime index kept out of local memory)
-            C r = cmk(T(0), T(0));
-#pragma unroll
-            for (int a = 0; a < 6; ++a)
-              if (k == a) r = Aa[a];
-            return r;
-          };
-          const C F0 = Aa[0];
-          C F1, F2, F3, F4, FA;
-          if (P.even_layout) {   // accumulators F_0, F_2, F_4 (when present) at 0, 1, 2, then F_0^A
-            F1 = F3 = cmk(T(0), T(0));
-            F2 = Aa[1];
-            F4 = Aa[2];
-            FA = P.acc_a == 1 ? Aa[1] : (P.acc_a == 2 ? Aa[2] : Aa[3]);
-          } else {
-            F1 = pick(P.acc_of[1]);
-            F2 = pick(P.acc_of[2]);
-            F3 = pick(P.acc_of[3]);
-            F4 = pick(P.acc_of[4]);
-            FA = pick(P.acc_a);
-          }
-          const T fi = T(i);
-          const T kk = sqrt(fi * fi + fjy * fjy + fkz * fkz);
-          if (P.global_los) {
-            const T mu = (fi * T(P.los[0]) + fjy * T(P.los[1]) + fkz * T(P.los[2])) / kk;
-            if (P.need_mask & 2) F1 = cscale(F0, legendre_p<T>(1, mu));
-            if (P.need_mask & 4) F2 = cscale(F0, legendre_p<T>(2, mu));
-            if (P.need_mask & 8) F3 = cscale(F0, legendre_p<T>(3, mu));
-            if (P.need_mask & 16) F4 = cscale(F0, legendre_p<T>(4, mu));
-          }
-          auto sel = [&](int l) { return l == 0 ? F0 : (l == 1 ? F1 : (l == 2 ? F2 : (l == 3 ? F3 : F4))); };
-#pragma unroll
-          for (int s = 0; s < MAX_SUMS; ++s) {
-            T v = T(0);
-            if (s < P.nell) {
-              const int l = P.ell_list[s];
-              const C b = sel(l);
-              const C a = P.acc_a >= 0 ? FA : F0;   // cross: F_0 of tracer A against F_l of B
-              // even l: Re a b^*; odd l: Im a b^* (Sec. 2.1, odd multipoles)
-              v = wgt * ((l & 1) ? (a.y * b.x - a.x * b.y) : (a.x * b.x + a.y * b.y));
-            } else if (s < P.nell + P.nll) {
-              const C a = sel(P.lla[s - P.nell]), b = sel(P.llb[s - P.nell]);
-              v = wgt * (a.x * b.x + a.y * b.y);
-            } else if (s == P.nsum - 2) {
-              v = wgt;
-            } else if (s == P.nsum - 1) {
-              v = wgt * T(P.kf) * kk;
-            }
-            vals[s] += v;
-          }
-        }
-      }
-      // warp-segmented inclusive scan over runs of consecutive lanes with equal bin; a run is
-      // identified by the number of run heads up to this lane, so runs of the same bin that are
-      // not adjacent (a warp spanning both kx halves when n < 64) stay separate
-      const int pb = __shfl_up_sync(0xffffffffu, bin, 1);
-      const bool head = (lane == 0) || (pb != bin);
-      const unsigned heads = __ballot_sync(0xffffffffu, head);
-      const int seg = __popc(heads & (0xffffffffu >> (31 - lane)));
-      unsigned addm = 0;
-#pragma unroll
-      for (int st = 0; st < 5; ++st) {
-        const int off = 1 << st;
-        const int os = __shfl_up_sync(0xffffffffu, seg, off);
-        if (lane >= off && os == seg) addm |= 1u << st;
-      }
-      const bool last = (lane == 31) || ((heads >> (lane + 1)) & 1u);
-      // run sums over at most 32 modes stay in T; only run ends convert to float64
-#pragma unroll
-      for (int s = 0; s < MAX_SUMS; ++s) {
-        if (s >= P.nsum) break;
-        T x = vals[s];
-#pragma unroll
-        for (int st = 0; st < 5; ++st) {
-          const T yv = __shfl_up_sync(0xffffffffu, x, 1 << st);
-          if (addm & (1u << st)) x += yv;
-        }
-        if (last && bin >= 0) atomicAdd(mypart + (size_t)bin * P.nsum + s, (double)x);
-      }
+    for (int i = tid; i < nent; i += blockDim.x) {
+      double x = 0.0;
+      for (int w = 0; w < nw; ++w) x += spart[(size_t)w * nent + i];
+      part[(size_t)blockIdx.x * nent + i] = x;
     }
-    __syncthreads();
   }
 }
 
@@ -842,7 +866,7 @@ struct FinalParams {
   int req_mask;          // requested P_l (bits)
 };
 
-constexpr int FIN_THREADS = 128;
+constexpr int FIN_THREADS = 256;
 
 // one block per bin: the partials are summed with a fixed per-thread stride and a fixed tree
 __global__ void __launch_bounds__(FIN_THREADS)
@@ -853,8 +877,11 @@ k_power_finalize(const double* __restrict__ part, const FinalParams F, const dou
   for (int b = blockIdx.x; b < nb; b += gridDim.x) {
     double S[MAX_SUMS];
     for (int s = 0; s < MAX_SUMS; ++s) S[s] = 0.0;
-    for (int p = threadIdx.x; p < F.nparts; p += FIN_THREADS)
-      for (int s = 0; s < F.nsum; ++s) S[s] += part[((size_t)p * nb + b) * F.nsum + s];
+    for (int p = threadIdx.x; p < F.nparts; p += FIN_THREADS) {
+#pragma unroll
+      for (int s = 0; s < MAX_SUMS; ++s)
+        if (s < F.nsum) S[s] += part[((size_t)p * nb + b) * F.nsum + s];
+    }
     for (int s = 0; s < MAX_SUMS; ++s) red[s][threadIdx.x] = S[s];
     __syncthreads();
     for (int off = FIN_THREADS / 2; off > 0; off >>= 1) {
@@ -1042,99 +1069,72 @@ npc_status contract_impl(npc_ctx* ctx, const PowerPlan& plan, const npc_mesh_spe
   const int16_t* bintab;
   NPC_TRY(get_bin_table(ctx, N, m.box, kb, &bintab));
   ContractParams P{};
-  P.nf = plan.fl.nf;
   P.nphase = plan.nphase;
-  P.ny = 0;
   int req_internal = plan.ells_mask;
   if (plan.mod_mask) req_internal |= 1 | 4 | 16;
-  P.need2 = (req_internal & 4) ? 1 : 0;
-  P.need4 = (req_internal & 16) ? 1 : 0;
-  P.need_mask = req_internal | 1;
   // accumulators: one per multipole with fields of tracer B (in l order), then F_0^A
-  for (int l = 0; l <= 4; ++l) P.acc_of[l] = -1;
-  P.nacc_b = 0;
+  int acc_of[5] = {-1, -1, -1, -1, -1};
+  int nacc_b = 0;
   if (plan.global_los) {
-    P.acc_of[0] = 0;
-    P.nacc_b = 1;
+    acc_of[0] = 0;
+    nacc_b = 1;
   } else {
     for (int l = 0; l <= 4; ++l) {
       bool has = false;
       for (int f = 0; f < plan.fl.nf; ++f) has |= !plan.fl.f[f].tracer && plan.fl.f[f].ell == l;
-      if (has) P.acc_of[l] = P.nacc_b++;
+      if (has) acc_of[l] = nacc_b++;
     }
   }
-  P.acc_a = plan.cross ? P.nacc_b : -1;
-  P.nacc = P.nacc_b + (plan.cross ? 1 : 0);
+  const int acc_a = plan.cross ? nacc_b : -1;
+  P.nacc = nacc_b + (plan.cross ? 1 : 0);
   if (P.nacc > 6) return set_err(ctx, NPC_ERR_UNSUPPORTED, "x pass: at most 6 accumulators");
-  P.even_layout = (P.acc_of[1] < 0 && P.acc_of[3] < 0 && (P.acc_of[2] == 1 || P.acc_of[2] < 0) &&
-                   (P.acc_of[4] == 2 || P.acc_of[4] < 0) && (P.acc_a < 0 || P.acc_a <= 3)) ? 1 : 0;
   if (plan.cross && plan.mod_mask)
     return set_err(ctx, NPC_ERR_UNSUPPORTED, "cross spectra: no modified multipoles");
-  P.ymask = 0;
+  const YNorm nrm = ylm_norm_table();
   for (int f = 0; f < plan.fl.nf; ++f) {
     const Comp c = plan.fl.f[f];
-    FieldCoef fc;
-    fc.acc = (int8_t)(c.tracer ? P.acc_a : (plan.global_los ? 0 : P.acc_of[c.ell]));
     if (c.tracer && (!plan.cross || c.part != PART_ONE))
       return set_err(ctx, NPC_ERR_INVALID_ARG, "x pass: tracer-A field must be an unweighted F_0");
-    fc.phase = c.phase;
-    fc.part = c.part;
-    fc.yidx = -1;
-    fc.scale_d = 1.0;
-    fc.scale_f = 1.0f;
-    if (c.part == PART_RE || c.part == PART_IM) {
-      if (c.ell < 1 || c.ell > 4 || c.m < 0 || c.m > c.ell)
-        return set_err(ctx, NPC_ERR_UNSUPPORTED, "Y_%d%d field in the x pass", c.ell, c.m);
-      fc.yidx = (int8_t)ytab_index(c.ell, c.m);
-      P.ymask |= 1 << c.ell;
-      P.ny = std::max(P.ny, (P.ymask & 10) ? 14 : ((P.ymask & 16) ? 8 : 3));
-      fc.scale_d = 4.0 * M_PI / (2 * c.ell + 1) * (c.m > 0 ? 2.0 : 1.0);
-      fc.scale_f = (float)fc.scale_d;
-    }
-    P.fc[f] = fc;
+    if (c.phase && P.nphase == 1) return set_err(ctx, NPC_ERR_INVALID_ARG, "phase-b field without interlacing");
+    if ((c.part == PART_RE || c.part == PART_IM) && (c.ell < 1 || c.ell > 4 || c.m < 0 || c.m > c.ell))
+      return set_err(ctx, NPC_ERR_UNSUPPORTED, "Y_%d%d field in the x pass", c.ell, c.m);
   }
-  {
-    // field slots: with two phases and an even number of row groups, even groups take the
-    // phase-a fields and odd groups the phase-b fields (in list order), so that a group's
-    // accumulators hold one phase and the window/interlacing factors are applied per mode
-    constexpr int G = XCfg<N>::G;
-    std::vector<int> ph[2];
-    for (int f = 0; f < plan.fl.nf; ++f) ph[plan.fl.f[f].phase ? 1 : 0].push_back(f);
-    P.phase_pure = (P.nphase == 1 || G % 2 == 0) ? 1 : 0;
-    if (P.nphase == 1 && !ph[1].empty()) return set_err(ctx, NPC_ERR_INVALID_ARG, "phase-b field without interlacing");
-    int nrounds;
-    if (P.phase_pure && P.nphase == 2) {
-      const int per = G / 2;
-      nrounds = (int)std::max((ph[0].size() + per - 1) / per, (ph[1].size() + per - 1) / per);
-    } else {
-      nrounds = (plan.fl.nf + G - 1) / G;
-    }
-    if ((size_t)nrounds * G > (size_t)MAX_SLOTS)
-      return set_err(ctx, NPC_ERR_UNSUPPORTED, "x pass: %d fields do not fit %d slots", plan.fl.nf, MAX_SLOTS);
-    P.nrounds = nrounds;
-    for (int r = 0; r < nrounds; ++r)
-      for (int g = 0; g < G; ++g) {
-        int f = -1;
-        if (P.phase_pure && P.nphase == 2) {
-          const size_t i = (size_t)r * (G / 2) + g / 2;
-          const std::vector<int>& l = ph[g & 1];
-          if (i < l.size()) f = l[i];
-        } else {
-          const int i = r * G + g;
-          if (i < plan.fl.nf) f = i;
+  // steps by accumulator, phase b first: its sum is rotated by the interlacing phase once
+  for (int acc = 0; acc < P.nacc; ++acc) {
+    for (int ph = P.nphase - 1; ph >= 0; --ph) {
+      for (int f = 0; f < plan.fl.nf; ++f) {
+        const Comp c = plan.fl.f[f];
+        if ((c.phase ? 1 : 0) != ph || (c.tracer ? acc_a : (plan.global_los ? 0 : acc_of[c.ell])) != acc) continue;
+        FieldStep& st = P.step[P.nsteps++];
+        st.field = (int8_t)f;
+        st.acc = (int8_t)acc;
+        st.scale_d = 1.0;
+        if (c.part == PART_RE || c.part == PART_IM) {
+          const int lm = c.ell * (c.ell + 1) / 2 + c.m;
+          st.weight = (int8_t)(2 * lm + (c.part == PART_IM ? 1 : 0));
+          st.scale_d = 4.0 * M_PI / (2 * c.ell + 1) * (c.m > 0 ? 2.0 : 1.0) * nrm.v[lm];
         }
-        P.slot[r * G + g] = (int8_t)f;
+        st.scale_f = (float)st.scale_d;
       }
+      if (ph == 1) P.step[P.nsteps - 1].flags |= STEP_ROTATE;
+    }
+    P.step[P.nsteps - 1].flags |= STEP_STORE;
   }
   P.nbins = kb.nbins;
-  P.nell = 0;
+  FinalParams F{};
   for (int l = 0; l <= 4; ++l)
-    if (req_internal & (1 << l)) P.ell_list[P.nell++] = l;
-  P.nll = 0;
-  if (plan.mod_mask & ((1 << 4) | (1 << 16))) { P.lla[P.nll] = 2; P.llb[P.nll] = 2; P.nll++; }
-  if (plan.mod_mask & ((1 << 6) | (1 << 8) | (1 << 17))) { P.lla[P.nll] = 4; P.llb[P.nll] = 2; P.nll++; }
-  if (plan.mod_mask & ((1 << 8) | (1 << 18))) { P.lla[P.nll] = 4; P.llb[P.nll] = 4; P.nll++; }
-  P.nsum = P.nell + P.nll + 2;
+    if (req_internal & (1 << l)) F.ell_list[F.nell++] = l;
+  auto add_ll = [&](int a, int b) { F.lla[F.nll] = a; F.llb[F.nll++] = b; };
+  if (plan.mod_mask & ((1 << 4) | (1 << 16))) add_ll(2, 2);
+  if (plan.mod_mask & ((1 << 6) | (1 << 8) | (1 << 17))) add_ll(4, 2);
+  if (plan.mod_mask & ((1 << 8) | (1 << 18))) add_ll(4, 4);
+  auto add_sum = [&](int lx, int ly, int acc_x) {
+    P.sum[P.nprod++] = SumDesc{(int8_t)lx, (int8_t)ly, (int8_t)acc_x, (int8_t)(plan.global_los ? 0 : acc_of[ly])};
+  };
+  // cross spectra take F_0 of tracer A against F_l of B
+  for (int e = 0; e < F.nell; ++e) add_sum(0, F.ell_list[e], plan.cross ? acc_a : 0);
+  for (int e = 0; e < F.nll; ++e) add_sum(F.lla[e], F.llb[e], plan.global_los ? 0 : acc_of[F.lla[e]]);
+  P.nsum = P.nprod + 2;
   P.KZ = plan.kz_keep > 0 ? std::min(plan.kz_keep, N / 2) : N / 2;
   P.global_los = plan.global_los;
   for (int a = 0; a < 3; ++a) P.los[a] = plan.los[a];
@@ -1147,37 +1147,47 @@ npc_status contract_impl(npc_ctx* ctx, const PowerPlan& plan, const npc_mesh_spe
     P.row_n2max = r2 >= 3.0 * (N / 2) * (N / 2) ? 3 * (N / 2) * (N / 2) : (int)std::floor(r2) + 1;
   }
 
-  constexpr int NP = row_pad_len<N>();
-  constexpr int G = XCfg<N>::G;
-  const size_t smem = sizeof(C) * ((size_t)N + (size_t)P.ny * N + (size_t)G * P.nacc * N +
-                                   (size_t)XCfg<N>::NBUF * NP + N) +
-                      sizeof(T) * (N / 2 + 2 + N);
-  auto kern = k_fft_x_contract<T, N>;
+  // shared memory of a CTA: tables, two exchange buffers per row, the finished F_l of one row (or of
+  // rows ky and -ky), the warps' partial sums where they are small
+  auto smem_of = [&](int threads) {
+    const int G = threads / XTeam<N>::TPF;
+    const int nbuf = G + (XTeam<N>::BLOCK && threads % XTeam<N>::TPF ? 1 : 0);
+    size_t b = sizeof(C) * ((size_t)3 * N + (size_t)nbuf * XTeam<N>::ROW +
+                            (size_t)G * (P.pair_rows ? 2 : 1) * P.nacc * N) + sizeof(T) * (N / 2 + 2);
+    b = (b + 15) & ~(size_t)15;
+    if (P.shared_part) b += sizeof(double) * (threads / 32) * P.nbins * P.nsum;
+    return b;
+  };
+  P.pair_rows = P.nacc == 1 ? 1 : 0;
+  P.shared_part = N <= 256 && sizeof(double) * (CONTRACT_THREADS / 32) * P.nbins * P.nsum <= 32768 ? 1 : 0;
+  // fewer threads per CTA where the rows would not fill the SMs four times over (a CTA of 256 threads
+  // holds 32 rows at n = 64), or where the shared memory asks for it (FP64 at 256^3 with odd multipoles)
+  const int nitems = P.KZ * (N / 2);
+  int threads = XTeam<N>::THREADS;
+  while (!XTeam<N>::BLOCK && threads > std::max(32, XTeam<N>::TPF) &&
+         (smem_of(threads) > 227 * 1024 || nitems < 4 * ctx->num_sms * (threads / XTeam<N>::TPF)))
+    threads /= 2;
+  const size_t smem = smem_of(threads);
+  auto kern = k_fft_x_contract<T, N, (sizeof(T) == 4 ? 2 : 1)>;
   NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
-  NPC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, CONTRACT_THREADS, smem));
+  NPC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
   if (per_sm < 1) return set_err(ctx, NPC_ERR_UNSUPPORTED, "contraction does not fit on an SM (%zu B smem)", smem);
-  const int nrows = P.KZ * N;
-  const int grid = std::min(nrows, per_sm * ctx->num_sms);
-  const int nw = CONTRACT_THREADS / 32;
-  const size_t nparts = (size_t)grid * nw;
+  const int G = threads / XTeam<N>::TPF;
+  const int grid = std::min((nitems + G - 1) / G, per_sm * ctx->num_sms);
+  const size_t nparts = (size_t)grid * (P.shared_part ? 1 : threads / 32);
   double* part;
   NPC_TRY(ws_get(ctx, "power.part", sizeof(double) * nparts * P.nbins * P.nsum, (void**)&part));
-  NPC_CUDA(ctx, cudaMemsetAsync(part, 0, sizeof(double) * nparts * P.nbins * P.nsum, ctx->stream));
+  if (!P.shared_part)
+    NPC_CUDA(ctx, cudaMemsetAsync(part, 0, sizeof(double) * nparts * P.nbins * P.nsum, ctx->stream));
   NPC_TRY(stage_mark(ctx, "contract_setup"));
-  kern<<<grid, CONTRACT_THREADS, smem, ctx->stream>>>((const C*)half, P, ylm_norm_table(), bintab, (const C*)twp,
-                                                      part);
+  kern<<<grid, threads, smem, ctx->stream>>>((const C*)half, P, bintab, (const C*)twp, part);
   NPC_LAUNCH(ctx);
   NPC_TRY(stage_mark(ctx, "fft_x_contract"));
 
-  FinalParams F{};
   F.nbins = P.nbins;
   F.nsum = P.nsum;
   F.nparts = (int)nparts;
-  F.nell = P.nell;
-  for (int e = 0; e < P.nell; ++e) F.ell_list[e] = P.ell_list[e];
-  F.nll = P.nll;
-  for (int e = 0; e < P.nll; ++e) { F.lla[e] = P.lla[e]; F.llb[e] = P.llb[e]; }
   F.nmod = 0;
   for (int lb = 4; lb <= 8; lb += 2)
     if (plan.mod_mask & (1 << lb)) F.mod_list[F.nmod++] = lb;
