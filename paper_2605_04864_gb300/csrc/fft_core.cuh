@@ -20,40 +20,51 @@ __device__ __forceinline__ C twiddle(const C* __restrict__ tw, int j) {
   return w;
 }
 
-template <typename C>
-__device__ __forceinline__ void bfly2(C& a, C& b) {
-  const C t = a;
-  a = cadd(t, b);
-  b = csub(t, b);
+// PACKED: sums as packed float pairs (fewer issues; for kernels with registers to spare, since the pairs
+// constrain their placement: the column passes that run at 40 registers measured 7 to 30 % slower).
+template <bool PACKED, typename C> __device__ __forceinline__ C bf_add(C a, C b) {
+  if constexpr (PACKED) return cadd_packed(a, b);
+  else return cadd(a, b);
+}
+template <bool PACKED, typename C> __device__ __forceinline__ C bf_sub(C a, C b) {
+  if constexpr (PACKED) return csub_packed(a, b);
+  else return csub(a, b);
 }
 
-// length-4 DFT in natural order on (a0, a1, a2, a3)
-template <int DIR, typename C>
+template <bool PACKED, typename C>
+__device__ __forceinline__ void bfly2(C& a, C& b) {
+  const C t = a;
+  a = bf_add<PACKED>(t, b);
+  b = bf_sub<PACKED>(t, b);
+}
+
+// length-4 DFT in natural order on (a0, a1, a2, a3); the difference that is turned by i is written turned
+template <int DIR, bool PACKED, typename C>
 __device__ __forceinline__ void dft4(C& a0, C& a1, C& a2, C& a3) {
-  const C b0 = cadd(a0, a2), b2 = csub(a0, a2);
-  const C b1 = cadd(a1, a3), b3 = cmul_i<DIR>(csub(a1, a3));
-  a0 = cadd(b0, b1);
-  a2 = csub(b0, b1);
-  a1 = cadd(b2, b3);
-  a3 = csub(b2, b3);
+  const C b0 = bf_add<PACKED>(a0, a2), b2 = bf_sub<PACKED>(a0, a2);
+  const C b1 = bf_add<PACKED>(a1, a3), b3 = csub_i<DIR>(a1, a3);
+  a0 = bf_add<PACKED>(b0, b1);
+  a2 = bf_sub<PACKED>(b0, b1);
+  a1 = bf_add<PACKED>(b2, b3);
+  a3 = bf_sub<PACKED>(b2, b3);
 }
 
 // length-8 DFT in natural order on v[0..7] (decimation in frequency into two length-4 DFTs)
-template <int DIR, typename C>
+template <int DIR, bool PACKED, typename C>
 __device__ __forceinline__ void dft8(C (&v)[8]) {
   using T = decltype(v[0].x);
   const T r = T(0.70710678118654752440);
-  C a0 = cadd(v[0], v[4]), a1 = cadd(v[1], v[5]), a2 = cadd(v[2], v[6]), a3 = cadd(v[3], v[7]);
-  C c0 = csub(v[0], v[4]);
-  C c1 = csub(v[1], v[5]);
-  C c2 = csub(v[2], v[6]);
-  C c3 = csub(v[3], v[7]);
-  // c1 *= w, c2 *= w^2 = DIR*i, c3 *= w^3 with w = exp(DIR*i*pi/4)
+  C a0 = bf_add<PACKED>(v[0], v[4]), a1 = bf_add<PACKED>(v[1], v[5]), a2 = bf_add<PACKED>(v[2], v[6]),
+    a3 = bf_add<PACKED>(v[3], v[7]);
+  C c0 = bf_sub<PACKED>(v[0], v[4]);
+  C c1 = bf_sub<PACKED>(v[1], v[5]);
+  C c2 = csub_i<DIR>(v[2], v[6]);   // times w^2 = DIR*i
+  C c3 = bf_sub<PACKED>(v[3], v[7]);
+  // c1 *= w, c3 *= w^3 with w = exp(DIR*i*pi/4)
   c1 = cmul(c1, cmk(r, T(DIR) * r));
-  c2 = cmul_i<DIR>(c2);
   c3 = cmul(c3, cmk(-r, T(DIR) * r));
-  dft4<DIR>(a0, a1, a2, a3);
-  dft4<DIR>(c0, c1, c2, c3);
+  dft4<DIR, PACKED>(a0, a1, a2, a3);
+  dft4<DIR, PACKED>(c0, c1, c2, c3);
   v[0] = a0; v[2] = a1; v[4] = a2; v[6] = a3;
   v[1] = c0; v[3] = c1; v[5] = c2; v[7] = c3;
 }
@@ -62,6 +73,7 @@ __device__ __forceinline__ void dft8(C (&v)[8]) {
 // from `off` on (off a multiple of 8), used by the sub-transforms of a composite length.  The exchange
 // after the stage with span Ns writes and reads through put<Ns> / get<Ns>.
 template <typename C> struct ColView {  // element n of column at p[n*stride]
+  static constexpr bool PACKED = false;
   C* p;
   int stride;
   __device__ __forceinline__ void st(int n, C v) const { p[n * stride] = v; }
@@ -75,6 +87,7 @@ template <typename C> struct ColView {  // element n of column at p[n*stride]
 // per 16), after span 8 it writes 64 (b div 8) + (b mod 8) + 8 r (eight slots per 64), later spans write
 // runs of 64; all read runs t, t + 1, ...  (With one slot per 8 throughout every read took two passes.)
 template <typename C> struct RowView {
+  static constexpr bool PACKED = true;
   C* p;
   __device__ __forceinline__ static int idx(int n) { return n + (n >> 3); }
   template <int Ns> __device__ __forceinline__ static int pos(int n) {
@@ -133,7 +146,7 @@ __host__ __device__ constexpr int twiddle_offset(int n, int span) {
 
 // Butterflies of the stage with span Ns on the thread's elements.  TS: stride into the natural twiddle
 // table (a length-N/TS sub-transform reads every TS-th twiddle of N); 1: the stage-by-stage table.
-template <int N, int DIR, int Ns, int TS, typename C>
+template <int N, int DIR, int Ns, int TS, bool PACKED, typename C>
 __device__ __forceinline__ void fft_butterflies(C (&v)[8], const int t, const C* __restrict__ tw) {
   constexpr int TPF = N / 8;
   constexpr int REM = N / Ns;
@@ -152,11 +165,11 @@ __device__ __forceinline__ void fft_butterflies(C (&v)[8], const int t, const C*
       }
     }
     if constexpr (R == 8) {
-      dft8<DIR>(v);
+      dft8<DIR, PACKED>(v);
     } else if constexpr (R == 4) {
-      dft4<DIR>(v[s], v[s + BPT], v[s + 2 * BPT], v[s + 3 * BPT]);
+      dft4<DIR, PACKED>(v[s], v[s + BPT], v[s + 2 * BPT], v[s + 3 * BPT]);
     } else {
-      bfly2(v[s], v[s + BPT]);
+      bfly2<PACKED>(v[s], v[s + BPT]);
     }
   }
 }
@@ -169,7 +182,7 @@ __device__ __forceinline__ void fft_stages(C (&v)[8], const int t, const C* __re
   constexpr int REM = N / Ns;
   constexpr int R = (REM >= 8) ? 8 : REM;
   constexpr int BPT = 8 / R;
-  fft_butterflies<N, DIR, Ns, TS>(v, t, tw);
+  fft_butterflies<N, DIR, Ns, TS, View::PACKED>(v, t, tw);
   if constexpr (Ns * R < N) {
 #pragma unroll
     for (int s = 0; s < BPT; ++s) {
@@ -200,7 +213,7 @@ __device__ __forceinline__ void fft_block_alternate(C (&v)[8], const int t, cons
   constexpr int REM = N / Ns;
   constexpr int R = (REM >= 8) ? 8 : REM;
   constexpr int BPT = 8 / R;
-  fft_butterflies<N, DIR, Ns, 1>(v, t, tw);
+  fft_butterflies<N, DIR, Ns, 1, View::PACKED>(v, t, tw);
   if constexpr (Ns * R < N) {
 #pragma unroll
     for (int s = 0; s < BPT; ++s) {
@@ -249,8 +262,8 @@ __device__ __forceinline__ void fft_block(C (&v)[8], const int t, const C* __res
       const int km = k % M;
       const int k2 = (2 * k) % N;
       C a = buf.ld(km);
-      a = cadd(a, cmul(buf.ld(M + km), twiddle<C, DIR>(tw, k)));
-      a = cadd(a, cmul(buf.ld(2 * M + km), twiddle<C, DIR>(tw, k2)));
+      a = cadd(a, cmul(buf.sub(M).ld(km), twiddle<C, DIR>(tw, k)));
+      a = cadd(a, cmul(buf.sub(2 * M).ld(km), twiddle<C, DIR>(tw, k2)));
       v[q] = a;
     }
     sync();

@@ -30,6 +30,26 @@ template <typename C> __host__ __device__ __forceinline__ C cconj(C a) { return 
 template <typename C, typename T> __host__ __device__ __forceinline__ C cscale(C a, T s) {
   return cmk(a.x * s, a.y * s);
 }
+// The same sums as one packed instruction (float): both halves round as the scalar add does, and one
+// issue slot serves both.  For operands that are not products (those are left to fuse).
+__device__ __forceinline__ float2 cadd_packed(float2 a, float2 b) {
+  float2 r;
+  asm("{.reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 z, x, y;\n mov.b64 {%0, %1}, z;}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 csub_packed(float2 a, float2 b) {
+  float2 r;
+  asm("{.reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n sub.rn.f32x2 z, x, y;\n mov.b64 {%0, %1}, z;}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ double2 cadd_packed(double2 a, double2 b) { return cadd(a, b); }
+__device__ __forceinline__ double2 csub_packed(double2 a, double2 b) { return csub(a, b); }
+// (a - b) times (sign * i), the factor taken by the order of the operands
+template <int SIGN, typename C> __device__ __forceinline__ C csub_i(C a, C b) {
+  return SIGN < 0 ? cmk(a.y - b.y, b.x - a.x) : cmk(b.y - a.y, a.x - b.x);
+}
 // multiply by (sign * i): sign = -1 gives -i, +1 gives +i
 template <int SIGN, typename C> __host__ __device__ __forceinline__ C cmul_i(C a) {
   return SIGN < 0 ? cmk(a.y, -a.x) : cmk(-a.y, a.x);

@@ -38,94 +38,6 @@ template <int N> struct ColCfg {
   static constexpr int THREADS = TX * N / 8;
 };
 
-// Weight of one real field at grid point (x, y, z): F times ReY/ImY of the direction from the
-// observer to the grid point (phase b sits half a cell lower), or F alone (PART_ONE).
-template <typename T>
-struct ColGeom {
-  T px[2], py[2], oz[2], h;   // per phase: x and y coordinates of this column, z origin
-};
-
-template <typename T>
-__device__ __forceinline__ T comp_value(const Comp cp, const T* tileA, const T* tileB, int z, int c, int tx,
-                                        const ColGeom<T>& cg, const YNorm& nrm) {
-  if (cp.part == PART_ZERO) return T(0);
-  const T F = (cp.phase ? tileB : tileA)[z * tx + c];
-  if (cp.part == PART_ONE) return F;
-  const int ph = cp.phase;
-  const T pz = cg.oz[ph] + T(z) * cg.h;
-  const T r2 = cg.px[ph] * cg.px[ph] + cg.py[ph] * cg.py[ph] + pz * pz;
-  const T inv = r2 > T(0) ? rsqrt(r2) : T(0);
-  T re, im;
-  ylm_fast<T>(cp.ell, cp.m, cg.px[ph] * inv, cg.py[ph] * inv, pz * inv, nrm, re, im);
-  return F * (cp.part == PART_RE ? re : im);
-}
-
-// First pass: weighted real fields -> half spectra along z.  Output layout half[f][kz][y][x].
-template <typename T, int N>
-__global__ void __launch_bounds__(ColCfg<N>::THREADS)
-k_fwd_z(const T* __restrict__ mesh_a, const T* __restrict__ mesh_b, cplx<T>* __restrict__ half,
-        const FieldList fl, const Geom g, const YNorm nrm, const cplx<T>* __restrict__ tw_g, int KZ) {
-  using C = cplx<T>;
-  constexpr int TX = ColCfg<N>::TX;
-  constexpr int TPF = N / 8;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* tw = reinterpret_cast<C*>(smem_raw);
-  C* work = tw + N;
-  T* tileA = reinterpret_cast<T*>(work + N * TX);
-  T* tileB = tileA + N * TX;
-  const int tid = threadIdx.x;
-  const int c = tid % TX, t = tid / TX;
-  const int x0 = blockIdx.x * TX, y = blockIdx.y;
-  for (int i = tid; i < N; i += blockDim.x) tw[i] = tw_g[i];
-  for (int i = tid; i < N * TX; i += blockDim.x) {
-    const int z = i / TX, cc = i % TX;
-    const size_t gi = ((size_t)z * N + y) * N + x0 + cc;
-    tileA[i] = mesh_a[gi];
-    if (mesh_b) tileB[i] = mesh_b[gi];
-  }
-  ColGeom<T> cg;
-  cg.h = (T)g.h;
-  for (int ph = 0; ph < 2; ++ph) {
-    const double sh = ph ? 0.5 : 0.0;
-    cg.px[ph] = (T)(g.o[0] + ((double)(x0 + c) - sh) * g.h);
-    cg.py[ph] = (T)(g.o[1] + ((double)y - sh) * g.h);
-    cg.oz[ph] = (T)(g.o[2] - sh * g.h);
-  }
-  __syncthreads();
-  const int npairs = (fl.nf + 1) / 2;
-  const size_t fstride = (size_t)KZ * N * N;
-  for (int p = 0; p < npairs; ++p) {
-    const Comp c0 = fl.f[2 * p];
-    Comp c1;
-    c1.phase = 0; c1.ell = 0; c1.m = 0; c1.part = PART_ZERO;
-    if (2 * p + 1 < fl.nf) c1 = fl.f[2 * p + 1];
-    C v[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int z = t + q * TPF;
-      const T re = comp_value<T>(c0, tileA, tileB, z, c, TX, cg, nrm);
-      const T im = comp_value<T>(c1, tileA, tileB, z, c, TX, cg, nrm);
-      v[q] = cmk(re, im);
-    }
-    fft_block<N, -1>(v, t, tw, ColView<C>{work + c, TX});
-#pragma unroll
-    for (int q = 0; q < 8; ++q) work[(t + q * TPF) * TX + c] = v[q];
-    __syncthreads();
-    for (int i = tid; i < KZ * TX; i += blockDim.x) {
-      const int kz = i / TX, cc = i % TX;
-      const C z1 = work[kz * TX + cc];
-      const C z2 = cconj(work[((N - kz) % N) * TX + cc]);
-      const C a = cscale(cadd(z1, z2), T(0.5));
-      const C d = csub(z1, z2);
-      const C b = cmk(T(0.5) * d.y, T(-0.5) * d.x);
-      const size_t gi = ((size_t)kz * N + y) * N + x0 + cc;
-      half[(size_t)(2 * p) * fstride + gi] = a;
-      if (2 * p + 1 < fl.nf) half[(size_t)(2 * p + 1) * fstride + gi] = b;
-    }
-    __syncthreads();
-  }
-}
-
 // First pass for a single unweighted real field (global line of sight without interlacing, mesh
 // gradients): two neighbouring x columns share one complex transform, c = F(x) + i F(x+1), and
 // their half spectra follow from c(kz) and conj c(N - kz).  grid = (N / (2 TX), N).
@@ -173,13 +85,6 @@ k_fwd_z_single(const T* __restrict__ mesh, cplx<T>* __restrict__ half, const cpl
   }
 }
 
-// ---------------------------------------------------------------------------------------------
-// Specialised first pass for the standard interlaced field layout (l in {0, 2, 4}, both phases):
-// pair p is (l, m, kind) known at compile time; kind 0 packs the m = 0 field of phase a (real
-// part) with that of phase b (imaginary part), kind 1/2 is the complex field F Y_l^m of phase
-// a/b whose real and imaginary parts share one Y evaluation.  Pairs are a prefix of
-//   (0,0,0) (2,0,0) (2,1,1) (2,1,2) (2,2,1) (2,2,2) (4,0,0) (4,1,1) (4,1,2) ... (4,4,1) (4,4,2).
-// ---------------------------------------------------------------------------------------------
 // Polynomial factor Q_lm(uz) of Y_lm = norm_lm Q_lm(uz) (ux + i uy)^m, l <= 4: the associated
 // Legendre function with its (-1)^m phase, divided by sin^m(theta).
 template <typename T, int L, int M>
@@ -202,144 +107,125 @@ __device__ __forceinline__ T ylm_q(T uz) {
   else return T(105);
 }
 
-template <typename T, int L, int M>
-__device__ __forceinline__ void ylm_ct(T ux, T uy, T uz, const YNorm& nrm, T& re, T& im) {
-  const T q = ylm_q<T, L, M>(uz);
-  T pr = T(1), pi = T(0);
-#pragma unroll
-  for (int j = 0; j < M; ++j) {
-    const T nr = pr * ux - pi * uy;
-    pi = pr * uy + pi * ux;
-    pr = nr;
-  }
-  const T c = ynorm<T>(nrm, L * (L + 1) / 2 + M) * q;
-  re = c * pr;
-  im = c * pi;
-}
-
-template <typename T> struct ZGeom {
-  T px[2], py[2], pxy2[2];  // column x, row y per phase and px^2 + py^2
-  T pz0[2];                 // z coordinate of element q = 0 of this thread, per phase
-  T dz;                     // z step between consecutive elements of a thread (TPF cells)
-};
-
 // Keeps a value where it is computed: the per-pair factors below must not be hoisted out of the
-// pair loop (all fifteen pairs' factors would then stay live in registers).
+// pair loop (every pair's factors would then stay live in registers).
 __device__ __forceinline__ void keep_here(float& x) { asm volatile("" : "+f"(x)); }
 __device__ __forceinline__ void keep_here(double& x) { asm volatile("" : "+d"(x)); }
 
-template <typename T, int N, int TX, int L, int M, int KIND>
-__device__ __forceinline__ void std_inputs(cplx<T> (&v)[8], const T* tileA, const T* tileB, int c, int t,
-                                           const ZGeom<T>& zg, const YNorm& nrm) {
-  constexpr int TPF = N / 8;
-  if constexpr (KIND == 0) {
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int z = t + q * TPF;
-      const T fa = tileA[z * TX + c], fb = tileB[z * TX + c];
-      if constexpr (L == 0) {
-        v[q] = cmk(fa, fb);
-      } else {
-        T ya, yb, dum;
-        {
-          const T pz = zg.pz0[0] + T(q) * zg.dz;
-          const T inv = rsqrt(zg.pxy2[0] + pz * pz);
-          ylm_ct<T, L, M>(zg.px[0] * inv, zg.py[0] * inv, pz * inv, nrm, ya, dum);
-        }
-        {
-          const T pz = zg.pz0[1] + T(q) * zg.dz;
-          const T inv = rsqrt(zg.pxy2[1] + pz * pz);
-          ylm_ct<T, L, M>(zg.px[1] * inv, zg.py[1] * inv, pz * inv, nrm, yb, dum);
-        }
-        v[q] = cmk(fa * ya, fb * yb);
-      }
-    }
-  } else {
-    // Y_lm(xhat) = norm Q(uz) (px + i py)^m / r^m: the column factor norm (px + i py)^m is formed
-    // once per pair, each element needs 1/r, uz and the power r^-m
-    constexpr int ph = KIND - 1;
-    T cr = ynorm<T>(nrm, L * (L + 1) / 2 + M), ci = T(0);
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-      const T nr = cr * zg.px[ph] - ci * zg.py[ph];
-      ci = cr * zg.py[ph] + ci * zg.px[ph];
-      cr = nr;
-    }
-    keep_here(cr);
-    keep_here(ci);
-    const T* tile = ph ? tileB : tileA;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int z = t + q * TPF;
-      const T pz = zg.pz0[ph] + T(q) * zg.dz;
-      const T inv = rsqrt(zg.pxy2[ph] + pz * pz);
-      T s = tile[z * TX + c] * ylm_q<T, L, M>(pz * inv);
-#pragma unroll
-      for (int j = 0; j < M; ++j) s *= inv;
-      v[q] = cmk(s * cr, s * ci);
-    }
-  }
-}
+// ---------------------------------------------------------------------------------------------
+// Weighted first passes.  Y_lm(xhat) = norm Q_lm(uz) ((px + i py)/r)^m splits into a real signal along z,
+// s(z) = mesh(z) Q_lm(uz) r^-m, and the column factor norm (px + i py)^m, constant along z.  So
+//   k_fwd_z     transforms the signals of every (phase, l, m), two real signals per complex transform
+//               (phases a and b of one harmonic where both exist), and stores one half spectrum S per
+//               signal: 18 for l = 0, 2, 4 and two phases, where the parts of Y_lm make 30 real fields;
+//   k_fft_cols_weighted  reads S once, multiplies it by the real and by the imaginary part of the column
+//               factor and transforms both along y.  S lies in the slot of the imaginary part's field:
+//               the CTA that overwrites a column of it has read that column before.
+// (With the column factors applied in the first pass the 30 fields were written by it and read by the
+// second: at 512^3 16.1 + 28.7 GB instead of 9.7 + 22.3 GB.)
+// ---------------------------------------------------------------------------------------------
+struct Signal {
+  int8_t phase, l, m;
+  int8_t re, im;     // fields of the real and of the imaginary part (-1: none; m = 0 has re only)
+  __host__ __device__ int slot() const { return im >= 0 ? im : re; }
+};
+// Two signals that share a complex transform have to be of one magnitude, since each is rounded at the
+// larger one's: phases a and b of a harmonic are, and without interlacing two harmonics of one m (r^-m)
+// are once they carry their norm.
+constexpr int MAX_SIGNALS = 32;   // 2 phases x 15 harmonics, and room to pair them
+struct SignalList {
+  int n;                          // pairs (2p, 2p + 1); one without a partner has a second with re = im = -1
+  int norm_in_signal;             // the norm of Y_lm multiplies s(z), else the column factor
+  Signal s[MAX_SIGNALS];
+};
 
-// The real column signal of the (L, M > 0) fields of mesh phase PH: Y_LM(xhat) = norm Q_LM(uz)
-// ((px + i py)/r)^M splits into s(z) = mesh(z) Q_LM(uz) r^-M, real, and the column factor
-// cr + i ci = norm (px + i py)^M, constant along z; the transforms of the fields' real and imaginary
-// parts are cr S(kz) and ci S(kz), S the transform of s.
-template <typename T, int N, int TX, int L, int M, int PH>
-__device__ __forceinline__ void std_real(T (&sv)[8], T& cr, T& ci, const T* tile, int c, int t, const ZGeom<T>& zg,
-                                         const YNorm& nrm) {
+// s(z) times norm of one signal at the thread's elements z = t + q TPF
+template <typename T, int N, int TX, int L, int M>
+__device__ __forceinline__ void column_signal(T (&sv)[8], const T* tile, int c, int t, T pxy2, T pz0, T dz, T norm) {
   constexpr int TPF = N / 8;
-  cr = ynorm<T>(nrm, L * (L + 1) / 2 + M);
-  ci = T(0);
-#pragma unroll
-  for (int j = 0; j < M; ++j) {
-    const T nr = cr * zg.px[PH] - ci * zg.py[PH];
-    ci = cr * zg.py[PH] + ci * zg.px[PH];
-    cr = nr;
-  }
-  keep_here(cr);
-  keep_here(ci);
+  keep_here(pxy2);
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    const int z = t + q * TPF;
-    const T pz = zg.pz0[PH] + T(q) * zg.dz;
-    const T inv = rsqrt(zg.pxy2[PH] + pz * pz);
-    T v = tile[z * TX + c] * ylm_q<T, L, M>(pz * inv);
+    const T F = tile[(t + q * TPF) * TX + c];
+    if constexpr (L == 0) {
+      sv[q] = F;
+    } else {
+      const T pz = pz0 + T(q) * dz;
+      const T r2 = pxy2 + pz * pz;
+      const T inv = r2 > T(0) ? rsqrt(r2) : T(0);
+      if constexpr (M == 0) {
+        sv[q] = F * (norm * ylm_q<T, L, 0>(pz * inv));
+      } else {
+        T v = F * (norm * ylm_q<T, L, M>(pz * inv));
 #pragma unroll
-    for (int j = 0; j < M; ++j) v *= inv;
-    sv[q] = v;
+        for (int j = 0; j < M; ++j) v *= inv;
+        sv[q] = v;
+      }
+    }
   }
 }
 
-// Phases a and b of one (L, M > 0): s_a + i s_b in one complex transform (two real signals), then
-// S_a(k) = (Z(k) + Z(N - k)^*) / 2 and S_b(k) = (Z(k) - Z(N - k)^*) / 2i give the four half spectra.
-template <typename T, int N, int TX, int L, int M>
-__device__ __forceinline__ void std_pair_ab(cplx<T> (&v)[8], T (&cf)[4], const T* tileA, const T* tileB, int c, int t,
-                                            const ZGeom<T>& zg, const YNorm& nrm) {
-  T sa[8], sb[8];
-  std_real<T, N, TX, L, M, 0>(sa, cf[0], cf[1], tileA, c, t, zg, nrm);
-  std_real<T, N, TX, L, M, 1>(sb, cf[2], cf[3], tileB, c, t, zg, nrm);
-#pragma unroll
-  for (int q = 0; q < 8; ++q) v[q] = cmk(sa[q], sb[q]);
+template <typename T, int N, int TX>
+__device__ __forceinline__ void any_signal(T (&sv)[8], const Signal& sg, const T* tileA, const T* tileB, int c, int t,
+                                           const T (&pxy2)[2], const T (&pz0)[2], T dz, const YNorm& nrm,
+                                           bool norm_in) {
+  const T* tile = sg.phase ? tileB : tileA;
+  const T p2 = sg.phase ? pxy2[1] : pxy2[0], z0 = sg.phase ? pz0[1] : pz0[0];
+#define NPC_S(L, M) \
+  case L * (L + 1) / 2 + M: column_signal<T, N, TX, L, M>(sv, tile, c, t, p2, z0, dz, M == 0 || norm_in ? ynorm<T>(nrm, L * (L + 1) / 2 + M) : T(1)); break;
+  switch (sg.l * (sg.l + 1) / 2 + sg.m) {
+    NPC_S(1, 0) NPC_S(1, 1) NPC_S(2, 0) NPC_S(2, 1) NPC_S(2, 2) NPC_S(3, 0) NPC_S(3, 1) NPC_S(3, 2) NPC_S(3, 3)
+    NPC_S(4, 0) NPC_S(4, 1) NPC_S(4, 2) NPC_S(4, 3) NPC_S(4, 4)
+    default: column_signal<T, N, TX, 0, 0>(sv, tile, c, t, p2, z0, dz, T(1));
+  }
+#undef NPC_S
 }
 
-// float: the occupancy of the form without packed phase pairs (64 registers at 512 threads, at most
-// 80 otherwise), so that the pairs' extra live values do not cost CTAs per SM
-template <typename T, int N> constexpr int zstd_min_blocks() {
+// Padded column exchange: with fewer than 16 columns a 16-lane access covers several rows, and after
+// span 1 thread t writes row 8 t + r, a multiple of the banks apart; one pad row per 8 separates them.
+template <typename C, int TX, bool PK> struct ColPadView {
+  static constexpr bool PACKED = PK;
+  C* p;
+  __device__ __forceinline__ void st(int n, C v) const { p[n * TX] = v; }
+  __device__ __forceinline__ C ld(int n) const { return p[n * TX]; }
+  template <int Ns> __device__ __forceinline__ static int row(int n) { return TX < 16 && Ns == 1 ? n + (n >> 3) : n; }
+  template <int Ns> __device__ __forceinline__ void put(int n, C v) const { p[row<Ns>(n) * TX] = v; }
+  template <int Ns> __device__ __forceinline__ C get(int n) const { return p[row<Ns>(n) * TX]; }
+  __device__ __forceinline__ ColPadView sub(int off) const { return ColPadView{p + (off + (TX < 16 ? off >> 3 : 0)) * TX}; }
+};
+template <int N, int TX> constexpr int col_rows() { return TX < 16 ? N + N / 8 : N; }
+
+// float: occupancy of the register counts this kernel needs (64 at 512 threads, at most 80 otherwise)
+template <typename T, int N> constexpr int zpass_min_blocks() {
   return sizeof(T) == 4 ? 65536 / (ColCfg<N>::THREADS * (ColCfg<N>::THREADS == 512 ? 64 : 80)) : 1;
 }
+
+// Coordinates of the grid points from the observer, tab[axis][phase][n], formed in float64 and rounded
+// once (phase b lies half a cell lower): the weighted passes look them up instead of forming them per
+// thread, since float64 arithmetic is scarce on this part (y pass at 512^3: 10.1 ms with, 5.5 without).
+template <typename T>
+__global__ void k_axis_coords(const Geom g, T* __restrict__ tab) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 6 * g.n; i += gridDim.x * blockDim.x) {
+    const int a = i / (2 * g.n), ph = (i / g.n) % 2, j = i % g.n;
+    const double o = a == 0 ? g.o[0] : (a == 1 ? g.o[1] : g.o[2]);
+    tab[i] = (T)(o + ((double)j - (ph ? 0.5 : 0.0)) * g.h);
+  }
+}
+
+// First pass: the signals' half spectra along z, S[slot][kz][y][x].
 template <typename T, int N>
-__global__ void __launch_bounds__(ColCfg<N>::THREADS, zstd_min_blocks<T, N>())
-k_fwd_z_std(const T* __restrict__ mesh_a, const T* __restrict__ mesh_b, cplx<T>* __restrict__ half, int npairs,
-            const Geom g, const YNorm nrm, const cplx<T>* __restrict__ tw_g, int KZ) {
+__global__ void __launch_bounds__(ColCfg<N>::THREADS, zpass_min_blocks<T, N>())
+k_fwd_z(const T* __restrict__ mesh_a, const T* __restrict__ mesh_b, cplx<T>* __restrict__ half,
+        const __grid_constant__ SignalList sl, const T* __restrict__ coords, const T dz, const YNorm nrm,
+        const cplx<T>* __restrict__ tw_g, int KZ) {
   using C = cplx<T>;
   constexpr int TX = ColCfg<N>::TX;
   constexpr int TPF = N / 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* work = tw + N;
-  T* tileA = reinterpret_cast<T*>(work + N * TX);
-  T* tileB = tileA + N * TX;
+  T* tileA = reinterpret_cast<T*>(work + col_rows<N, TX>() * TX);
+  T* tileB = mesh_b ? tileA + N * TX : tileA;
   const int tid = threadIdx.x;
   const int c = tid % TX, t = tid / TX;
   const int x0 = blockIdx.x * TX, y = blockIdx.y;
@@ -348,118 +234,172 @@ k_fwd_z_std(const T* __restrict__ mesh_a, const T* __restrict__ mesh_b, cplx<T>*
     const int z = i / TX, cc = i % TX;
     const size_t gi = ((size_t)z * N + y) * N + x0 + cc;
     tileA[i] = mesh_a[gi];
-    tileB[i] = mesh_b[gi];
+    if (mesh_b) tileB[i] = mesh_b[gi];
   }
-  ZGeom<T> zg;
-  for (int ph = 0; ph < 2; ++ph) {
-    const double sh = ph ? 0.5 : 0.0;
-    zg.px[ph] = (T)(g.o[0] + ((double)(x0 + c) - sh) * g.h);
-    zg.py[ph] = (T)(g.o[1] + ((double)y - sh) * g.h);
-    zg.pxy2[ph] = zg.px[ph] * zg.px[ph] + zg.py[ph] * zg.py[ph];
-    zg.pz0[ph] = (T)(g.o[2] + ((double)t - sh) * g.h);
+  T pxy2[2] = {T(0), T(0)}, pz0[2] = {T(0), T(0)};
+  if (coords) {
+#pragma unroll
+    for (int ph = 0; ph < 2; ++ph) {
+      const T px = coords[ph * N + x0 + c], py = coords[(2 + ph) * N + y];
+      pxy2[ph] = px * px + py * py;
+      pz0[ph] = coords[(4 + ph) * N + t];
+    }
   }
-  zg.dz = (T)(g.h * TPF);
   __syncthreads();
   const size_t fstride = (size_t)KZ * N * N;
-  for (int p = 0; p < npairs; ++p) {
+#pragma unroll 1
+  for (int p = 0; p < sl.n; p += 2) {
+    const Signal s0 = sl.s[p], s1 = sl.s[p + 1];
     C v[8];
-    // pairs 2k and 2k + 1 of an m > 0 harmonic (phase a, phase b): one transform for both
-    const bool ab = (p == 2 || p == 4 || p == 7 || p == 9 || p == 11 || p == 13) && p + 1 < npairs;
-    if (ab) {
-      T cf[4];   // cr, ci of phase a, then of phase b
-      switch (p) {
-        case 2: std_pair_ab<T, N, TX, 2, 1>(v, cf, tileA, tileB, c, t, zg, nrm); break;
-        case 4: std_pair_ab<T, N, TX, 2, 2>(v, cf, tileA, tileB, c, t, zg, nrm); break;
-        case 7: std_pair_ab<T, N, TX, 4, 1>(v, cf, tileA, tileB, c, t, zg, nrm); break;
-        case 9: std_pair_ab<T, N, TX, 4, 2>(v, cf, tileA, tileB, c, t, zg, nrm); break;
-        case 11: std_pair_ab<T, N, TX, 4, 3>(v, cf, tileA, tileB, c, t, zg, nrm); break;
-        default: std_pair_ab<T, N, TX, 4, 4>(v, cf, tileA, tileB, c, t, zg, nrm); break;
-      }
-      fft_block<N, -1>(v, t, tw, ColView<C>{work + c, TX});
+    {
+      T a[8], b[8];
+      any_signal<T, N, TX>(a, s0, tileA, tileB, c, t, pxy2, pz0, dz, nrm, sl.norm_in_signal);
+      if (s1.re >= 0) {
+        any_signal<T, N, TX>(b, s1, tileA, tileB, c, t, pxy2, pz0, dz, nrm, sl.norm_in_signal);
+      } else {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) work[(t + q * TPF) * TX + c] = v[q];
-      __syncthreads();
-      {
-        // thread tid owns (kz0 + j KZSTEP, cc) with cc = tid % TX = c: its column's factors
-        constexpr int KZSTEP = ColCfg<N>::THREADS / TX;
-        const int kz0 = tid / TX, cc = tid % TX;
-        C* o0 = half + (size_t)(2 * p) * fstride + ((size_t)kz0 * N + y) * N + x0 + cc;
-        for (int kz = kz0; kz < KZ; kz += KZSTEP, o0 += (size_t)KZSTEP * N * N) {
-          const C z1 = work[kz * TX + cc];
-          const C z2 = cconj(work[(kz == 0 ? 0 : N - kz) * TX + cc]);
-          const C sa = cscale(cadd(z1, z2), T(0.5));
-          const C d = csub(z1, z2);
-          const C sb = cmk(T(0.5) * d.y, T(-0.5) * d.x);
-          o0[0] = cscale(sa, cf[0]);
-          o0[fstride] = cscale(sa, cf[1]);
-          o0[2 * fstride] = cscale(sb, cf[2]);
-          o0[3 * fstride] = cscale(sb, cf[3]);
-        }
+        for (int q = 0; q < 8; ++q) b[q] = T(0);
       }
-      __syncthreads();
-      ++p;
-      continue;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = cmk(a[q], b[q]);
     }
-    switch (p) {
-      case 0: std_inputs<T, N, TX, 0, 0, 0>(v, tileA, tileB, c, t, zg, nrm); break;
-      case 1: std_inputs<T, N, TX, 2, 0, 0>(v, tileA, tileB, c, t, zg, nrm); break;
-      case 2: std_inputs<T, N, TX, 2, 1, 1>(v, tileA, tileB, c, t, zg, nrm); break;
-      case 3: std_inputs<T, N, TX, 2, 1, 2>(v, tileA, tileB, c, t, zg, nrm); break;
-      case 4: std_inputs<T, N, TX, 2, 2, 1>(v, tileA, tileB, c, t, zg, nrm); break;
-      case 5: std_inputs<T, N, TX, 2, 2, 2>(v, tileA, tileB, c, t, zg, nrm); break;
-      case 6: std_inputs<T, N, TX, 4, 0, 0>(v, tileA, tileB, c, t, zg, nrm); break;
-      case 7: std_inputs<T, N, TX, 4, 1, 1>(v, tileA, tileB, c, t, zg, nrm); break;
-      case 8: std_inputs<T, N, TX, 4, 1, 2>(v, tileA, tileB, c, t, zg, nrm); break;
-      case 9: std_inputs<T, N, TX, 4, 2, 1>(v, tileA, tileB, c, t, zg, nrm); break;
-      case 10: std_inputs<T, N, TX, 4, 2, 2>(v, tileA, tileB, c, t, zg, nrm); break;
-      case 11: std_inputs<T, N, TX, 4, 3, 1>(v, tileA, tileB, c, t, zg, nrm); break;
-      case 12: std_inputs<T, N, TX, 4, 3, 2>(v, tileA, tileB, c, t, zg, nrm); break;
-      case 13: std_inputs<T, N, TX, 4, 4, 1>(v, tileA, tileB, c, t, zg, nrm); break;
-      default: std_inputs<T, N, TX, 4, 4, 2>(v, tileA, tileB, c, t, zg, nrm); break;
-    }
-    fft_block<N, -1>(v, t, tw, ColView<C>{work + c, TX});
+    fft_block<N, -1>(v, t, tw, ColPadView<C, TX, true>{work + c});
 #pragma unroll
     for (int q = 0; q < 8; ++q) work[(t + q * TPF) * TX + c] = v[q];
     __syncthreads();
-    // split the packed pair into its two half spectra; thread tid owns (kz0 + j KZSTEP, cc)
+    // split the packed pair, S_0 = (Z(k) + Z(N - k)^*) / 2 and S_1 = (Z(k) - Z(N - k)^*) / 2i; thread tid
+    // owns (kz0 + j KZSTEP, c)
     {
       constexpr int KZSTEP = ColCfg<N>::THREADS / TX;
-      const int kz0 = tid / TX, cc = tid % TX;
-      C* o0 = half + (size_t)(2 * p) * fstride + ((size_t)kz0 * N + y) * N + x0 + cc;
-      C* o1 = o0 + fstride;
-      for (int kz = kz0; kz < KZ; kz += KZSTEP, o0 += (size_t)KZSTEP * N * N, o1 += (size_t)KZSTEP * N * N) {
-        const C z1 = work[kz * TX + cc];
-        const C z2 = cconj(work[(kz == 0 ? 0 : N - kz) * TX + cc]);
+      const size_t row0 = ((size_t)t * N + y) * N + x0 + c;
+      C* o0 = half + (size_t)s0.slot() * fstride + row0;
+      C* o1 = half + (size_t)(s1.re >= 0 ? s1.slot() : 0) * fstride + row0;
+      for (int kz = t; kz < KZ; kz += KZSTEP, o0 += (size_t)KZSTEP * N * N, o1 += (size_t)KZSTEP * N * N) {
+        const C z1 = work[kz * TX + c];
+        const C z2 = cconj(work[(kz == 0 ? 0 : N - kz) * TX + c]);
         *o0 = cscale(cadd(z1, z2), T(0.5));
         const C d = csub(z1, z2);
-        *o1 = cmk(T(0.5) * d.y, T(-0.5) * d.x);
+        if (s1.re >= 0) *o1 = cmk(T(0.5) * d.y, T(-0.5) * d.x);
       }
     }
     __syncthreads();
   }
 }
 
-// Number of leading standard pairs the field list matches (0 if it does not follow the layout).
-static int std_pairs(const FieldList& fl) {
-  static const int8_t tbl[15][3] = {{0, 0, 0}, {2, 0, 0}, {2, 1, 1}, {2, 1, 2}, {2, 2, 1}, {2, 2, 2}, {4, 0, 0},
-                                    {4, 1, 1}, {4, 1, 2}, {4, 2, 1}, {4, 2, 2}, {4, 3, 1}, {4, 3, 2}, {4, 4, 1},
-                                    {4, 4, 2}};
-  if (fl.nf % 2) return 0;
-  const int np = fl.nf / 2;
-  if (np > 15) return 0;
-  for (int p = 0; p < np; ++p) {
-    const Comp a = fl.f[2 * p], b = fl.f[2 * p + 1];
-    const int l = tbl[p][0], m = tbl[p][1], kind = tbl[p][2];
-    if (a.ell != l || b.ell != l || a.m != m || b.m != m) return 0;
-    if (kind == 0) {
-      const int part = l == 0 ? PART_ONE : PART_RE;
-      if (a.phase != 0 || b.phase != 1 || a.part != part || b.part != part) return 0;
+// The signals of a field list: phases a and b of one harmonic paired, the others two of one m.
+static SignalList make_signals(const FieldList& fl) {
+  std::vector<Signal> all;
+  for (int f = 0; f < fl.nf; ++f) {
+    const Comp c = fl.f[f];
+    const bool one = c.part == PART_ONE;
+    Signal* s = nullptr;
+    for (Signal& x : all)
+      if (x.phase == c.phase && x.l == (one ? 0 : c.ell) && x.m == (one ? 0 : c.m)) s = &x;
+    if (!s) {
+      all.push_back(Signal{c.phase, (int8_t)(one ? 0 : c.ell), (int8_t)(one ? 0 : c.m), -1, -1});
+      s = &all.back();
+    }
+    (c.part == PART_IM ? s->im : s->re) = (int8_t)f;
+  }
+  SignalList sl{};
+  std::vector<Signal> rest;
+  for (const Signal& a : all) {
+    if (a.phase) continue;
+    const Signal* b = nullptr;
+    for (const Signal& x : all)
+      if (x.phase && x.l == a.l && x.m == a.m) b = &x;
+    if (b) {
+      sl.s[sl.n++] = a;
+      sl.s[sl.n++] = *b;
     } else {
-      const int ph = kind - 1;
-      if (a.phase != ph || b.phase != ph || a.part != PART_RE || b.part != PART_IM) return 0;
+      rest.push_back(a);
     }
   }
-  return np;
+  sl.norm_in_signal = rest.empty() ? 0 : 1;
+  for (int m = 0; m <= 4; ++m) {
+    for (const Signal& x : rest)
+      if (x.m == m) sl.s[sl.n++] = x;
+    if (sl.n % 2) sl.s[sl.n++] = Signal{0, 0, 0, -1, -1};
+  }
+  return sl;
+}
+
+// v = S norm Re (px + i py)^M and keep = S norm Im (px + i py)^M at the thread's elements
+template <typename T, int N, int TX, int M>
+__device__ __forceinline__ void column_factors(cplx<T> (&v)[8], cplx<T>* keep, const T* __restrict__ pys, T px, T norm,
+                                               int c, int t) {
+  constexpr int TPF = N / 8;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const T py = pys[t + q * TPF];
+    T cr = norm, ci = T(0);
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+      const T nr = cr * px - ci * py;
+      ci = cr * py + ci * px;
+      cr = nr;
+    }
+    keep[(t + q * TPF) * TX + c] = cscale(v[q], ci);
+    v[q] = cscale(v[q], cr);
+  }
+}
+
+// y pass with the column factors: plane (signal, kz) = blockIdx.y; the transforms of S times the
+// real and the imaginary part of norm (px + i py)^m go to the two parts' fields (m = 0: S itself, in place).
+template <typename T, int N, int TX>
+__global__ void __launch_bounds__(TX * N / 8, (sizeof(T) == 4 && TX * N / 8 <= 512 ? 1536 / (TX * N / 8) : 1))
+k_fft_cols_weighted(cplx<T>* __restrict__ half, const __grid_constant__ SignalList sl, const T* __restrict__ coords,
+                    const YNorm nrm, const cplx<T>* __restrict__ tw_g, int KZ, int row_n2max) {
+  using C = cplx<T>;
+  constexpr int TPF = N / 8;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* tw = reinterpret_cast<C*>(smem_raw);
+  C* work = tw + N;
+  C* keep = work + col_rows<N, TX>() * TX;   // the imaginary part's elements, each thread its own
+  const int tid = threadIdx.x;
+  const int c = tid % TX, t = tid / TX;
+  const int plane = blockIdx.y, kz = plane % KZ;
+  const Signal sg = sl.s[plane / KZ];
+  if (sg.re < 0) return;
+  const int x = blockIdx.x * TX + c;
+  const size_t fstride = (size_t)KZ * N * N, poff = (size_t)kz * N * N + x;
+  for (int i = tid; i < N; i += blockDim.x) tw[i] = tw_g[i];
+  C v[8];
+  {
+    const C* src = half + (size_t)sg.slot() * fstride + poff;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = src[(size_t)(t + q * TPF) * N];
+  }
+  if (sg.m > 0) {
+    const T px = coords[sg.phase * N + x];
+    const T* __restrict__ pys = coords + (2 + sg.phase) * N;
+    const T norm = sl.norm_in_signal ? T(1) : ynorm<T>(nrm, sg.l * (sg.l + 1) / 2 + sg.m);
+    switch (sg.m) {
+      case 1: column_factors<T, N, TX, 1>(v, keep, pys, px, norm, c, t); break;
+      case 2: column_factors<T, N, TX, 2>(v, keep, pys, px, norm, c, t); break;
+      case 3: column_factors<T, N, TX, 3>(v, keep, pys, px, norm, c, t); break;
+      default: column_factors<T, N, TX, 4>(v, keep, pys, px, norm, c, t);
+    }
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int part = 0; part < 2; ++part) {
+    const int f = part ? sg.im : sg.re;
+    if (f < 0) continue;
+    if (part) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = keep[(t + q * TPF) * TX + c];
+    }
+    fft_block<N, -1>(v, t, tw, ColPadView<C, TX, false>{work + c});
+    // rows (ky, kz) outside every k-bin are never read again: not stored
+    C* dst = half + (size_t)f * fstride + poff;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int yi = t + q * TPF;
+      const int jy = yi < N / 2 ? yi : yi - N;
+      if (jy * jy + kz * kz <= row_n2max) dst[(size_t)yi * N] = v[q];
+    }
+  }
 }
 
 // Column transform along a strided axis: element j of column (plane, x) at
@@ -976,6 +916,37 @@ npc_status y_pass(npc_ctx* ctx, cplx<T>* data, int nplanes, const cplx<T>* tw, i
   return set_err(ctx, NPC_ERR_INVALID_ARG, "y pass: unsupported columns per CTA %d", tx);
 }
 
+template <typename T, int N, int TX>
+npc_status y_pass_weighted_tx(npc_ctx* ctx, cplx<T>* half, const SignalList& sl, const T* coords, const YNorm& nrm,
+                              const cplx<T>* tw, int KZ, int row_n2max) {
+  using C = cplx<T>;
+  if constexpr (!ytx_ok<N>(TX)) {
+    return set_err(ctx, NPC_ERR_INVALID_ARG, "y pass: %d columns per CTA not valid at n = %d", TX, N);
+  } else {
+    const size_t smem = sizeof(C) * (N + col_rows<N, TX>() * TX + N * TX);
+    auto kern = k_fft_cols_weighted<T, N, TX>;
+    NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int nplanes = sl.n * KZ;   // at most 32 x 512
+    kern<<<dim3(N / TX, nplanes), TX * N / 8, smem, ctx->stream>>>(half, sl, coords, nrm, tw, KZ, row_n2max);
+    NPC_LAUNCH(ctx);
+    return NPC_OK;
+  }
+}
+
+template <typename T, int N>
+npc_status y_pass_weighted(npc_ctx* ctx, cplx<T>* half, const SignalList& sl, const T* coords, const YNorm& nrm,
+                           const cplx<T>* tw, int tx, int KZ, int row_n2max) {
+  // 32 columns of the longest FP64 lines and their copy would not fit an SM's shared memory
+  if (sizeof(cplx<T>) * N * tx * 2 > 150 * 1024) tx = 16;
+  switch (tx) {
+    case 4: return y_pass_weighted_tx<T, N, 4>(ctx, half, sl, coords, nrm, tw, KZ, row_n2max);
+    case 8: return y_pass_weighted_tx<T, N, 8>(ctx, half, sl, coords, nrm, tw, KZ, row_n2max);
+    case 16: return y_pass_weighted_tx<T, N, 16>(ctx, half, sl, coords, nrm, tw, KZ, row_n2max);
+    case 32: return y_pass_weighted_tx<T, N, 32>(ctx, half, sl, coords, nrm, tw, KZ, row_n2max);
+  }
+  return set_err(ctx, NPC_ERR_INVALID_ARG, "y pass: unsupported columns per CTA %d", tx);
+}
+
 // Autotuner for the y pass: times every valid columns-per-CTA choice on a scratch buffer of
 // `nplanes` planes (values irrelevant to the timing) and keeps the fastest for (n, precision).
 template <typename T, int N>
@@ -1026,36 +997,41 @@ npc_status fwd_impl(npc_ctx* ctx, const PowerPlan& plan, const Geom& g, const vo
   NPC_TRY(get_twiddles(ctx, N, sizeof(T) == 8 ? NPC_PREC_FP64 : NPC_PREC_MIXED, &twp));
   const C* tw = (const C*)twp;
   const YNorm nrm = ylm_norm_table();
-  {
-    const size_t smem = sizeof(C) * (N + N * TX) + sizeof(T) * 2 * N * TX;
-    dim3 grid(N / TX, N);
-    const int nstd = mesh_b ? std_pairs(plan.fl) : 0;
-    const bool single = !mesh_b && plan.fl.nf == 1 && plan.fl.f[0].part == PART_ONE && plan.fl.f[0].phase == 0;
-    if (single) {
-      constexpr int STX = SingleCfg<N>::TX;
-      static_assert(N % (2 * STX) == 0, "column pairs must tile the mesh");
-      const size_t ssmem = sizeof(C) * (N + N * STX);
-      auto kern = k_fwd_z_single<T, N>;
-      NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem));
-      kern<<<dim3(N / (2 * STX), N), SingleCfg<N>::THREADS, ssmem, ctx->stream>>>((const T*)mesh_a, (C*)half, tw,
-                                                                                   KZ);
-    } else if (nstd > 0) {
-      auto kern = k_fwd_z_std<T, N>;
-      NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      kern<<<grid, ColCfg<N>::THREADS, smem, ctx->stream>>>((const T*)mesh_a, (const T*)mesh_b, (C*)half, nstd, g,
-                                                            nrm, tw, KZ);
-    } else {
-      auto kern = k_fwd_z<T, N>;
-      NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      kern<<<grid, ColCfg<N>::THREADS, smem, ctx->stream>>>((const T*)mesh_a, (const T*)mesh_b, (C*)half, plan.fl,
-                                                            g, nrm, tw, KZ);
-    }
-    NPC_LAUNCH(ctx);
-    NPC_TRY(stage_mark(ctx, "fft_z_weighted"));
+  const bool single = !mesh_b && plan.fl.nf == 1 && plan.fl.f[0].part == PART_ONE && plan.fl.f[0].phase == 0;
+  const SignalList sl = make_signals(plan.fl);
+  bool directions = false, weighted = false;   // harmonics of l > 0, of m > 0
+  for (int i = 0; i < sl.n; ++i) {
+    directions |= sl.s[i].l > 0;
+    weighted |= sl.s[i].m > 0;
   }
+  T* coords = nullptr;
+  if (directions) {
+    NPC_TRY(ws_get(ctx, "fwd.coords", sizeof(T) * 6 * N, (void**)&coords));
+    k_axis_coords<T><<<(6 * N + 255) / 256, 256, 0, ctx->stream>>>(g, coords);
+    NPC_LAUNCH(ctx);
+  }
+  if (single) {
+    constexpr int STX = SingleCfg<N>::TX;
+    static_assert(N % (2 * STX) == 0, "column pairs must tile the mesh");
+    const size_t ssmem = sizeof(C) * (N + N * STX);
+    auto kern = k_fwd_z_single<T, N>;
+    NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem));
+    kern<<<dim3(N / (2 * STX), N), SingleCfg<N>::THREADS, ssmem, ctx->stream>>>((const T*)mesh_a, (C*)half, tw, KZ);
+  } else {
+    const size_t smem = sizeof(C) * (N + col_rows<N, TX>() * TX) + sizeof(T) * (mesh_b ? 2 : 1) * N * TX;
+    auto kern = k_fwd_z<T, N>;
+    NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<dim3(N / TX, N), ColCfg<N>::THREADS, smem, ctx->stream>>>((const T*)mesh_a, (const T*)mesh_b, (C*)half, sl,
+                                                                     coords, (T)(g.h * (N / 8)), nrm, tw, KZ);
+  }
+  NPC_LAUNCH(ctx);
+  NPC_TRY(stage_mark(ctx, "fft_z_weighted"));
+  const int n2max = plan.row_n2max > 0 ? plan.row_n2max : (1 << 30);
   // planes (f, kz) are contiguous N*N blocks; y rows have stride N
-  NPC_TRY((y_pass<T, N>(ctx, (C*)half, plan.fl.nf * KZ, tw, ytx_for(ctx, N, sizeof(T) == 8), KZ,
-                        plan.row_n2max > 0 ? plan.row_n2max : (1 << 30))));
+  if (weighted)
+    NPC_TRY((y_pass_weighted<T, N>(ctx, (C*)half, sl, coords, nrm, tw, ytx_for(ctx, N, sizeof(T) == 8), KZ, n2max)));
+  else
+    NPC_TRY((y_pass<T, N>(ctx, (C*)half, plan.fl.nf * KZ, tw, ytx_for(ctx, N, sizeof(T) == 8), KZ, n2max)));
   NPC_TRY(stage_mark(ctx, "fft_y"));
   return NPC_OK;
 }
