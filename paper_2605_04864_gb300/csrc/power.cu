@@ -29,6 +29,15 @@
 
 namespace {
 
+// 1/sqrt(a) for the direction of a mode: the hardware approximation errs to one side, and P_4b and P_8b are
+// small differences of sums that all scale with the length of khat (to the powers 2 and 4); one Newton step
+// brought their errors from 1.7e-6 and 4.9e-6 to 1.0e-6 and 0.9e-6 (256^3, mean over eight catalogues).
+__device__ __forceinline__ float rsqrt_unbiased(float a) {
+  const float y = rsqrt(a);
+  return fmaf(0.5f * y, fmaf(-a * y, y, 1.0f), y);
+}
+__device__ __forceinline__ double rsqrt_unbiased(double a) { return rsqrt(a); }
+
 constexpr int CONTRACT_THREADS = 256;
 constexpr int MAX_PRODS = 8;              // P_0 .. P_4 and P_22, P_42, P_44
 constexpr int MAX_SUMS = MAX_PRODS + 2;   // and the modes and their |k|
@@ -434,22 +443,38 @@ k_fft_cols(cplx<T>* __restrict__ data, size_t plane_stride, int row_stride, cons
 }
 
 // One step of the x pass: a stored real field, its k-space coefficient scale * part of Q_lm(uz)
-// (ux + i uy)^m (scale = 4 pi/(2l+1) * (m > 0 ? 2 : 1) * the norm of Y_lm), and what follows it.
+// (ux + i uy)^m, and what follows it.  scale = 4 pi/(2l+1) * (m > 0 ? 2 : 1) * norm_lm^2 = 2 (l-m)!/(l+m)!
+// (m > 0) over the norm that the first passes applied, in the value it had there.  A rounding of scale
+// would be common to all modes, and P_4 is a small difference of large terms of different m, so the float
+// coefficient is a product of two factors chosen to match it to about 2^-36; the products round per mode.
 struct FieldStep {
   int8_t field;  // index into the half-spectrum buffer
   int8_t weight; // 2 (l(l+1)/2 + m) + (1 for the imaginary part); 0: no weight (F_0, global line of sight)
   int8_t acc;    // accumulator of the step's multipole
   int8_t flags;  // STEP_ROTATE, STEP_STORE
-  float scale_f;
+  float scale_f[2];
   double scale_d;
 };
 // the accumulator holds phase b only so far: apply the interlacing phase e^{i pi (i + j + l)/N}
 constexpr int8_t STEP_ROTATE = 1;
 // the accumulator's last field: apply the window factor and store F_l
 constexpr int8_t STEP_STORE = 2;
-template <typename T> __device__ __forceinline__ T step_scale(const FieldStep& c);
-template <> __device__ __forceinline__ float step_scale<float>(const FieldStep& c) { return c.scale_f; }
-template <> __device__ __forceinline__ double step_scale<double>(const FieldStep& c) { return c.scale_d; }
+__device__ __forceinline__ float scaled(const FieldStep& c, float w) { return c.scale_f[1] * (c.scale_f[0] * w); }
+__device__ __forceinline__ double scaled(const FieldStep& c, double w) { return c.scale_d * w; }
+
+// factors f[0] f[1] = w to about 2^-36
+static void split_scale(double w, float (&f)[2]) {
+  double best = 1e300;
+  for (int k = 0; k < 4096; ++k) {
+    const float a = 1.0f + (float)k * 1.1920929e-07f, b = (float)(w / (double)a);
+    const double e = std::fabs((double)a * (double)b - w);
+    if (e < best) {
+      best = e;
+      f[0] = a;
+      f[1] = b;
+    }
+  }
+}
 
 // A binned sum: Re (Im, when one of the two l is odd) of F_lx F_ly^*, and the accumulators that hold them
 // (F_0's for every l with a global line of sight).
@@ -514,10 +539,10 @@ template <int N> struct XTeam {
   static constexpr int THREADS = BLOCK ? 96 : CONTRACT_THREADS;
 };
 
-// v[q] (mode kx = t + q TPF) times scale * the part of Q_LM(uz) (ux + i uy)^M, added to acc.
+// v[q] (mode kx = t + q TPF) times the step's scale * the part of Q_LM(uz) (ux + i uy)^M, added to acc.
 template <typename T, int N, int L, int M, int IM>
-__device__ __forceinline__ void add_weighted(cplx<T> (&acc)[8], const cplx<T> (&v)[8], const T (&inv)[8], T scale,
-                                             int t, T fj, T fk) {
+__device__ __forceinline__ void add_weighted(cplx<T> (&acc)[8], const cplx<T> (&v)[8], const T (&inv)[8],
+                                             const FieldStep& st, int t, T fj, T fk) {
   constexpr int TPF = N / 8;
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
@@ -531,7 +556,7 @@ __device__ __forceinline__ void add_weighted(cplx<T> (&acc)[8], const cplx<T> (&
       pi = pr * uy + pi * ux;
       pr = nr;
     }
-    const T w = scale * (ylm_q<T, L, M>(fk * iv) * (IM ? pi : pr));
+    const T w = scaled(st, ylm_q<T, L, M>(fk * iv) * (IM ? pi : pr));
     acc[q] = cmk(acc[q].x + w * v[q].x, acc[q].y + w * v[q].y);
   }
 }
@@ -632,7 +657,7 @@ k_fft_x_contract(const cplx<T>* __restrict__ half, const __grid_constant__ Contr
         for (int q = 0; q < 8; ++q) {
           const T fi = T(t + (q < 4 ? q : q - 8) * TPF), fj = T(jy), fk = T(kz);
           const T r2 = fi * fi + fj * fj + fk * fk;
-          inv[q] = r2 > T(0) ? rsqrt(r2) : T(0);
+          inv[q] = r2 > T(0) ? rsqrt_unbiased(r2) : T(0);
           racc[q] = cmk(T(0), T(0));
         }
         if (team_any(live)) {
@@ -662,9 +687,9 @@ k_fft_x_contract(const cplx<T>* __restrict__ half, const __grid_constant__ Contr
               else fft_block_alternate<N, -1>(v, t, tw, b0, b1, SyncNamed{1 + g, TPF});
               flip ^= fft_exchanges<N>() & 1;
             }
-            const T sc = step_scale<T>(c), fj = T(jy), fk = T(kz);
+            const T fj = T(jy), fk = T(kz);
 #define NPC_W(L, M, IM) \
-  case 2 * (L * (L + 1) / 2 + M) + IM: add_weighted<T, N, L, M, IM>(racc, v, inv, sc, t, fj, fk); break;
+  case 2 * (L * (L + 1) / 2 + M) + IM: add_weighted<T, N, L, M, IM>(racc, v, inv, c, t, fj, fk); break;
             switch (c.weight) {
               NPC_W(1, 0, 0) NPC_W(1, 1, 0) NPC_W(1, 1, 1)
               NPC_W(2, 0, 0) NPC_W(2, 1, 0) NPC_W(2, 1, 1) NPC_W(2, 2, 0) NPC_W(2, 2, 1)
@@ -1088,9 +1113,10 @@ npc_status contract_impl(npc_ctx* ctx, const PowerPlan& plan, const npc_mesh_spe
         if (c.part == PART_RE || c.part == PART_IM) {
           const int lm = c.ell * (c.ell + 1) / 2 + c.m;
           st.weight = (int8_t)(2 * lm + (c.part == PART_IM ? 1 : 0));
-          st.scale_d = 4.0 * M_PI / (2 * c.ell + 1) * (c.m > 0 ? 2.0 : 1.0) * nrm.v[lm];
+          const double applied = sizeof(T) == 4 ? (double)nrm.f[lm] : nrm.v[lm];   // by the first passes
+          st.scale_d = 4.0 * M_PI / (2 * c.ell + 1) * (c.m > 0 ? 2.0 : 1.0) * nrm.v[lm] * nrm.v[lm] / applied;
+          if (sizeof(T) == 4) split_scale(st.scale_d, st.scale_f);
         }
-        st.scale_f = (float)st.scale_d;
       }
       if (ph == 1) P.step[P.nsteps - 1].flags |= STEP_ROTATE;
     }
