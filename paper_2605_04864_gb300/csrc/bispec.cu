@@ -409,34 +409,47 @@ struct LosFrame {
   double e1[3], e2[3], e3[3];
 };
 
-// power-basis coefficients of the Legendre polynomials L_0 .. L_4
-__constant__ double c_legendre[5][5] = {{1.0, 0.0, 0.0, 0.0, 0.0},
-                                        {0.0, 1.0, 0.0, 0.0, 0.0},
-                                        {-0.5, 0.0, 1.5, 0.0, 0.0},
-                                        {0.0, -1.5, 0.0, 2.5, 0.0},
-                                        {0.375, 0.0, -3.75, 0.0, 4.375}};
+// Power-basis coefficients of d^m L_l/dmu^m for 0 <= m <= l <= 4 (all exact in float), entry [l][m][j] the
+// factor of mu^j, and the Racah norms (-1)^m sqrt((l-m)!/(l+m)!), as tables of both types: formed per
+// element in float64 they cost more than the transforms (x pass of the TripoSH shells 513 -> 190 us at
+// 256^3), float64 conversions and arithmetic being scarce on this part.
+#define NPC_DLEG                                                                                       \
+  {{{1}},                                                                                              \
+   {{0, 1}, {1}},                                                                                      \
+   {{-0.5, 0, 1.5}, {0, 3}, {3}},                                                                      \
+   {{0, -1.5, 0, 2.5}, {-1.5, 0, 7.5}, {0, 15}, {15}},                                                 \
+   {{0.375, 0, -3.75, 0, 4.375}, {0, -7.5, 0, 17.5}, {-7.5, 0, 52.5}, {0, 105}, {105}}}
+__constant__ float c_dleg_f[5][5][5] = NPC_DLEG;
+__constant__ double c_dleg_d[5][5][5] = NPC_DLEG;
+#undef NPC_DLEG
+template <typename T> __device__ __forceinline__ T dleg(int l, int m, int j);
+template <> __device__ __forceinline__ float dleg<float>(int l, int m, int j) { return c_dleg_f[l][m][j]; }
+template <> __device__ __forceinline__ double dleg<double>(int l, int m, int j) { return c_dleg_d[l][m][j]; }
 
 template <typename T>
 __device__ __forceinline__ T legendre_dev(int l, T mu) {
   T r = T(0);
-  for (int k = l; k >= 0; --k) r = r * mu + T(c_legendre[l][k]);
+  for (int k = l; k >= 0; --k) r = r * mu + dleg<T>(l, 0, k);
   return r;
 }
 
-// Racah-normalised y_l^m = sqrt(4 pi/(2l+1)) Y_l^m for 0 <= m <= l <= 4 at the unit vector (x, y, z):
-// (-1)^m sqrt((l-m)!/(l+m)!) (d^m L_l/dmu^m)(z) (x + i y)^m, the Condon-Shortley phase included.
+// (-1)^m sqrt((l-m)!/(l+m)!)
 template <typename T>
-__device__ __forceinline__ void ylm_frame(int l, int m, T x, T y, T z, T& re, T& im) {
+__device__ __forceinline__ T racah_norm(int l, int m) {
+  T ratio = T(1);   // (l+m)!/(l-m)!, at most 8!
+  for (int q = l - m + 1; q <= l + m; ++q) ratio *= T(q);
+  return T((m & 1) ? -1.0 : 1.0) / sqrt(ratio);
+}
+
+// Racah-normalised y_l^m = sqrt(4 pi/(2l+1)) Y_l^m for 0 <= m <= l <= 4 at the unit vector (x, y, z):
+// norm (d^m L_l/dmu^m)(z) (x + i y)^m with norm = racah_norm(l, m), the Condon-Shortley phase included.
+template <typename T>
+__device__ __forceinline__ void ylm_frame(int l, int m, T nrm, T x, T y, T z, T& re, T& im) {
   T d = T(0), zp = T(1);
   for (int k = m; k <= l; ++k) {
-    T f = T(c_legendre[l][k]);
-    for (int q = k - m + 1; q <= k; ++q) f *= T(q);   // k!/(k-m)!
-    d += f * zp;
+    d += dleg<T>(l, m, k - m) * zp;
     zp *= z;
   }
-  double ratio = 1.0;
-  for (int q = l - m + 1; q <= l + m; ++q) ratio *= q;
-  const T nrm = T((m & 1) ? -1.0 : 1.0) / sqrt(T(ratio));
   T pr = T(1), pi = T(0);
   for (int q = 0; q < m; ++q) {
     const T t = pr * x - pi * y;
@@ -474,7 +487,8 @@ k_shell_x(const cplx<T>* __restrict__ X0, const cplx<T>* __restrict__ XN, const 
   T* murow = reinterpret_cast<T*>(xcrow + NS);  // mu = qhat . los per kx
   int* binrow = reinterpret_cast<int*>(murow + NS);  // bin per kx (-1 excluded), n2 per kx
   int* n2row = binrow + NS;
-  C* bufs = reinterpret_cast<C*>(n2row + NS);   // NBUF x NP
+  T* urow = reinterpret_cast<T*>(n2row + NS);   // (YW) unit vector of the mode in the frame, [3][NS]
+  C* bufs = reinterpret_cast<C*>(urow + (YW ? 3 * NS : 0));   // NBUF x NP
   const int tid = threadIdx.x;
   for (int i = tid; i < NS; i += blockDim.x) tw[i] = tw_g[i];
   const int g = tid / TPF, t = tid % TPF;
@@ -503,6 +517,13 @@ k_shell_x(const cplx<T>* __restrict__ X0, const cplx<T>* __restrict__ XN, const 
       murow[kx] = n2 > 0 ? (T(i) * T(fr.e3[0]) + T(jy) * T(fr.e3[1]) + T(kz) * T(fr.e3[2])) / kk : T(0);
       binrow[kx] = inrange ? tab[n2] : -1;
       n2row[kx] = inrange ? n2 : -1;
+      if (YW) {
+        const T ii = T(i), jj = T(jy), zz = T(kz);
+        const T inv = inrange && n2 > 0 ? T(1) / sqrt(T(n2)) : T(0);
+        urow[kx] = (ii * T(fr.e1[0]) + jj * T(fr.e1[1]) + zz * T(fr.e1[2])) * inv;
+        urow[NS + kx] = (ii * T(fr.e2[0]) + jj * T(fr.e2[1]) + zz * T(fr.e2[2])) * inv;
+        urow[2 * NS + kx] = (ii * T(fr.e3[0]) + jj * T(fr.e3[1]) + zz * T(fr.e3[2])) * inv;
+      }
     }
     __syncthreads();
     // fields active on this row
@@ -514,6 +535,7 @@ k_shell_x(const cplx<T>* __restrict__ X0, const cplx<T>* __restrict__ XN, const 
         sf = fields[f];
         live = kz <= sf.K && ay <= sf.K;
       }
+      const T ynrm = YW ? racah_norm<T>(sf.yl, sf.ym) : T(1);
       C v[8];
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
@@ -548,13 +570,8 @@ k_shell_x(const cplx<T>* __restrict__ X0, const cplx<T>* __restrict__ XN, const 
               // F_l^m = sum_q e^{iqx} (Re y - i Im y) X: for even l the real weights Re y (real part)
               // and -Im y (imaginary part) are even in q; for odd l the parts are -i Im y X and
               // -i Re y X.  Every weighted spectrum stays Hermitian, so each part is a real field.
-              const T ii = T(kx < NS / 2 ? kx : kx - NS), jj = T(jy), zz = T(kz);
-              const T inv = n2row[kx] > 0 ? T(1) / sqrt(T(n2row[kx])) : T(0);
-              const T ux = (ii * T(fr.e1[0]) + jj * T(fr.e1[1]) + zz * T(fr.e1[2])) * inv;
-              const T uy = (ii * T(fr.e2[0]) + jj * T(fr.e2[1]) + zz * T(fr.e2[2])) * inv;
-              const T uz = (ii * T(fr.e3[0]) + jj * T(fr.e3[1]) + zz * T(fr.e3[2])) * inv;
               T yr, yi;
-              ylm_frame<T>(sf.yl, sf.ym, ux, uy, uz, yr, yi);
+              ylm_frame<T>(sf.yl, sf.ym, ynrm, urow[kx], urow[NS + kx], urow[2 * NS + kx], yr, yi);
               if (sf.yl & 1) {
                 const T w = sf.ypart ? yr : yi;
                 a = cmk(a.y * w, -a.x * w);
@@ -1317,7 +1334,7 @@ __global__ void k_bispec_finalize(const int* __restrict__ tri, const int* __rest
 __device__ double racah_assoc(int l, int n, double x) {
   double re, im;
   const int an = n < 0 ? -n : n;
-  ylm_frame<double>(l, an, sqrt(fmax(0.0, 1.0 - x * x)), 0.0, x, re, im);
+  ylm_frame<double>(l, an, racah_norm<double>(l, an), sqrt(fmax(0.0, 1.0 - x * x)), 0.0, x, re, im);
   return (n < 0 && (an & 1)) ? -re : re;
 }
 
@@ -1479,7 +1496,7 @@ k_sugi_binsums(const cplx<T>* __restrict__ X0, const cplx<T>* __restrict__ XN, i
 #pragma unroll
           for (int m = 0; m <= l; ++m) {
             T yr, yi;
-            ylm_frame<T>(l, m, ux, uy, uz, yr, yi);
+            ylm_frame<T>(l, m, racah_norm<T>(l, m), ux, uy, uz, yr, yi);
             const T sr = yr, si = -yi;   // y^{m*}
             const T mir = kz > 0 ? ((l & 1) ? T(-1) : T(1)) : T(0);
             const int o = 4 * (l * (l + 1) / 2 + m);
@@ -1642,7 +1659,7 @@ npc_status shell_passes(npc_ctx* ctx, const ShellLaunch& sl, cplx<T>* T1, cplx<T
   const C* tw = (const C*)twp;
   {
     const size_t smem = sizeof(C) * (8 * NS + (size_t)RowGroups<NS, BT>::NBUF * row_pad_len<NS>()) +
-                        sizeof(T) * NS + sizeof(int) * 2 * NS;
+                        sizeof(T) * NS + sizeof(int) * 2 * NS + (sl.has_yw ? sizeof(T) * 3 * NS : 0);
     auto kern = sl.has_yw ? k_shell_x<T, NS, true> : k_shell_x<T, NS, false>;
     NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int nrows = (sl.Kmax + 1) * (2 * sl.Kmax + 1);
