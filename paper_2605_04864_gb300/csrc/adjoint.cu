@@ -415,19 +415,18 @@ k_adj_y_fwd(const cplx<T>* __restrict__ T2, const AFieldTable* __restrict__ ftp,
   }
 }
 
-enum { ZMODE_CUBE = 0, ZMODE_SQUARE_FWD = 1, ZMODE_WRITE = 2 };
+enum { ZMODE_CUBE = 0, ZMODE_SQUARE_FWD = 1, ZMODE_WRITE = 2 };   // WRITE: k_adj_z_write
 
 // z columns of two real fields a, b (b may be absent): inverse transform of
 //   c(kz) = A(kz) + i B(kz),  c(n - kz) = conj A(kz) + i conj B(kz)  (kz <= K_a resp. K_b)
 // gives F_a = Re c(z), F_b = Im c(z).  Then, per mode:
 //   CUBE        per-block float64 sums of F_a^3 and F_b^3 -> cube[field][block];
 //   SQUARE_FWD  forward transform of F_a^2 + i F_b^2, split into the two half spectra and written
-//               back in place for kz <= K_a, K_b;
-//   WRITE       F_a written to the real mesh out[z][y][x].
+//               back in place for kz <= K_a, K_b.
 template <typename T, int N>
 __global__ void __launch_bounds__(ACol<N>::THREADS)
 k_adj_z(cplx<T>* __restrict__ T2, const AFieldTable* __restrict__ ftp, const int2* __restrict__ pairs, int mode,
-        const cplx<T>* __restrict__ tw_g, double* __restrict__ cube, T* __restrict__ out) {
+        const cplx<T>* __restrict__ tw_g, double* __restrict__ cube) {
   using C = cplx<T>;
   constexpr int TX = ACol<N>::TX;
   constexpr int TPF = N / 8;
@@ -435,7 +434,7 @@ k_adj_z(cplx<T>* __restrict__ T2, const AFieldTable* __restrict__ ftp, const int
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* work = tw + N;
-  double* red = reinterpret_cast<double*>(work + N * TX);  // [2][NT/32]
+  T* red = reinterpret_cast<T*>(work);   // [2][NT], once the transform is done with it (2 NT <= N TX)
   const int tid = threadIdx.x;
   const int c = tid % TX, t = tid / TX;
   for (int i = tid; i < N; i += blockDim.x) tw[i] = tw_g[i];
@@ -463,12 +462,6 @@ k_adj_z(cplx<T>* __restrict__ T2, const AFieldTable* __restrict__ ftp, const int
   }
   __syncthreads();
   fft_block<N, +1>(v, t, tw, ColView<C>{work + c, TX});
-  if (mode == ZMODE_WRITE) {
-    T* o = out + cell0;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) o[(size_t)(t + q * TPF) * plane] = v[q].x;
-    return;
-  }
   if (mode == ZMODE_CUBE) {
     T sa = T(0), sb = T(0);
 #pragma unroll
@@ -476,28 +469,21 @@ k_adj_z(cplx<T>* __restrict__ T2, const AFieldTable* __restrict__ ftp, const int
       sa += v[q].x * v[q].x * v[q].x;
       sb += v[q].y * v[q].y * v[q].y;
     }
-    double da = (double)sa, db = (double)sb;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      da += __shfl_down_sync(0xffffffffu, da, o);
-      db += __shfl_down_sync(0xffffffffu, db, o);
-    }
-    const int lane = tid & 31, w = tid >> 5;
-    if (lane == 0) {
-      red[w] = da;
-      red[NT / 32 + w] = db;
-    }
+    // the block's float sums in float64 by one warp per field, in a fixed order: a shuffle tree in float64
+    // by every warp would take five times the float64 adds, which are scarce on this part
     __syncthreads();
-    if (tid == 0) {
-      double ra = 0, rb = 0;
-      for (int k = 0; k < NT / 32; ++k) {
-        ra += red[k];
-        rb += red[NT / 32 + k];
-      }
+    red[tid] = sa;
+    red[NT + tid] = sb;
+    __syncthreads();
+    const int lane = tid & 31;
+    for (int w = tid >> 5; w < 2; w += NT / 32) {
+      double d = 0.0;
+      for (int k = lane; k < NT; k += 32) d += (double)red[w * NT + k];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+      const int f = w ? pr.y : pr.x;
       const size_t nblk = (size_t)gridDim.x * gridDim.y;
-      const size_t blk = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
-      cube[(size_t)pr.x * nblk + blk] = ra;
-      if (hasb) cube[(size_t)pr.y * nblk + blk] = rb;
+      if (lane == 0 && f >= 0) cube[(size_t)f * nblk + (size_t)blockIdx.y * gridDim.x + blockIdx.x] = d;
     }
     return;
   }
@@ -516,6 +502,61 @@ k_adj_z(cplx<T>* __restrict__ T2, const AFieldTable* __restrict__ ftp, const int
     if (kz <= Kb) {
       const C d = csub(z1, z2);
       B[(size_t)kz * plane] = cmk(T(0.5) * d.y, T(-0.5) * d.x);
+    }
+  }
+}
+
+template <int N> struct AWrite {   // column pairs per CTA
+  static constexpr int TX = N >= 512 || N % 32 ? 8 : 16;
+  static constexpr int THREADS = TX * N / 8;
+};
+
+// The real mesh of one field: two neighbouring x columns share one inverse transform, c(kz) = A(kz, x) +
+// i A(kz, x + 1), whose real and imaginary parts are the two columns (half the transforms of one column
+// each).  grid = (N / (2 TX), N).
+template <typename T, int N>
+__global__ void __launch_bounds__(AWrite<N>::THREADS)
+k_adj_z_write(const cplx<T>* __restrict__ T2, const AFieldTable* __restrict__ ftp, const cplx<T>* __restrict__ tw_g,
+              T* __restrict__ out, int aligned) {
+  using C = cplx<T>;
+  constexpr int TX = AWrite<N>::TX;
+  constexpr int TPF = N / 8;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* tw = reinterpret_cast<C*>(smem_raw);
+  C* work = tw + N;
+  const int tid = threadIdx.x;
+  const int c = tid % TX, t = tid / TX;
+  for (int i = tid; i < N; i += blockDim.x) tw[i] = tw_g[i];
+  const AField fa = ftp->f[0];
+  const int K = fa.K;
+  const size_t plane = (size_t)N * N;
+  const size_t cell0 = (size_t)blockIdx.y * N + (blockIdx.x * TX + c) * 2;
+  const C* A = T2 + fa.off2 + cell0;
+  C v[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int zi = t + q * TPF;
+    C a = cmk(T(0), T(0)), b = a;
+    if (zi <= K) {
+      a = A[(size_t)zi * plane];
+      b = A[(size_t)zi * plane + 1];
+    } else if (N - zi <= K) {
+      a = cconj(A[(size_t)(N - zi) * plane]);
+      b = cconj(A[(size_t)(N - zi) * plane + 1]);
+    }
+    v[q] = cmk(a.x - b.y, a.y + b.x);
+  }
+  __syncthreads();
+  fft_block<N, +1>(v, t, tw, ColPadView<C, TX, true>{work + c});
+  T* o = out + cell0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const size_t zo = (size_t)(t + q * TPF) * plane;
+    if (aligned) {
+      *reinterpret_cast<C*>(o + zo) = v[q];
+    } else {
+      o[zo] = v[q].x;
+      o[zo + 1] = v[q].y;
     }
   }
 }
@@ -800,21 +841,32 @@ npc_status shell_pass(npc_ctx* ctx, const AFieldTable& ft, const std::string& ta
   }
   NPC_TRY(stage_mark(ctx, "shell_y_inv"));
   {
-    const size_t zsmem = csmem + sizeof(double) * 2 * (ACol<NS>::THREADS / 32);
+    if (mode == ZMODE_WRITE) {
+      constexpr int WTX = AWrite<NS>::TX;
+      static_assert(NS % (2 * WTX) == 0, "column pairs must tile the mesh");
+      const size_t wsmem = sizeof(C) * (NS + (size_t)col_rows<NS, WTX>() * WTX);
+      auto kern = k_adj_z_write<T, NS>;
+      NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem));
+      kern<<<dim3(NS / (2 * WTX), NS), AWrite<NS>::THREADS, wsmem, ctx->stream>>>(T2, dft, tw, out,
+                                                                               (uintptr_t)out % sizeof(C) == 0);
+      NPC_LAUNCH(ctx);
+      NPC_TRY(stage_mark(ctx, "grad_z_inv"));
+      return NPC_OK;
+    }
     auto kern = k_adj_z<T, NS>;
-    NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zsmem));
+    NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem));
     double* cube = nullptr;
     const size_t nblk = (size_t)(NS / TX) * NS;
     if (mode == ZMODE_CUBE) NPC_TRY(ws_get(ctx, "adj.cube", sizeof(double) * nblk * t.nf, (void**)&cube));
-    kern<<<dim3(NS / TX, NS, (unsigned)pairs.size()), ACol<NS>::THREADS, zsmem, ctx->stream>>>(T2, dft, dpairs, mode,
-                                                                                             tw, cube, out);
+    kern<<<dim3(NS / TX, NS, (unsigned)pairs.size()), ACol<NS>::THREADS, csmem, ctx->stream>>>(T2, dft, dpairs, mode,
+                                                                                             tw, cube);
     NPC_LAUNCH(ctx);
     if (mode == ZMODE_CUBE) {
       k_adj_cube_reduce<<<t.nf, 256, 0, ctx->stream>>>(cube, nblk, cube_sums);
       NPC_LAUNCH(ctx);
     }
   }
-  NPC_TRY(stage_mark(ctx, mode == ZMODE_WRITE ? "grad_z_inv" : (mode == ZMODE_CUBE ? "shell_z_cube" : "shell_z_sq_fwd")));
+  NPC_TRY(stage_mark(ctx, mode == ZMODE_CUBE ? "shell_z_cube" : "shell_z_sq_fwd"));
   if (mode != ZMODE_SQUARE_FWD) return NPC_OK;
   {
     auto kern = k_adj_y_fwd<T, NS>;

@@ -411,7 +411,7 @@ struct LosFrame {
 
 // Power-basis coefficients of d^m L_l/dmu^m for 0 <= m <= l <= 4 (all exact in float), entry [l][m][j] the
 // factor of mu^j, and the Racah norms (-1)^m sqrt((l-m)!/(l+m)!), as tables of both types: formed per
-// element in float64 they cost more than the transforms (x pass of the TripoSH shells 513 -> 190 us at
+// element in float64 they cost more than the transforms (x pass of the TripoSH shells 641 -> 324 us at
 // 256^3), float64 conversions and arithmetic being scarce on this part.
 #define NPC_DLEG                                                                                       \
   {{{1}},                                                                                              \
@@ -650,7 +650,7 @@ __host__ __device__ __forceinline__ size_t rf_index(int field, int64_t cell, int
 // order as unsigned integers; a NaN orders above every finite value)
 template <int THREADS>
 __device__ __forceinline__ void block_absmax(unsigned m, unsigned* red, unsigned* fmax) {
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  m = __reduce_max_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -856,17 +856,24 @@ k_triple(const float* __restrict__ R, const TripleArgs A, const int* __restrict_
   for (int64_t c0 = beg; c0 < end; c0 += TRI_CHUNK) {
     const int nc = (int)((end - c0) < (int64_t)TRI_CHUNK ? (end - c0) : (int64_t)TRI_CHUNK);
     __syncthreads();
-    // one 128-cell row of a staged field per warp and step: a 16-byte load per lane, the row's
-    // rotation undone on the store (nc is a multiple of RCH: ncell is)
+    // one 128-cell row of a staged field per warp and step, 16 bytes per lane copied without passing
+    // through registers, so that all of a warp's rows are in flight together (loaded and stored one by
+    // one their latencies added up: 105 us per TripoSH launch at 256^3); the row's rotation is undone by
+    // the destination (nc is a multiple of RCH: ncell is)
     for (int rw = warp; rw < A.nstage * (TRI_CHUNK / RCH); rw += TRI_WARPS) {
       const int sl = rw / (TRI_CHUNK / RCH), half = rw % (TRI_CHUNK / RCH);
       const int field = A.stage_field[sl], rot = rf_rot(field);
       const int cl = (lane * 4 - rot) & (RCH - 1);   // logical cell of the lane's first value
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (half * RCH < nc)
-        v = *reinterpret_cast<const float4*>(R + (((size_t)(c0 / RCH) + half) * A.nfield_r + field) * RCH + lane * 4);
-      *reinterpret_cast<float4*>(stage + (size_t)sl * TRI_SPAD + half * RCH + cl) = v;
+      float* dst = stage + (size_t)sl * TRI_SPAD + half * RCH + cl;
+      if (half * RCH < nc) {
+        const float* src = R + (((size_t)(c0 / RCH) + half) * A.nfield_r + field) * RCH + lane * 4;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                     : "memory");
+      } else {
+        *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     constexpr int KPW = SK ? TRI_CHUNK / TRI_WARPS : TRI_CHUNK;   // cells of the chunk per warp
     const int kbeg = SK ? warp * KPW : 0;
@@ -883,24 +890,27 @@ k_triple(const float* __restrict__ R, const TripleArgs A, const int* __restrict_
         split_tf32(v0, bh[nt][0], bl[nt][0]);
         split_tf32(v1, bh[nt][1], bl[nt][1]);
       }
+      uint32_t ah[TRI_MT][4], al[TRI_MT][4];
 #pragma unroll
       for (int mt = 0; mt < TRI_MT; ++mt) {
-        uint32_t ah[4], al[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int h = q & 1;
           const int kc = kk + t + ((q >> 1) ? 4 : 0);
           float e = 0.f;
           if (sa[mt][h] >= 0) e = stage[(size_t)sa[mt][h] * TRI_SPAD + kc] * stage[(size_t)sb[mt][h] * TRI_SPAD + kc];
-          split_tf32(e, ah[q], al[q]);
-        }
-#pragma unroll
-        for (int nt = 0; nt < TRI_NT; ++nt) {
-          mma_tf32(d[mt][nt], ah, bh[nt][0], bh[nt][1]);
-          mma_tf32(d[mt][nt], ah, bl[nt][0], bl[nt][1]);
-          mma_tf32(d[mt][nt], al, bh[nt][0], bh[nt][1]);
+          split_tf32(e, ah[mt][q], al[mt][q]);
         }
       }
+      // per accumulator hi hi, hi lo, lo hi; tile by tile within each, so that successive instructions
+      // do not wait for one another's accumulator
+#pragma unroll
+      for (int s = 0; s < 3; ++s)
+#pragma unroll
+        for (int mt = 0; mt < TRI_MT; ++mt)
+#pragma unroll
+          for (int nt = 0; nt < TRI_NT; ++nt)
+            mma_tf32(d[mt][nt], s == 2 ? al[mt] : ah[mt], s == 1 ? bl[nt][0] : bh[nt][0], s == 1 ? bl[nt][1] : bh[nt][1]);
     }
     if (++nchunk == TRI_FLUSH || c0 + TRI_CHUNK >= end) {
       nchunk = 0;

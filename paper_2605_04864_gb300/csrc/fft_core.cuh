@@ -99,6 +99,20 @@ template <typename C> struct RowView {
   template <int Ns> __device__ __forceinline__ C get(int n) const { return p[pos<Ns>(n)]; }
   __device__ __forceinline__ RowView sub(int off) const { return RowView{p + idx(off)}; }
 };
+// Padded column exchange: with fewer than 16 columns a 16-lane access covers several rows, and after
+// span 1 thread t writes row 8 t + r, a multiple of the banks apart; one pad row per 8 separates them.
+template <typename C, int TX, bool PK> struct ColPadView {
+  static constexpr bool PACKED = PK;
+  C* p;
+  __device__ __forceinline__ void st(int n, C v) const { p[n * TX] = v; }
+  __device__ __forceinline__ C ld(int n) const { return p[n * TX]; }
+  template <int Ns> __device__ __forceinline__ static int row(int n) { return TX < 16 && Ns == 1 ? n + (n >> 3) : n; }
+  template <int Ns> __device__ __forceinline__ void put(int n, C v) const { p[row<Ns>(n) * TX] = v; }
+  template <int Ns> __device__ __forceinline__ C get(int n) const { return p[row<Ns>(n) * TX]; }
+  __device__ __forceinline__ ColPadView sub(int off) const { return ColPadView{p + (off + (TX < 16 ? off >> 3 : 0)) * TX}; }
+};
+template <int N, int TX> __host__ __device__ constexpr int col_rows() { return TX < 16 ? N + N / 8 : N; }
+
 template <int N> __host__ __device__ constexpr int row_pad_len() { return N + N / 8; }
 
 // Supported transform lengths: powers of two >= 16, and three times a power of two >= 48.

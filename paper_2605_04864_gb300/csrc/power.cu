@@ -56,8 +56,9 @@ template <int N> struct SingleCfg {   // column pairs per CTA: 2 TX divides N, T
   static constexpr int THREADS = TX * N / 8;
 };
 
-template <typename T, int N>
-__global__ void __launch_bounds__(SingleCfg<N>::THREADS)
+// The two columns' values are neighbours in memory: one 8-byte load when the mesh is aligned to it (VEC).
+template <typename T, int N, bool VEC>
+__global__ void __launch_bounds__(SingleCfg<N>::THREADS, (sizeof(T) == 4 && SingleCfg<N>::THREADS == 512 ? 2 : 1))
 k_fwd_z_single(const T* __restrict__ mesh, cplx<T>* __restrict__ half, const cplx<T>* __restrict__ tw_g, int KZ) {
   using C = cplx<T>;
   constexpr int TX = SingleCfg<N>::TX;
@@ -74,10 +75,11 @@ k_fwd_z_single(const T* __restrict__ mesh, cplx<T>* __restrict__ half, const cpl
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const size_t zoff = (size_t)(t + q * TPF) * N * N;
-    v[q] = cmk(col[zoff], col[zoff + 1]);
+    if constexpr (VEC) v[q] = *reinterpret_cast<const C*>(col + zoff);
+    else v[q] = cmk(col[zoff], col[zoff + 1]);
   }
   __syncthreads();
-  fft_block<N, -1>(v, t, tw, ColView<C>{work + c, TX});
+  fft_block<N, -1>(v, t, tw, ColPadView<C, TX, true>{work + c});
 #pragma unroll
   for (int q = 0; q < 8; ++q) work[(t + q * TPF) * TX + c] = v[q];
   __syncthreads();
@@ -190,20 +192,6 @@ __device__ __forceinline__ void any_signal(T (&sv)[8], const Signal& sg, const T
 #undef NPC_S
 }
 
-// Padded column exchange: with fewer than 16 columns a 16-lane access covers several rows, and after
-// span 1 thread t writes row 8 t + r, a multiple of the banks apart; one pad row per 8 separates them.
-template <typename C, int TX, bool PK> struct ColPadView {
-  static constexpr bool PACKED = PK;
-  C* p;
-  __device__ __forceinline__ void st(int n, C v) const { p[n * TX] = v; }
-  __device__ __forceinline__ C ld(int n) const { return p[n * TX]; }
-  template <int Ns> __device__ __forceinline__ static int row(int n) { return TX < 16 && Ns == 1 ? n + (n >> 3) : n; }
-  template <int Ns> __device__ __forceinline__ void put(int n, C v) const { p[row<Ns>(n) * TX] = v; }
-  template <int Ns> __device__ __forceinline__ C get(int n) const { return p[row<Ns>(n) * TX]; }
-  __device__ __forceinline__ ColPadView sub(int off) const { return ColPadView{p + (off + (TX < 16 ? off >> 3 : 0)) * TX}; }
-};
-template <int N, int TX> constexpr int col_rows() { return TX < 16 ? N + N / 8 : N; }
-
 // float: occupancy of the register counts this kernel needs (64 at 512 threads, at most 80 otherwise)
 template <typename T, int N> constexpr int zpass_min_blocks() {
   return sizeof(T) == 4 ? 65536 / (ColCfg<N>::THREADS * (ColCfg<N>::THREADS == 512 ? 64 : 80)) : 1;
@@ -211,7 +199,7 @@ template <typename T, int N> constexpr int zpass_min_blocks() {
 
 // Coordinates of the grid points from the observer, tab[axis][phase][n], formed in float64 and rounded
 // once (phase b lies half a cell lower): the weighted passes look them up instead of forming them per
-// thread, since float64 arithmetic is scarce on this part (y pass at 512^3: 10.1 ms with, 5.5 without).
+// thread, since float64 arithmetic is scarce on this part (y pass at 512^3: 10.1 ms with, 6.0 without).
 template <typename T>
 __global__ void k_axis_coords(const Geom g, T* __restrict__ tab) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 6 * g.n; i += gridDim.x * blockDim.x) {
@@ -1038,8 +1026,8 @@ npc_status fwd_impl(npc_ctx* ctx, const PowerPlan& plan, const Geom& g, const vo
   if (single) {
     constexpr int STX = SingleCfg<N>::TX;
     static_assert(N % (2 * STX) == 0, "column pairs must tile the mesh");
-    const size_t ssmem = sizeof(C) * (N + N * STX);
-    auto kern = k_fwd_z_single<T, N>;
+    const size_t ssmem = sizeof(C) * (N + col_rows<N, STX>() * STX);
+    auto kern = (uintptr_t)mesh_a % sizeof(C) == 0 ? k_fwd_z_single<T, N, true> : k_fwd_z_single<T, N, false>;
     NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem));
     kern<<<dim3(N / (2 * STX), N), SingleCfg<N>::THREADS, ssmem, ctx->stream>>>((const T*)mesh_a, (C*)half, tw, KZ);
   } else {
