@@ -104,7 +104,8 @@ npc_status run_item(npc_ctx* sub, const Item& I, uint32_t ell_mask, int prec, do
   NPC_TRY(launch_catalog_scalars(sub, d, rp, it.mesh.box, sc));
   NPC_TRY(power_core(sub, it.mesh, d, rp, it.power_bins, ell_mask, 0, prec, sc, out + I.off_p));
   if (it.bispec_bins.nbins > 0)
-    NPC_TRY(run_bispectrum(sub, it.mesh, it.bispec_bins, 1, 0, 1, prec, d, rp, sc, out + I.off_b, I.len_b));
+    NPC_TRY(run_bispectrum(sub, it.mesh, it.bispec_bins, 1, 0, 1, prec, d, rp, sc, out + I.off_b, I.len_b,
+                           true));
   return NPC_OK;
 }
 

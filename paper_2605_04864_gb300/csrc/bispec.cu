@@ -1720,7 +1720,7 @@ template <typename T, int N>
 npc_status bispec_impl(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins& kb, int scoc_mask, int tripo_mask,
                        int shot, const DevCatalog& d, const DevCatalog* r, double* sc, double* dev_out,
                        int64_t out_len, const SugiReq* sug = nullptr, const CrossReq* crq = nullptr,
-                       double* sc_own = nullptr) {
+                       double* sc_own = nullptr, bool painted = false) {
   // multi-tracer bispectra (crq): `sc` holds the combined normalisation, `sc_own` tracer 1's own
   // scalars (its FKP field needs its alpha)
   double* const sc_paint = (crq && sc_own) ? sc_own : sc;
@@ -1846,11 +1846,11 @@ npc_status bispec_impl(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins& kb
   C* halfF = (C*)half;
   C* halfN = (C*)((char*)half + halfbytes);
   NPC_TRY(stage_mark(ctx, "alloc"));
-  NPC_TRY(launch_paint(ctx, d, r, m, 1, prec, sc_paint, ma, mb));
+  if (!painted) NPC_TRY(launch_paint(ctx, d, r, m, 1, prec, sc_paint, ma, mb));
   NPC_TRY(stage_mark(ctx, "paint_fold"));
   NPC_TRY(run_forward_transforms(ctx, prec, plan, gfwd, ma, mb, halfF));
   if (shot) {
-    NPC_TRY(launch_paint(ctx, d, r, m, 2, prec, sc, ma, mb));
+    NPC_TRY(launch_paint(ctx, d, r, m, 2, prec, sc, ma, mb, true));   // the FKP mesh's brick sort holds
     NPC_TRY(run_forward_transforms(ctx, prec, planN, gfwdN, ma, mb, halfN));
   }
   NPC_TRY(stage_mark(ctx, "forward_yz"));
@@ -2795,19 +2795,20 @@ npc_status bispec_impl(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins& kb
 template <typename T>
 npc_status bispec_dispatch(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins& kb, int sm, int tm, int shot,
                            const DevCatalog& d, const DevCatalog* r, double* sc, double* out, int64_t len,
-                           const SugiReq* sug = nullptr, const CrossReq* crq = nullptr, double* sc_own = nullptr) {
+                           const SugiReq* sug = nullptr, const CrossReq* crq = nullptr, double* sc_own = nullptr,
+                           bool painted = false) {
   switch (m.n) {
-    case 16: return bispec_impl<T, 16>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own);
-    case 32: return bispec_impl<T, 32>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own);
-    case 64: return bispec_impl<T, 64>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own);
-    case 128: return bispec_impl<T, 128>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own);
-    case 256: return bispec_impl<T, 256>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own);
-    case 48: return bispec_impl<T, 48>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own);
-    case 96: return bispec_impl<T, 96>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own);
-    case 192: return bispec_impl<T, 192>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own);
+    case 16: return bispec_impl<T, 16>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own, painted);
+    case 32: return bispec_impl<T, 32>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own, painted);
+    case 64: return bispec_impl<T, 64>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own, painted);
+    case 128: return bispec_impl<T, 128>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own, painted);
+    case 256: return bispec_impl<T, 256>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own, painted);
+    case 48: return bispec_impl<T, 48>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own, painted);
+    case 96: return bispec_impl<T, 96>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own, painted);
+    case 192: return bispec_impl<T, 192>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own, painted);
   }
   if constexpr (sizeof(T) == 4) {
-    if (m.n == 512) return bispec_impl<T, 512>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own);
+    if (m.n == 512) return bispec_impl<T, 512>(ctx, m, kb, sm, tm, shot, d, r, sc, out, len, sug, crq, sc_own, painted);
   }
   return set_err(ctx, NPC_ERR_UNSUPPORTED, "bispectrum mesh size %d not supported at this precision", m.n);
 }
@@ -2816,10 +2817,12 @@ npc_status bispec_dispatch(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins
 
 npc_status run_bispectrum(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins& kb, int scoc_mask, int tripo_mask,
                           int shot, int prec, const DevCatalog& d, const DevCatalog* r, double* sc, double* out,
-                          int64_t len) {
+                          int64_t len, bool painted) {
   if (prec == NPC_PREC_FP64)
-    return bispec_dispatch<double>(ctx, m, kb, scoc_mask, tripo_mask, shot, d, r, sc, out, len);
-  return bispec_dispatch<float>(ctx, m, kb, scoc_mask, tripo_mask, shot, d, r, sc, out, len);
+    return bispec_dispatch<double>(ctx, m, kb, scoc_mask, tripo_mask, shot, d, r, sc, out, len, nullptr, nullptr, nullptr,
+                                   painted);
+  return bispec_dispatch<float>(ctx, m, kb, scoc_mask, tripo_mask, shot, d, r, sc, out, len, nullptr, nullptr, nullptr,
+                                painted);
 }
 
 npc_status run_bispectrum_cross(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins& kb, int scoc_mask,

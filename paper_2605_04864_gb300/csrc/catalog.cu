@@ -891,7 +891,7 @@ npc_status launch_tiles(npc_ctx* ctx, const void* rec, const uint32_t* meta, con
 
 template <int ASSIGN, typename T>
 npc_status paint_impl(npc_ctx* ctx, const DevCatalog& d, const DevCatalog* r, const npc_mesh_spec& m,
-                      int weight_power, const double* sc, void* mesh_a, void* mesh_b) {
+                      int weight_power, const double* sc, void* mesh_a, void* mesh_b, bool sorted) {
   PaintGeo g;
   g.n = m.n;
   g.bs = (m.n >= 48 && m.n % 16 == 0) ? 16 : m.n / 4;   // 16 for every size >= 48; 4, 8 at n = 16, 32
@@ -924,7 +924,6 @@ npc_status paint_impl(npc_ctx* ctx, const DevCatalog& d, const DevCatalog* r, co
   NPC_TRY(ws_get(ctx, "paint.meta", sizeof(uint32_t) * std::max<int64_t>(ntot, 1), (void**)&meta));
   NPC_TRY(ws_get(ctx, "paint.rec", sizeof(typename RecOf<T>::type) * std::max<int64_t>(ntot, 1), &rec));
   NPC_TRY(ws_get(ctx, "paint.tiles", sizeof(T) * ts3 * nbricks * nphase, &tiles));
-  NPC_CUDA(ctx, cudaMemsetAsync(count, 0, sizeof(int) * nbricks * COUNT_STRIDE, ctx->stream));
   // data and randoms share the brick counters (ranks continue): one launch each for counting and for
   // scattering when both catalogues have one type
   const bool joint = r && r->dtype == d.dtype;
@@ -933,18 +932,21 @@ npc_status paint_impl(npc_ctx* ctx, const DevCatalog& d, const DevCatalog* r, co
     if (r && !joint) NPC_TRY(run(r, (const DevCatalog*)nullptr, d.n, true));
     return NPC_OK;
   };
-  NPC_TRY(each([&](const DevCatalog* a, const DevCatalog* b, int64_t off, bool) {
-    return a->dtype == 1 ? paint_count<double>(ctx, cat_pair<double>(a, b), g, nbricks, count, brick + off, rank + off)
-                         : paint_count<float>(ctx, cat_pair<float>(a, b), g, nbricks, count, brick + off, rank + off);
-  }));
-  const int chunks = nbricks / SCAN_CHUNK + 1;   // of the nbricks + 1 entries
-  int* total;
-  NPC_TRY(ws_get(ctx, "paint.total", sizeof(int) * chunks, (void**)&total));
-  k_scan<<<chunks, SCAN_THREADS, 0, ctx->stream>>>(count, nbricks, start, total);
-  NPC_LAUNCH(ctx);
-  if (chunks > 1) {
-    k_scan_add<<<chunks, SCAN_THREADS, 0, ctx->stream>>>(total, nbricks, start);
+  if (!sorted) {
+    NPC_CUDA(ctx, cudaMemsetAsync(count, 0, sizeof(int) * nbricks * COUNT_STRIDE, ctx->stream));
+    NPC_TRY(each([&](const DevCatalog* a, const DevCatalog* b, int64_t off, bool) {
+      return a->dtype == 1 ? paint_count<double>(ctx, cat_pair<double>(a, b), g, nbricks, count, brick + off, rank + off)
+                           : paint_count<float>(ctx, cat_pair<float>(a, b), g, nbricks, count, brick + off, rank + off);
+    }));
+    const int chunks = nbricks / SCAN_CHUNK + 1;   // of the nbricks + 1 entries
+    int* total;
+    NPC_TRY(ws_get(ctx, "paint.total", sizeof(int) * chunks, (void**)&total));
+    k_scan<<<chunks, SCAN_THREADS, 0, ctx->stream>>>(count, nbricks, start, total);
     NPC_LAUNCH(ctx);
+    if (chunks > 1) {
+      k_scan_add<<<chunks, SCAN_THREADS, 0, ctx->stream>>>(total, nbricks, start);
+      NPC_LAUNCH(ctx);
+    }
   }
   NPC_TRY(stage_mark(ctx, "paint_count"));
   NPC_TRY(each([&](const DevCatalog* a, const DevCatalog* b, int64_t off, bool rf) {
@@ -1036,16 +1038,17 @@ npc_status launch_catalog_scalars(npc_ctx* ctx, const DevCatalog& d, const DevCa
 }
 
 npc_status launch_paint(npc_ctx* ctx, const DevCatalog& d, const DevCatalog* r, const npc_mesh_spec& m,
-                        int weight_power, int prec, const double* dev_scalars, void* mesh_a, void* mesh_b) {
+                        int weight_power, int prec, const double* dev_scalars, void* mesh_a, void* mesh_b,
+                        bool sorted) {
   const bool any_double = d.dtype == 1 || (r && r->dtype == 1);
   if (prec == NPC_PREC_FP64) {
-    if (m.assign == 2) return paint_impl<2, double>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b);
-    return paint_impl<3, double>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b);
+    if (m.assign == 2) return paint_impl<2, double>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b, sorted);
+    return paint_impl<3, double>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b, sorted);
   }
   // records keep the fraction s - floor(s) (< 1) in float32 in the mixed path
   (void)any_double;
-  if (m.assign == 2) return paint_impl<2, float>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b);
-  return paint_impl<3, float>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b);
+  if (m.assign == 2) return paint_impl<2, float>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b, sorted);
+  return paint_impl<3, float>(ctx, d, r, m, weight_power, dev_scalars, mesh_a, mesh_b, sorted);
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -304,9 +304,10 @@ npc_status launch_cross3_scalars(npc_ctx* ctx, const double* s1, const double* s
 
 // Paint the FKP field (weight_power 1) or the N-field (2) on 1 or 2 interlacing phases.
 // meshes: nphase pointers to n^3 arrays of T (layout [z][y][x]).
+// sorted: the call's last launch_paint took the same catalogues and mesh, so its brick sort still holds.
 npc_status launch_paint(npc_ctx* ctx, const DevCatalog& d, const DevCatalog* r, const npc_mesh_spec& m,
                         int weight_power, int prec, const double* dev_scalars, void* mesh_a,
-                        void* mesh_b);
+                        void* mesh_b, bool sorted = false);
 
 // ---------------------------------------------------------------------------------------------
 // Power spectrum passes (power.cu)
@@ -351,9 +352,11 @@ npc_status get_twiddles(npc_ctx* ctx, int n, int prec, const void** out);
 // ---------------------------------------------------------------------------------------------
 // Bispectrum (bispec.cu)
 // ---------------------------------------------------------------------------------------------
+// painted: the FKP meshes of these catalogues, mesh and precision lie in the workspace (painted by power_core
+// just before, on the same stream)
 npc_status run_bispectrum(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins& kb, int scoc_mask, int tripo_mask,
                           int shot, int prec, const DevCatalog& d, const DevCatalog* r, double* sc, double* out,
-                          int64_t len);
+                          int64_t len, bool painted = false);
 int64_t bispec_counts(const npc_kbins& kb, int64_t* ntri, int64_t* npair);
 
 // Sugiyama TripoSH multipoles B_{l1 l2 L} requested from the bispectrum pipeline (global line of
