@@ -770,8 +770,8 @@ int bin_radius(double box, const npc_kbins& kb, int b, int KM) {
 template <typename T, int N>
 npc_status row_grid(npc_ctx* ctx, const void* kern, size_t smem, int nrows, int rows_per_block, int* grid) {
   int per_sm = 0;
-  NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  NPC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, AT, smem));
+  NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
+  NPC_TRY(ctas_per_sm(ctx, (const void*)kern, AT, smem, &per_sm));
   if (per_sm < 1) return set_err(ctx, NPC_ERR_UNSUPPORTED, "row kernel does not fit on an SM (%zu B smem)", smem);
   const int need = (nrows + rows_per_block - 1) / rows_per_block;
   *grid = std::max(1, std::min(need, per_sm * ctx->num_sms));
@@ -832,7 +832,7 @@ npc_status shell_pass(npc_ctx* ctx, const AFieldTable& ft, const std::string& ta
   const size_t csmem = sizeof(C) * (NS + (size_t)NS * TX);
   {
     auto kern = k_adj_y_inv<T, NS>;
-    NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem));
+    NPC_TRY(allow_smem(ctx, (const void*)kern, csmem));
     for (size_t p0 = 0; p0 < planes.size(); p0 += 65535) {
       const int np = (int)std::min<size_t>(65535, planes.size() - p0);
       kern<<<dim3(NS / TX, np), ACol<NS>::THREADS, csmem, ctx->stream>>>(T1, dft, dplanes + p0, tw, T2);
@@ -846,7 +846,7 @@ npc_status shell_pass(npc_ctx* ctx, const AFieldTable& ft, const std::string& ta
       static_assert(NS % (2 * WTX) == 0, "column pairs must tile the mesh");
       const size_t wsmem = sizeof(C) * (NS + (size_t)col_rows<NS, WTX>() * WTX);
       auto kern = k_adj_z_write<T, NS>;
-      NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem));
+      NPC_TRY(allow_smem(ctx, (const void*)kern, wsmem));
       kern<<<dim3(NS / (2 * WTX), NS), AWrite<NS>::THREADS, wsmem, ctx->stream>>>(T2, dft, tw, out,
                                                                                (uintptr_t)out % sizeof(C) == 0);
       NPC_LAUNCH(ctx);
@@ -854,7 +854,7 @@ npc_status shell_pass(npc_ctx* ctx, const AFieldTable& ft, const std::string& ta
       return NPC_OK;
     }
     auto kern = k_adj_z<T, NS>;
-    NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem));
+    NPC_TRY(allow_smem(ctx, (const void*)kern, csmem));
     double* cube = nullptr;
     const size_t nblk = (size_t)(NS / TX) * NS;
     if (mode == ZMODE_CUBE) NPC_TRY(ws_get(ctx, "adj.cube", sizeof(double) * nblk * t.nf, (void**)&cube));
@@ -870,7 +870,7 @@ npc_status shell_pass(npc_ctx* ctx, const AFieldTable& ft, const std::string& ta
   if (mode != ZMODE_SQUARE_FWD) return NPC_OK;
   {
     auto kern = k_adj_y_fwd<T, NS>;
-    NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem));
+    NPC_TRY(allow_smem(ctx, (const void*)kern, csmem));
     for (size_t p0 = 0; p0 < planes.size(); p0 += 65535) {
       const int np = (int)std::min<size_t>(65535, planes.size() - p0);
       kern<<<dim3(NS / TX, np), ACol<NS>::THREADS, csmem, ctx->stream>>>(T2, dft, dplanes + p0, tw, T1);

@@ -26,6 +26,34 @@ std::string slot_name(const npc_ctx* ctx, const std::string& name) {
   return ctx->slot_base ? name + "#" + std::to_string(ctx->slot_base) : name;
 }
 
+npc_status allow_smem(npc_ctx* ctx, const void* kernel, size_t smem) {
+  if (smem <= 47 * 1024) return NPC_OK;   // (a little of the 48 KB may be static)
+  auto it = ctx->kernel_smem.find(kernel);
+  if (it == ctx->kernel_smem.end()) {
+    int most = 0;
+    cudaFuncAttributes a;
+    NPC_CUDA(ctx, cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
+    NPC_CUDA(ctx, cudaFuncGetAttributes(&a, kernel));
+    most -= (int)a.sharedSizeBytes;
+    NPC_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    it = ctx->kernel_smem.emplace(kernel, (size_t)most).first;
+  }
+  if (smem > it->second)
+    return set_err(ctx, NPC_ERR_CUDA, "a kernel needs %zu bytes of shared memory, an SM gives %zu", smem, it->second);
+  return NPC_OK;
+}
+
+npc_status ctas_per_sm(npc_ctx* ctx, const void* kernel, int threads, size_t smem, int* ctas) {
+  const auto key = std::make_tuple(kernel, threads, smem);
+  auto it = ctx->kernel_ctas.find(key);
+  if (it == ctx->kernel_ctas.end()) {
+    NPC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, kernel, threads, smem));
+    it = ctx->kernel_ctas.emplace(key, *ctas).first;
+  }
+  *ctas = it->second;
+  return NPC_OK;
+}
+
 npc_status ws_get(npc_ctx* ctx, const char* name, size_t bytes, void** out) {
   Workspace& w = ctx->ws[name];
   if (bytes == 0) bytes = 16;

@@ -1671,7 +1671,7 @@ npc_status shell_passes(npc_ctx* ctx, const ShellLaunch& sl, cplx<T>* T1, cplx<T
     const size_t smem = sizeof(C) * (8 * NS + (size_t)RowGroups<NS, BT>::NBUF * row_pad_len<NS>()) +
                         sizeof(T) * NS + sizeof(int) * 2 * NS + (sl.has_yw ? sizeof(T) * 3 * NS : 0);
     auto kern = sl.has_yw ? k_shell_x<T, NS, true> : k_shell_x<T, NS, false>;
-    NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
     const int nrows = (sl.Kmax + 1) * (2 * sl.Kmax + 1);
     kern<<<std::min(nrows, ctx->num_sms * 4), BT, smem, ctx->stream>>>(
         (const C*)sl.X, (const C*)sl.XN, (const C*)sl.X2, (const C*)sl.X1, (const C*)sl.X3, (const C*)sl.XB,
@@ -1683,7 +1683,7 @@ npc_status shell_passes(npc_ctx* ctx, const ShellLaunch& sl, cplx<T>* T1, cplx<T
   constexpr int TX = BCol<NS>::TX;
   const size_t smem = sizeof(C) * (NS + (size_t)NS * TX);
   auto ky = k_shell_y<T, NS>;
-  NPC_CUDA(ctx, cudaFuncSetAttribute(ky, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  NPC_TRY(allow_smem(ctx, (const void*)ky, smem));
   for (int p0 = 0; p0 < sl.nplanes; p0 += 65535) {
     const int np_ = std::min(65535, sl.nplanes - p0);
     ky<<<dim3(NS / TX, np_), BCol<NS>::THREADS, smem, ctx->stream>>>(T1, sl.fields, sl.plane_f + p0,
@@ -1691,7 +1691,7 @@ npc_status shell_passes(npc_ctx* ctx, const ShellLaunch& sl, cplx<T>* T1, cplx<T
     NPC_LAUNCH(ctx);
   }
   auto kz = k_shell_z<T, NS>;
-  NPC_CUDA(ctx, cudaFuncSetAttribute(kz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  NPC_TRY(allow_smem(ctx, (const void*)kz, smem));
   kz<<<dim3(NS / TX, NS, sl.nzp), BCol<NS>::THREADS, smem, ctx->stream>>>(T2, sl.fields, sl.za, sl.zb, sl.oa, sl.ob,
                                                                           tw, R, sl.nfield, sl.fmax);
   NPC_LAUNCH(ctx);
@@ -1873,7 +1873,7 @@ npc_status bispec_impl(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins& kb
                           sizeof(T) * (N / 2 + 2);
       if (smem > 227 * 1024) return set_err(ctx, NPC_ERR_UNSUPPORTED, "survey multipoles: mesh too large at this precision");
       auto kern = k_fft_x_assemble_yam<T, N>;
-      NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
       kern<<<grid, BT, smem, ctx->stream>>>(src, nphase, KZ, K2, m.assign, ylm_norm_table(), yc, tw, x0, x1, x2, x3,
                                             comps);
       NPC_LAUNCH(ctx);
@@ -1883,7 +1883,7 @@ npc_status bispec_impl(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins& kb
       const size_t smem =
           sizeof(C) * (2 * N + (size_t)(nphase + RowGroups<N, BT>::NBUF) * row_pad_len<N>()) + sizeof(T) * (N / 2 + 2);
       auto kern = k_fft_x_combine<T, N>;
-      NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
       kern<<<grid, BT, smem, ctx->stream>>>(src, 1, nphase, KZ, K2, m.assign, tw, dst);
       NPC_LAUNCH(ctx);
       return NPC_OK;
@@ -2584,7 +2584,7 @@ npc_status bispec_impl(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins& kb
         kp.runs = (const int*)(tc_tab + P->o_runs);
         kp.gidx = (const int*)(tc_tab + P->o_gidx);
         auto go = [&](auto kern) -> npc_status {
-          NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P->smem));
+          NPC_TRY(allow_smem(ctx, (const void*)kern, P->smem));
           kern<<<dim3(grid, P->groups), P->nt * 128 * tc::PPR + (tc::NBW + 2) * 32, P->smem, ctx->stream>>>(
               (const float*)R, a.ncell, kp, fmax_dev, part, ctx->dev_status, wait_cycles(ctx), P->nbuf);
           return NPC_OK;
@@ -2600,7 +2600,7 @@ npc_status bispec_impl(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins& kb
       auto run = [&](auto kern, int nt) -> npc_status {
         const size_t smem = sizeof(float) * (size_t)a.nstage * TRI_SPAD +
                             sizeof(double) * (size_t)TRI_WARPS * 32 * mt * nt * 4;
-        NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
         kern<<<dim3(grid, groups), TRI_WARPS * 32, smem, ctx->stream>>>(
             (const float*)R, ak, (const int*)(dtab + tp), (const int*)(dtab + trp), part);
         return NPC_OK;
@@ -2612,7 +2612,7 @@ npc_status bispec_impl(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins& kb
         // few rows: all warps on the same two m tiles, each on its own cells
         const size_t smem = sizeof(float) * (size_t)a.nstage * TRI_SPAD + sizeof(double) * (size_t)TRI_WARPS * 32 * 2 * 3 * 4;
         auto kern = k_triple<3, 2, true>;
-        NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
         kern<<<dim3(grid, 1), TRI_WARPS * 32, smem, ctx->stream>>>((const float*)R, ak, (const int*)(dtab + tp),
                                                                    (const int*)(dtab + trp), part);
       } else if (a.ncol <= 24) {

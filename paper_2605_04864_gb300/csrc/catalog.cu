@@ -882,7 +882,7 @@ npc_status launch_tiles(npc_ctx* ctx, const void* rec, const uint32_t* meta, con
                         int nphase, const double* sc, int slot, void* tiles) {
   const size_t smem = tile_smem<T, BS>();
   auto kern = k_paint_brick<ASSIGN, T, BS>;
-  NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
   kern<<<nbricks * nphase, 512, smem, ctx->stream>>>((const typename RecOf<T>::type*)rec, meta, start, nphase, sc,
                                                      slot, (T*)tiles);
   NPC_LAUNCH(ctx);

@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <map>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "../../include/npc.h"
@@ -214,6 +215,8 @@ struct npc_ctx {
   int batch_branches = 0;              // 0: not tuned (default 4)
   std::map<int, int> ytx;              // tuned columns per CTA of the y pass, per (n * 2 + fp64)
   cudaStream_t batch_hub = nullptr;    // stream the batch graphs are captured on and launched from
+  std::map<const void*, size_t> kernel_smem;                            // allow_smem: limit given per kernel
+  std::map<std::tuple<const void*, int, size_t>, int> kernel_ctas;      // ctas_per_sm answers
 };
 
 // default bound of a device-side wait: about one second at the GPU's clock
@@ -256,6 +259,13 @@ npc_status set_err(npc_ctx* ctx, npc_status s, const char* fmt, ...);
     npc_status s_ = (expr);                                                                  \
     if (s_ != NPC_OK) return s_;                                                             \
   } while (0)
+
+// Lets a kernel be launched with `smem` bytes of dynamic shared memory: asked of the runtime once per
+// context and kernel (for the most an SM gives, so that contexts do not undo each other), and not at all
+// up to the 48 KB that need no asking.  A measurement on a small mesh makes dozens of such launches.
+npc_status allow_smem(npc_ctx* ctx, const void* kernel, size_t smem);
+// Resident CTAs per SM of a kernel at this block size and shared memory, looked up once per context.
+npc_status ctas_per_sm(npc_ctx* ctx, const void* kernel, int threads, size_t smem, int* ctas);
 
 // grow-only named device buffer
 npc_status ws_get(npc_ctx* ctx, const char* name, size_t bytes, void** out);

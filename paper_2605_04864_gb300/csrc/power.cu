@@ -906,7 +906,7 @@ npc_status y_pass_tx(npc_ctx* ctx, cplx<T>* data, int nplanes, const cplx<T>* tw
   } else {
     const size_t smem = sizeof(C) * (N + N * TX);
     auto kern = k_fft_cols<T, N, -1, TX>;
-    NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
     for (int p0 = 0; p0 < nplanes; p0 += 65535) {
       const int np = std::min(65535, nplanes - p0);
       kern<<<dim3(N / TX, np), TX * N / 8, smem, ctx->stream>>>(data + (size_t)p0 * N * N, (size_t)N * N, N, tw, p0,
@@ -938,7 +938,7 @@ npc_status y_pass_weighted_tx(npc_ctx* ctx, cplx<T>* half, const SignalList& sl,
   } else {
     const size_t smem = sizeof(C) * (N + col_rows<N, TX>() * TX + N * TX);
     auto kern = k_fft_cols_weighted<T, N, TX>;
-    NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
     const int nplanes = sl.n * KZ;   // at most 32 x 512
     kern<<<dim3(N / TX, nplanes), TX * N / 8, smem, ctx->stream>>>(half, sl, coords, nrm, tw, KZ, row_n2max);
     NPC_LAUNCH(ctx);
@@ -1028,12 +1028,12 @@ npc_status fwd_impl(npc_ctx* ctx, const PowerPlan& plan, const Geom& g, const vo
     static_assert(N % (2 * STX) == 0, "column pairs must tile the mesh");
     const size_t ssmem = sizeof(C) * (N + col_rows<N, STX>() * STX);
     auto kern = (uintptr_t)mesh_a % sizeof(C) == 0 ? k_fwd_z_single<T, N, true> : k_fwd_z_single<T, N, false>;
-    NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem));
+    NPC_TRY(allow_smem(ctx, (const void*)kern, ssmem));
     kern<<<dim3(N / (2 * STX), N), SingleCfg<N>::THREADS, ssmem, ctx->stream>>>((const T*)mesh_a, (C*)half, tw, KZ);
   } else {
     const size_t smem = sizeof(C) * (N + col_rows<N, TX>() * TX) + sizeof(T) * (mesh_b ? 2 : 1) * N * TX;
     auto kern = k_fwd_z<T, N>;
-    NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
     kern<<<dim3(N / TX, N), ColCfg<N>::THREADS, smem, ctx->stream>>>((const T*)mesh_a, (const T*)mesh_b, (C*)half, sl,
                                                                      coords, (T)(g.h * (N / 8)), nrm, tw, KZ);
   }
@@ -1159,9 +1159,9 @@ npc_status contract_impl(npc_ctx* ctx, const PowerPlan& plan, const npc_mesh_spe
     threads /= 2;
   const size_t smem = smem_of(threads);
   auto kern = k_fft_x_contract<T, N, (sizeof(T) == 4 ? 2 : 1)>;
-  NPC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
   int per_sm = 0;
-  NPC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
+  NPC_TRY(ctas_per_sm(ctx, (const void*)kern, threads, smem, &per_sm));
   if (per_sm < 1) return set_err(ctx, NPC_ERR_UNSUPPORTED, "contraction does not fit on an SM (%zu B smem)", smem);
   const int G = threads / XTeam<N>::TPF;
   const int grid = std::min((nitems + G - 1) / G, per_sm * ctx->num_sms);
