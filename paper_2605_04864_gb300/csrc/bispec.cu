@@ -812,8 +812,10 @@ __global__ void __launch_bounds__(TRI_WARPS * 32, TRI_MT == 1 ? 3 : 2)
 k_triple(const float* __restrict__ R, const TripleArgs A, const int* __restrict__ pair_ij,
          const int* __restrict__ row_pair, double* __restrict__ part) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* stage = reinterpret_cast<float*>(smem_raw);                               // [nstage][TRI_SPAD]
-  double* dacc = reinterpret_cast<double*>(stage + (size_t)A.nstage * TRI_SPAD);  // [tid][NACC]
+  // SK: two buffers of half a chunk each, otherwise one of a chunk
+  constexpr int SCELLS = SK ? TRI_CHUNK / 2 : TRI_CHUNK, SPAD = SCELLS + 4;
+  float* stage0 = reinterpret_cast<float*>(smem_raw);                                           // [1 or 2][nstage][SPAD]
+  double* dacc = reinterpret_cast<double*>(stage0 + (size_t)(SK ? 2 : 1) * A.nstage * SPAD);  // [tid][NACC]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
   const int rowbase = SK ? blockIdx.y * TRI_MT * 16 : blockIdx.y * tri_rows<TRI_MT>() + warp * TRI_MT * 16;
@@ -823,7 +825,9 @@ k_triple(const float* __restrict__ R, const TripleArgs A, const int* __restrict_
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int r = rowbase + mt * 16 + g + 8 * h;
-      sa[mt][h] = sb[mt][h] = orow[mt][h] = -1;
+      // rows past the last repeat slot 0 (no branch per product; their sums are not written)
+      sa[mt][h] = sb[mt][h] = 0;
+      orow[mt][h] = -1;
       if (r < A.nrows) {
         const int fam = r / A.npair, p = row_pair[r % A.npair];
         const int pij = pair_ij[p];
@@ -837,7 +841,7 @@ k_triple(const float* __restrict__ R, const TripleArgs A, const int* __restrict_
 #pragma unroll
   for (int nt = 0; nt < TRI_NT; ++nt) {
     const int c = nt * 8 + g;
-    scol[nt] = c < A.ncol ? A.c_slot[c] : -1;
+    scol[nt] = c < A.ncol ? max(A.c_slot[c], 0) : 0;   // columns past the last or empty likewise
   }
   constexpr int NACC = TRI_MT * TRI_NT * 4;
   double* myacc = dacc + (size_t)tid * NACC;
@@ -853,64 +857,82 @@ k_triple(const float* __restrict__ R, const TripleArgs A, const int* __restrict_
   const int64_t beg = (int64_t)blockIdx.x * per;
   const int64_t end = min(A.ncell, beg + per);
   int nchunk = 0;
+  // Staging: per warp and step 16 bytes per lane of a field's cells, copied without passing through
+  // registers, so that all of a warp's rows are in flight together; the row's rotation is undone by the
+  // destination.  Cells at or past the end are zero (ncell is a multiple of RCH).
+  auto copy16 = [&](float* dst, const float* src, bool in) {
+    if (in)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                   : "memory");
+    else
+      *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  // SK: half h of the chunk at c0 holds the h-th 16 of every warp's 32 cells, so that one half is copied
+  // while the warps work on the other (the copies' latency and the products added up: 105 us per TripoSH
+  // launch at 256^3) and every warp still takes its cells in order
+  auto stage_half = [&](int64_t c0, int h) {
+    float* stage = stage0 + (size_t)h * A.nstage * SPAD;
+    const int j = lane * 4;                                  // place in the half
+    const int cell = (j >> 4) * 32 + h * 16 + (j & 15);      // cell of the chunk
+    for (int sl = warp; sl < A.nstage; sl += TRI_WARPS) {
+      const int field = A.stage_field[sl];
+      const float* src = R + (((size_t)(c0 / RCH) + (cell >> 7)) * A.nfield_r + field) * RCH +
+                         (((cell & (RCH - 1)) + rf_rot(field)) & (RCH - 1));
+      copy16(stage + (size_t)sl * SPAD + j, src, c0 + cell < end);
+    }
+  };
+  if (SK && beg < end) stage_half(beg, 0);
   for (int64_t c0 = beg; c0 < end; c0 += TRI_CHUNK) {
-    const int nc = (int)((end - c0) < (int64_t)TRI_CHUNK ? (end - c0) : (int64_t)TRI_CHUNK);
-    __syncthreads();
-    // one 128-cell row of a staged field per warp and step, 16 bytes per lane copied without passing
-    // through registers, so that all of a warp's rows are in flight together (loaded and stored one by
-    // one their latencies added up: 105 us per TripoSH launch at 256^3); the row's rotation is undone by
-    // the destination (nc is a multiple of RCH: ncell is)
-    for (int rw = warp; rw < A.nstage * (TRI_CHUNK / RCH); rw += TRI_WARPS) {
-      const int sl = rw / (TRI_CHUNK / RCH), half = rw % (TRI_CHUNK / RCH);
-      const int field = A.stage_field[sl], rot = rf_rot(field);
-      const int cl = (lane * 4 - rot) & (RCH - 1);   // logical cell of the lane's first value
-      float* dst = stage + (size_t)sl * TRI_SPAD + half * RCH + cl;
-      if (half * RCH < nc) {
-        const float* src = R + (((size_t)(c0 / RCH) + half) * A.nfield_r + field) * RCH + lane * 4;
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                     : "memory");
-      } else {
-        *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (!SK) {
+      __syncthreads();
+      for (int rw = warp; rw < A.nstage * (TRI_CHUNK / RCH); rw += TRI_WARPS) {
+        const int sl = rw / (TRI_CHUNK / RCH), half = rw % (TRI_CHUNK / RCH);
+        const int field = A.stage_field[sl], rot = rf_rot(field);
+        const int cl = (lane * 4 - rot) & (RCH - 1);   // logical cell of the lane's first value
+        copy16(stage0 + (size_t)sl * SPAD + half * RCH + cl,
+               R + (((size_t)(c0 / RCH) + half) * A.nfield_r + field) * RCH + lane * 4, c0 + half * RCH < end);
       }
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
-    constexpr int KPW = SK ? TRI_CHUNK / TRI_WARPS : TRI_CHUNK;   // cells of the chunk per warp
-    const int kbeg = SK ? warp * KPW : 0;
-    for (int kk = kbeg; kk < kbeg + KPW; kk += 8) {
-      uint32_t bh[TRI_NT][2], bl[TRI_NT][2];
-#pragma unroll
-      for (int nt = 0; nt < TRI_NT; ++nt) {
-        float v0 = 0.f, v1 = 0.f;
-        if (scol[nt] >= 0) {
-          const float* col = stage + (size_t)scol[nt] * TRI_SPAD + kk;
-          v0 = col[t];
-          v1 = col[t + 4];
-        }
-        split_tf32(v0, bh[nt][0], bl[nt][0]);
-        split_tf32(v1, bh[nt][1], bl[nt][1]);
+#pragma unroll 1
+    for (int h = 0; h < (SK ? 2 : 1); ++h) {
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncthreads();
+      if constexpr (SK) {   // the other buffer was last read before this barrier
+        if (h == 0) stage_half(c0, 1);
+        else if (c0 + TRI_CHUNK < end) stage_half(c0 + TRI_CHUNK, 0);
       }
-      uint32_t ah[TRI_MT][4], al[TRI_MT][4];
+      const float* stage = stage0 + (size_t)h * A.nstage * SPAD;
+      constexpr int KPW = SK ? SCELLS / TRI_WARPS : TRI_CHUNK;   // staged cells per warp
+      const int kbeg = SK ? warp * KPW : 0;
+#pragma unroll(SK ? 2 : 1)
+      for (int kk = kbeg; kk < kbeg + KPW; kk += 8) {
+        uint32_t bh[TRI_NT][2], bl[TRI_NT][2];
 #pragma unroll
-      for (int mt = 0; mt < TRI_MT; ++mt) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int h = q & 1;
-          const int kc = kk + t + ((q >> 1) ? 4 : 0);
-          float e = 0.f;
-          if (sa[mt][h] >= 0) e = stage[(size_t)sa[mt][h] * TRI_SPAD + kc] * stage[(size_t)sb[mt][h] * TRI_SPAD + kc];
-          split_tf32(e, ah[mt][q], al[mt][q]);
+        for (int nt = 0; nt < TRI_NT; ++nt) {
+          const float* col = stage + (size_t)scol[nt] * SPAD + kk;
+          split_tf32(col[t], bh[nt][0], bl[nt][0]);
+          split_tf32(col[t + 4], bh[nt][1], bl[nt][1]);
         }
+        uint32_t ah[TRI_MT][4], al[TRI_MT][4];
+#pragma unroll
+        for (int mt = 0; mt < TRI_MT; ++mt) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int h = q & 1;
+            const int kc = kk + t + ((q >> 1) ? 4 : 0);
+            split_tf32(stage[(size_t)sa[mt][h] * SPAD + kc] * stage[(size_t)sb[mt][h] * SPAD + kc], ah[mt][q], al[mt][q]);
+          }
+        }
+        // per accumulator hi hi, hi lo, lo hi; tile by tile within each, so that successive instructions
+        // do not wait for one another's accumulator
+#pragma unroll
+        for (int s = 0; s < 3; ++s)
+#pragma unroll
+          for (int mt = 0; mt < TRI_MT; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < TRI_NT; ++nt)
+              mma_tf32(d[mt][nt], s == 2 ? al[mt] : ah[mt], s == 1 ? bl[nt][0] : bh[nt][0], s == 1 ? bl[nt][1] : bh[nt][1]);
       }
-      // per accumulator hi hi, hi lo, lo hi; tile by tile within each, so that successive instructions
-      // do not wait for one another's accumulator
-#pragma unroll
-      for (int s = 0; s < 3; ++s)
-#pragma unroll
-        for (int mt = 0; mt < TRI_MT; ++mt)
-#pragma unroll
-          for (int nt = 0; nt < TRI_NT; ++nt)
-            mma_tf32(d[mt][nt], s == 2 ? al[mt] : ah[mt], s == 1 ? bl[nt][0] : bh[nt][0], s == 1 ? bl[nt][1] : bh[nt][1]);
     }
     if (++nchunk == TRI_FLUSH || c0 + TRI_CHUNK >= end) {
       nchunk = 0;
@@ -946,7 +968,8 @@ k_triple(const float* __restrict__ R, const TripleArgs A, const int* __restrict_
       for (int q = 0; q < 4; ++q, ++e) {
         const int r = orow[mt][q >> 1];
         const int c = nt * 8 + 2 * t + (q & 1);
-        if (r >= 0 && c < A.ncol) part[((size_t)blockIdx.x * A.nrows + r) * A.ncol + c] = myacc[e];
+        if (r >= 0 && c < A.ncol)
+          part[((size_t)blockIdx.x * A.nrows + r) * A.ncol + c] = A.c_slot[c] >= 0 ? myacc[e] : 0.0;
       }
 }
 
@@ -2610,7 +2633,8 @@ npc_status bispec_impl(npc_ctx* ctx, const npc_mesh_spec& m, const npc_kbins& kb
           3.0 * 2.0 * (a.nrows <= 32 && a.ncol <= 24 ? 32 : groups * rows) * (a.ncol <= 24 ? 24 : 32) * (double)a.ncell;
       if (a.nrows <= 32 && a.ncol <= 24) {
         // few rows: all warps on the same two m tiles, each on its own cells
-        const size_t smem = sizeof(float) * (size_t)a.nstage * TRI_SPAD + sizeof(double) * (size_t)TRI_WARPS * 32 * 2 * 3 * 4;
+        const size_t smem = sizeof(float) * (size_t)a.nstage * 2 * (TRI_CHUNK / 2 + 4) +
+                            sizeof(double) * (size_t)TRI_WARPS * 32 * 2 * 3 * 4;
         auto kern = k_triple<3, 2, true>;
         NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
         kern<<<dim3(grid, 1), TRI_WARPS * 32, smem, ctx->stream>>>((const float*)R, ak, (const int*)(dtab + tp),
