@@ -175,10 +175,13 @@ def algorithmic_bytes(w, stage, nf):
     nph = 2 if w["interlace"] else 1
     ntot = w["n_gal"] + w["n_ran"]
     act = active_row_fraction(w)
+    # the z pass writes one spectrum per (phase, l, m >= 0), the y pass reads it and writes the fields of
+    # both parts of Y_lm: sum(l + 1) = (sum(2l + 1) + number of l) / 2
+    sig = (nf + nph * len(w["ells"])) // 2
     if stage == "fft_z_weighted":
-        return nph * mesh + nf * half
+        return nph * mesh + sig * half
     if stage == "fft_y":
-        return nf * half * (1 + act)
+        return (sig + nf * act) * half
     if stage == "fft_x_contract":
         return nf * half * act
     tiles = nph * mesh * ((16 + 4) / 16) ** 3   # (bs+4)^3 tiles per bs^3 brick, per phase

@@ -7,7 +7,8 @@
 //   3. k_scatter      particles regrouped by brick as records {x, y, z, weight coefficient}.
 //   4. k_paint_brick  one CTA per brick accumulates every tap of its particles into a
 //                     (BS+4)^3 shared-memory tile (the brick plus the cells its particles can
-//                     reach) in 64-bit fixed point, so the sum is independent of thread order;
+//                     reach) in 64-bit fixed point (words of 32 bits), so the sum is independent of
+//                     thread order;
 //                     the tile is written out once.
 //   5. k_fold         each mesh cell sums, in a fixed order, the (up to 8) tiles that cover it.
 // The mesh is therefore bitwise reproducible run to run without any floating-point atomics.

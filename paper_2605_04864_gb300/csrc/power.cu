@@ -12,14 +12,15 @@
 // excluded from every bin) and every stored mode also stands for -k.
 //
 // Passes (3D transform by axes, shared-memory Stockham stages):
-//   k_fwd_z           reads the painted meshes, applies Y_l^m(xhat) at each grid point (phase a
-//                     at origin + jH, phase b at origin + (j - 1/2)H), transforms two real fields
-//                     at a time as one complex column along z, splits them into two half spectra.
-//   k_fft_cols        plain column transform along y.
-//   k_fft_x_contract  transforms every field's x-row of one (ky, kz), then per mode: interlacing
-//                     1/2[A_a + e^{iH(kx+ky+kz)/2} A_b], division by W(k) (Eq. compensation), F_l
-//                     assembly, Re[F_0 F_l^*] and Re[F_l F_l'^*] (Eq. Pllp), binned in float64
-//                     with a warp-segmented reduction into per-warp partial sums (no atomics
+//   k_fwd_z           reads the painted meshes and transforms, per (phase, l, m), the real signal
+//                     F(z) Q_lm(uz) r^-m of each column along z (phase a at grid points origin + jH,
+//                     phase b at origin + (j - 1/2)H), two signals per complex transform.
+//   k_fft_cols_weighted  multiplies by the real and imaginary part of the column factor
+//                     (px + i py)^m and transforms both along y (k_fft_cols: without factors).
+//   k_fft_x_contract  transforms every field's x-row of one (ky, kz), one row per thread group, then per
+//                     mode: interlacing 1/2[A_a + e^{iH(kx+ky+kz)/2} A_b], division by W(k) (Eq.
+//                     compensation), F_l assembly, Re[F_0 F_l^*] and Re[F_l F_l'^*] (Eq. Pllp), binned
+//                     in float64 with a warp-segmented reduction into per-warp partial sums (no atomics
 //                     between warps, fixed order: reproducible run to run).
 //   k_power_finalize  fixed-order sum of the partials, normalisation (2l+1)/I22, shot noise,
 //                     the modified multipoles of Eq. Plnew.
