@@ -161,6 +161,44 @@ npc_status get_twiddles(npc_ctx* ctx, int n, int prec, const void** out) {
   return NPC_OK;
 }
 
+// Formed in float64 and rounded once.  Formed in float by every CTA, the window's factor of an axis was off by
+// up to 1.5e-7 and by the same in every mode of that |k_axis|: the factors of the three axes enter a spectrum
+// squared, so at low k, where the modes of a bin cancel, they outweighed the roundings of the transforms
+// (1.1e-7 per mode at 192^3).
+template <typename T> static std::vector<cplx<T>> mode_factors(int n, int assign) {
+  std::vector<cplx<T>> h(2 * n + n / 4 + 1);
+  for (int i = 0; i < 2 * n; ++i) {
+    const double a = M_PI * (i - n) / n;
+    h[i] = cmk((T)std::cos(a), (T)std::sin(a));
+  }
+  T* winv = reinterpret_cast<T*>(h.data() + 2 * n);
+  for (int j = 0; j <= n / 2; ++j) {
+    const double a = M_PI * j / n;
+    winv[j] = (T)(j ? std::pow(a / std::sin(a), assign) : 1.0);
+  }
+  return h;
+}
+
+npc_status get_mode_factors(npc_ctx* ctx, int n, int assign, int prec, const void** out) {
+  std::vector<char> key;
+  key_push(key, n);
+  key_push(key, assign);
+  const std::string name =
+      std::string(prec == NPC_PREC_FP64 ? "modes64." : "modes32.") + std::to_string(n) + "." + std::to_string(assign);
+  void* p;
+  if (!table_cached(ctx, name, key, &p)) {
+    if (prec == NPC_PREC_FP64) {
+      const auto h = mode_factors<double>(n, assign);
+      NPC_TRY(ws_table(ctx, name, key, h.data(), sizeof(double2) * h.size(), &p));
+    } else {
+      const auto h = mode_factors<float>(n, assign);
+      NPC_TRY(ws_table(ctx, name, key, h.data(), sizeof(float2) * h.size(), &p));
+    }
+  }
+  *out = p;
+  return NPC_OK;
+}
+
 // bin of every integer |k|^2 = i^2+j^2+l^2 (host, float64, no contraction: -ffp-contract=off)
 npc_status get_bin_table(npc_ctx* ctx, int n, double box, const npc_kbins& kb, const int16_t** out, int slot) {
   const std::string name = "bintab" + std::to_string(slot);

@@ -358,6 +358,9 @@ npc_status run_power_contract(npc_ctx* ctx, int prec, const PowerPlan& plan, con
 npc_status get_bin_table(npc_ctx* ctx, int n, double box, const npc_kbins& kb, const int16_t** out, int slot = 0);
 // twiddle table of length-n transforms (n entries, laid out as fft_core.cuh describes), as cplx<T>
 npc_status get_twiddles(npc_ctx* ctx, int n, int prec, const void** out);
+// mode factors of the binning x pass, as cplx<T>: e^{i pi m/n} for m = -n .. n - 1, then (as T) the inverse
+// window (a/sin a)^assign of one axis, a = pi j/n for j = 0 .. n/2
+npc_status get_mode_factors(npc_ctx* ctx, int n, int assign, int prec, const void** out);
 
 // ---------------------------------------------------------------------------------------------
 // Bispectrum (bispec.cu)

@@ -489,17 +489,6 @@ struct ContractParams {
   double kf;
 };
 
-template <typename T>
-__device__ __forceinline__ T sinc_pow(T a, int p) {
-  const T s = a == T(0) ? T(1) : sin(a) / a;
-  T r = s;
-  for (int i = 1; i < p; ++i) r *= s;
-  return r;
-}
-
-__device__ __forceinline__ void sincospi_t(float x, float* s, float* c) { sincospif(x, s, c); }
-__device__ __forceinline__ void sincospi_t(double x, double* s, double* c) { sincospi(x, s, c); }
-
 // L_l(mu), l <= 4, as polynomials (uniform l, no division)
 template <typename T> __device__ __forceinline__ T legendre_0to4(int l, T mu) {
   const T m2 = mu * mu;
@@ -560,7 +549,8 @@ __device__ __forceinline__ void add_weighted(cplx<T> (&acc)[8], const cplx<T> (&
 template <typename T, int N, int MINB>
 __global__ void __launch_bounds__(CONTRACT_THREADS, MINB)
 k_fft_x_contract(const cplx<T>* __restrict__ half, const __grid_constant__ ContractParams P,
-                 const int16_t* __restrict__ bintab, const cplx<T>* __restrict__ tw_g, double* __restrict__ part) {
+                 const int16_t* __restrict__ bintab, const cplx<T>* __restrict__ tw_g,
+                 const cplx<T>* __restrict__ factors, double* __restrict__ part) {
   using C = cplx<T>;
   using Team = XTeam<N>;
   constexpr int TPF = Team::TPF;
@@ -579,12 +569,8 @@ k_fft_x_contract(const cplx<T>* __restrict__ half, const __grid_constant__ Contr
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nent = P.nbins * P.nsum;
   for (int i = tid; i < N; i += blockDim.x) tw[i] = tw_g[i];
-  for (int i = tid; i <= N / 2; i += blockDim.x) winv[i] = T(1) / sinc_pow<T>(T(M_PI) * T(i) / T(N), P.assign);
-  for (int i = tid; i < 2 * N; i += blockDim.x) {
-    T sn, cs;
-    sincospi_t(T(i - N) / T(N), &sn, &cs);
-    phs[i] = cmk(cs, sn);
-  }
+  for (int i = tid; i < 2 * N; i += blockDim.x) phs[i] = factors[i];
+  for (int i = tid; i <= N / 2; i += blockDim.x) winv[i] = reinterpret_cast<const T*>(factors + 2 * N)[i];
   if (P.shared_part)
     for (int i = tid; i < nw * nent; i += blockDim.x) spart[i] = 0.0;
   __syncthreads();
@@ -1056,6 +1042,8 @@ npc_status contract_impl(npc_ctx* ctx, const PowerPlan& plan, const npc_mesh_spe
   using C = cplx<T>;
   const void* twp;
   NPC_TRY(get_twiddles(ctx, N, sizeof(T) == 8 ? NPC_PREC_FP64 : NPC_PREC_MIXED, &twp));
+  const void* factors;
+  NPC_TRY(get_mode_factors(ctx, N, plan.assign, sizeof(T) == 8 ? NPC_PREC_FP64 : NPC_PREC_MIXED, &factors));
   const int16_t* bintab;
   NPC_TRY(get_bin_table(ctx, N, m.box, kb, &bintab));
   ContractParams P{};
@@ -1172,7 +1160,7 @@ npc_status contract_impl(npc_ctx* ctx, const PowerPlan& plan, const npc_mesh_spe
   if (!P.shared_part)
     NPC_CUDA(ctx, cudaMemsetAsync(part, 0, sizeof(double) * nparts * P.nbins * P.nsum, ctx->stream));
   NPC_TRY(stage_mark(ctx, "contract_setup"));
-  kern<<<grid, threads, smem, ctx->stream>>>((const C*)half, P, bintab, (const C*)twp, part);
+  kern<<<grid, threads, smem, ctx->stream>>>((const C*)half, P, bintab, (const C*)twp, (const C*)factors, part);
   NPC_LAUNCH(ctx);
   NPC_TRY(stage_mark(ctx, "fft_x_contract"));
 
