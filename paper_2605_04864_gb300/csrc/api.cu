@@ -314,7 +314,10 @@ Geom make_geom(const npc_mesh_spec& m) {
   Geom g{};
   g.n = m.n;
   g.h = m.box / m.n;
-  for (int a = 0; a < 3; ++a) g.o[a] = m.origin[a] - m.observer[a];
+  for (int a = 0; a < 3; ++a) {
+    g.o[a] = m.origin[a];
+    g.obs[a] = m.observer[a];
+  }
   const double l = std::sqrt(m.los_dir[0] * m.los_dir[0] + m.los_dir[1] * m.los_dir[1] + m.los_dir[2] * m.los_dir[2]);
   for (int a = 0; a < 3; ++a) g.los[a] = l > 0 ? m.los_dir[a] / l : 0.0;
   g.global_los = m.los;

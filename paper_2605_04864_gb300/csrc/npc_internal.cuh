@@ -164,7 +164,8 @@ struct FieldList {
 struct Geom {
   int n;
   double h;          // box / n
-  double o[3];       // origin - observer
+  double o[3];       // origin
+  double obs[3];     // observer
   double los[3];     // unit global LOS
   int global_los;
 };

@@ -151,7 +151,62 @@ struct SignalList {
   Signal s[MAX_SIGNALS];
 };
 
-// s(z) times norm of one signal at the thread's elements z = t + q TPF
+// A grid point can lie at the observer up to the rounding of its coordinates, and r^-m and (px + i py)^m can
+// then leave the range of float32 while their product cannot.  The coordinates are in units of a power of two
+// that makes the largest one about 1, whatever the user's unit of length.  Columns with |px|, |py| < near, a
+// power of two of at most half a cell (`near` columns: the one or few at the observer's x and y) take out of
+// r^-m a power of two f^m <= 1 that their column factor puts back.  f = 2^floor(log2(max(|px|, |py|))) / near
+// comes from the bits of px and py, so both passes form the same one; it is at most r / near, which leaves
+// the signal no larger than its neighbours'.  Every other column has r >= near.
+__device__ __forceinline__ float pow2_floor(float x) { return __uint_as_float(__float_as_uint(x) & 0x7f800000u); }
+__device__ __forceinline__ double pow2_floor(double x) {
+  return __longlong_as_double(__double_as_longlong(x) & 0x7ff0000000000000ll);
+}
+// 1 / pow2_floor(x), finite at x = 0
+__device__ __forceinline__ float pow2_inv(float x) {
+  return __uint_as_float(0x7f000000u - (__float_as_uint(x) & 0x7f800000u));
+}
+__device__ __forceinline__ double pow2_inv(double x) {
+  return __longlong_as_double(0x7fe0000000000000ll - (__double_as_longlong(x) & 0x7ff0000000000000ll));
+}
+__device__ __forceinline__ float absmax(float x, float y) { return fmaxf(fabsf(x), fabsf(y)); }
+__device__ __forceinline__ double absmax(double x, double y) { return fmax(fabs(x), fabs(y)); }
+
+// s(z) times norm of one signal of a near column, pz from the table (near r = 0 the rounding of a sum would
+// turn the direction).  A grid point exactly at the observer has the direction of the z axis.
+template <typename T, int N, int TX>
+__device__ __forceinline__ void near_signal(T (&sv)[8], int l, int m, const T* tile, int c, int t,
+                                            const T* __restrict__ coords, int phase, int x, int y, T near, T norm) {
+  constexpr int TPF = N / 8;
+  const T px = coords[phase * N + x], py = coords[(2 + phase) * N + y];
+  const T own = absmax(px, py);
+  T near_sv[8];
+#pragma unroll 1
+  for (int q = 0; q < 8; ++q) {
+    const int z = t + q * TPF;
+    const T pz = coords[(4 + phase) * N + z];
+    const T scale = pow2_inv(absmax(own, pz));   // the largest coordinate near 1: r^2 cannot underflow
+    const T ux = px * scale, uy = py * scale, uz0 = pz * scale;
+    const T r2 = ux * ux + uy * uy + uz0 * uz0;
+    const T inv = r2 > T(0) ? rsqrt(r2) : T(0);
+    const T uz = r2 > T(0) ? uz0 * inv : T(1);
+    T v;
+#define NPC_Q(L, M) case L * (L + 1) / 2 + M: v = ylm_q<T, L, M>(uz); break;
+    switch (l * (l + 1) / 2 + m) {
+      NPC_Q(1, 0) NPC_Q(1, 1) NPC_Q(2, 0) NPC_Q(2, 1) NPC_Q(2, 2) NPC_Q(3, 0) NPC_Q(3, 1) NPC_Q(3, 2) NPC_Q(3, 3)
+      NPC_Q(4, 0) NPC_Q(4, 1) NPC_Q(4, 2) NPC_Q(4, 3) NPC_Q(4, 4)
+      default: v = T(1);
+    }
+#undef NPC_Q
+    v = tile[z * TX + c] * (norm * v);
+    for (int j = 0; j < m; ++j) v *= pow2_floor(own) * scale * inv / near;
+    near_sv[q] = v;
+  }
+#pragma unroll
+  for (int q = 0; q < 8; ++q) sv[q] = near_sv[q];
+}
+
+// s(z) times norm of one signal at the thread's elements z = t + q TPF of a column that is not near
 template <typename T, int N, int TX, int L, int M>
 __device__ __forceinline__ void column_signal(T (&sv)[8], const T* tile, int c, int t, T pxy2, T pz0, T dz, T norm) {
   constexpr int TPF = N / 8;
@@ -164,7 +219,7 @@ __device__ __forceinline__ void column_signal(T (&sv)[8], const T* tile, int c, 
     } else {
       const T pz = pz0 + T(q) * dz;
       const T r2 = pxy2 + pz * pz;
-      const T inv = r2 > T(0) ? rsqrt(r2) : T(0);
+      const T inv = rsqrt(r2);
       if constexpr (M == 0) {
         sv[q] = F * (norm * ylm_q<T, L, 0>(pz * inv));
       } else {
@@ -180,8 +235,15 @@ __device__ __forceinline__ void column_signal(T (&sv)[8], const T* tile, int c, 
 template <typename T, int N, int TX>
 __device__ __forceinline__ void any_signal(T (&sv)[8], const Signal& sg, const T* tileA, const T* tileB, int c, int t,
                                            const T (&pxy2)[2], const T (&pz0)[2], T dz, const YNorm& nrm,
-                                           bool norm_in) {
+                                           bool norm_in, int near_phases, const T* __restrict__ coords, int x, int y,
+                                           T near) {
   const T* tile = sg.phase ? tileB : tileA;
+  if (near_phases & (1 << sg.phase)) {
+    const int lm = sg.l * (sg.l + 1) / 2 + sg.m;
+    near_signal<T, N, TX>(sv, sg.l, sg.m, tile, c, t, coords, sg.phase, x, y, near,
+                          sg.l > 0 && (sg.m == 0 || norm_in) ? ynorm<T>(nrm, lm) : T(1));
+    return;
+  }
   const T p2 = sg.phase ? pxy2[1] : pxy2[0], z0 = sg.phase ? pz0[1] : pz0[0];
 #define NPC_S(L, M) \
   case L * (L + 1) / 2 + M: column_signal<T, N, TX, L, M>(sv, tile, c, t, p2, z0, dz, M == 0 || norm_in ? ynorm<T>(nrm, L * (L + 1) / 2 + M) : T(1)); break;
@@ -198,15 +260,17 @@ template <typename T, int N> constexpr int zpass_min_blocks() {
   return sizeof(T) == 4 ? 65536 / (ColCfg<N>::THREADS * (ColCfg<N>::THREADS == 512 ? 64 : 80)) : 1;
 }
 
-// Coordinates of the grid points from the observer, tab[axis][phase][n], formed in float64 and rounded
-// once (phase b lies half a cell lower): the weighted passes look them up instead of forming them per
-// thread, since float64 arithmetic is scarce on this part (y pass at 512^3: 10.1 ms with, 6.0 without).
+// Coordinates of the grid points from the observer times `unit`, tab[axis][phase][n], formed in float64 step
+// by step (no fused multiply-add: half a box plus minus half a box is 0) and rounded once; phase b lies half
+// a cell lower.  The weighted passes look them up instead of forming them per thread, since float64
+// arithmetic is scarce on this part (y pass at 512^3: 10.1 ms with, 6.0 without).
 template <typename T>
-__global__ void k_axis_coords(const Geom g, T* __restrict__ tab) {
+__global__ void k_axis_coords(const Geom g, double unit, T* __restrict__ tab) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 6 * g.n; i += gridDim.x * blockDim.x) {
     const int a = i / (2 * g.n), ph = (i / g.n) % 2, j = i % g.n;
     const double o = a == 0 ? g.o[0] : (a == 1 ? g.o[1] : g.o[2]);
-    tab[i] = (T)(o + ((double)j - (ph ? 0.5 : 0.0)) * g.h);
+    const double obs = a == 0 ? g.obs[0] : (a == 1 ? g.obs[1] : g.obs[2]);
+    tab[i] = (T)((__dadd_rn(o, __dmul_rn((double)j - (ph ? 0.5 : 0.0), g.h)) - obs) * unit);
   }
 }
 
@@ -214,7 +278,7 @@ __global__ void k_axis_coords(const Geom g, T* __restrict__ tab) {
 template <typename T, int N>
 __global__ void __launch_bounds__(ColCfg<N>::THREADS, zpass_min_blocks<T, N>())
 k_fwd_z(const T* __restrict__ mesh_a, const T* __restrict__ mesh_b, cplx<T>* __restrict__ half,
-        const __grid_constant__ SignalList sl, const T* __restrict__ coords, const T dz, const YNorm nrm,
+        const __grid_constant__ SignalList sl, const T* __restrict__ coords, const T dz, const T near, const YNorm nrm,
         const cplx<T>* __restrict__ tw_g, int KZ) {
   using C = cplx<T>;
   constexpr int TX = ColCfg<N>::TX;
@@ -235,12 +299,14 @@ k_fwd_z(const T* __restrict__ mesh_a, const T* __restrict__ mesh_b, cplx<T>* __r
     if (mesh_b) tileB[i] = mesh_b[gi];
   }
   T pxy2[2] = {T(0), T(0)}, pz0[2] = {T(0), T(0)};
+  int near_phases = 0;
   if (coords) {
 #pragma unroll
     for (int ph = 0; ph < 2; ++ph) {
       const T px = coords[ph * N + x0 + c], py = coords[(2 + ph) * N + y];
       pxy2[ph] = px * px + py * py;
       pz0[ph] = coords[(4 + ph) * N + t];
+      near_phases |= absmax(px, py) < near ? 1 << ph : 0;
     }
   }
   __syncthreads();
@@ -251,9 +317,11 @@ k_fwd_z(const T* __restrict__ mesh_a, const T* __restrict__ mesh_b, cplx<T>* __r
     C v[8];
     {
       T a[8], b[8];
-      any_signal<T, N, TX>(a, s0, tileA, tileB, c, t, pxy2, pz0, dz, nrm, sl.norm_in_signal);
+      any_signal<T, N, TX>(a, s0, tileA, tileB, c, t, pxy2, pz0, dz, nrm, sl.norm_in_signal, near_phases, coords,
+                           x0 + c, y, near);
       if (s1.re >= 0) {
-        any_signal<T, N, TX>(b, s1, tileA, tileB, c, t, pxy2, pz0, dz, nrm, sl.norm_in_signal);
+        any_signal<T, N, TX>(b, s1, tileA, tileB, c, t, pxy2, pz0, dz, nrm, sl.norm_in_signal, near_phases, coords,
+                             x0 + c, y, near);
       } else {
 #pragma unroll
         for (int q = 0; q < 8; ++q) b[q] = T(0);
@@ -324,17 +392,23 @@ static SignalList make_signals(const FieldList& fl) {
 
 // v = S norm Re (px + i py)^M and keep = S norm Im (px + i py)^M at the thread's elements
 template <typename T, int N, int TX, int M>
-__device__ __forceinline__ void column_factors(cplx<T> (&v)[8], cplx<T>* keep, const T* __restrict__ pys, T px, T norm,
-                                               int c, int t) {
+__device__ __forceinline__ void column_factors(cplx<T> (&v)[8], cplx<T>* keep, const T* __restrict__ pys, T px, T near,
+                                               T norm, int c, int t) {
   constexpr int TPF = N / 8;
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    const T py = pys[t + q * TPF];
+    T fx = px, fy = pys[t + q * TPF];
+    const T own = absmax(fx, fy);
+    if (own < near) {
+      const T back = near * pow2_inv(own);
+      fx *= back;
+      fy *= back;
+    }
     T cr = norm, ci = T(0);
 #pragma unroll
     for (int j = 0; j < M; ++j) {
-      const T nr = cr * px - ci * py;
-      ci = cr * py + ci * px;
+      const T nr = cr * fx - ci * fy;
+      ci = cr * fy + ci * fx;
       cr = nr;
     }
     keep[(t + q * TPF) * TX + c] = cscale(v[q], ci);
@@ -347,7 +421,7 @@ __device__ __forceinline__ void column_factors(cplx<T> (&v)[8], cplx<T>* keep, c
 template <typename T, int N, int TX>
 __global__ void __launch_bounds__(TX * N / 8, (sizeof(T) == 4 && TX * N / 8 <= 512 ? 1536 / (TX * N / 8) : 1))
 k_fft_cols_weighted(cplx<T>* __restrict__ half, const __grid_constant__ SignalList sl, const T* __restrict__ coords,
-                    const YNorm nrm, const cplx<T>* __restrict__ tw_g, int KZ, int row_n2max) {
+                    const T near, const YNorm nrm, const cplx<T>* __restrict__ tw_g, int KZ, int row_n2max) {
   using C = cplx<T>;
   constexpr int TPF = N / 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -373,10 +447,10 @@ k_fft_cols_weighted(cplx<T>* __restrict__ half, const __grid_constant__ SignalLi
     const T* __restrict__ pys = coords + (2 + sg.phase) * N;
     const T norm = sl.norm_in_signal ? T(1) : ynorm<T>(nrm, sg.l * (sg.l + 1) / 2 + sg.m);
     switch (sg.m) {
-      case 1: column_factors<T, N, TX, 1>(v, keep, pys, px, norm, c, t); break;
-      case 2: column_factors<T, N, TX, 2>(v, keep, pys, px, norm, c, t); break;
-      case 3: column_factors<T, N, TX, 3>(v, keep, pys, px, norm, c, t); break;
-      default: column_factors<T, N, TX, 4>(v, keep, pys, px, norm, c, t);
+      case 1: column_factors<T, N, TX, 1>(v, keep, pys, px, near, norm, c, t); break;
+      case 2: column_factors<T, N, TX, 2>(v, keep, pys, px, near, norm, c, t); break;
+      case 3: column_factors<T, N, TX, 3>(v, keep, pys, px, near, norm, c, t); break;
+      default: column_factors<T, N, TX, 4>(v, keep, pys, px, near, norm, c, t);
     }
   }
   __syncthreads();
@@ -917,8 +991,8 @@ npc_status y_pass(npc_ctx* ctx, cplx<T>* data, int nplanes, const cplx<T>* tw, i
 }
 
 template <typename T, int N, int TX>
-npc_status y_pass_weighted_tx(npc_ctx* ctx, cplx<T>* half, const SignalList& sl, const T* coords, const YNorm& nrm,
-                              const cplx<T>* tw, int KZ, int row_n2max) {
+npc_status y_pass_weighted_tx(npc_ctx* ctx, cplx<T>* half, const SignalList& sl, const T* coords, T near,
+                              const YNorm& nrm, const cplx<T>* tw, int KZ, int row_n2max) {
   using C = cplx<T>;
   if constexpr (!ytx_ok<N>(TX)) {
     return set_err(ctx, NPC_ERR_INVALID_ARG, "y pass: %d columns per CTA not valid at n = %d", TX, N);
@@ -927,22 +1001,22 @@ npc_status y_pass_weighted_tx(npc_ctx* ctx, cplx<T>* half, const SignalList& sl,
     auto kern = k_fft_cols_weighted<T, N, TX>;
     NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
     const int nplanes = sl.n * KZ;   // at most 32 x 512
-    kern<<<dim3(N / TX, nplanes), TX * N / 8, smem, ctx->stream>>>(half, sl, coords, nrm, tw, KZ, row_n2max);
+    kern<<<dim3(N / TX, nplanes), TX * N / 8, smem, ctx->stream>>>(half, sl, coords, near, nrm, tw, KZ, row_n2max);
     NPC_LAUNCH(ctx);
     return NPC_OK;
   }
 }
 
 template <typename T, int N>
-npc_status y_pass_weighted(npc_ctx* ctx, cplx<T>* half, const SignalList& sl, const T* coords, const YNorm& nrm,
-                           const cplx<T>* tw, int tx, int KZ, int row_n2max) {
+npc_status y_pass_weighted(npc_ctx* ctx, cplx<T>* half, const SignalList& sl, const T* coords, T near,
+                           const YNorm& nrm, const cplx<T>* tw, int tx, int KZ, int row_n2max) {
   // 32 columns of the longest FP64 lines and their copy would not fit an SM's shared memory
   if (sizeof(cplx<T>) * N * tx * 2 > 150 * 1024) tx = 16;
   switch (tx) {
-    case 4: return y_pass_weighted_tx<T, N, 4>(ctx, half, sl, coords, nrm, tw, KZ, row_n2max);
-    case 8: return y_pass_weighted_tx<T, N, 8>(ctx, half, sl, coords, nrm, tw, KZ, row_n2max);
-    case 16: return y_pass_weighted_tx<T, N, 16>(ctx, half, sl, coords, nrm, tw, KZ, row_n2max);
-    case 32: return y_pass_weighted_tx<T, N, 32>(ctx, half, sl, coords, nrm, tw, KZ, row_n2max);
+    case 4: return y_pass_weighted_tx<T, N, 4>(ctx, half, sl, coords, near, nrm, tw, KZ, row_n2max);
+    case 8: return y_pass_weighted_tx<T, N, 8>(ctx, half, sl, coords, near, nrm, tw, KZ, row_n2max);
+    case 16: return y_pass_weighted_tx<T, N, 16>(ctx, half, sl, coords, near, nrm, tw, KZ, row_n2max);
+    case 32: return y_pass_weighted_tx<T, N, 32>(ctx, half, sl, coords, near, nrm, tw, KZ, row_n2max);
   }
   return set_err(ctx, NPC_ERR_INVALID_ARG, "y pass: unsupported columns per CTA %d", tx);
 }
@@ -1004,10 +1078,15 @@ npc_status fwd_impl(npc_ctx* ctx, const PowerPlan& plan, const Geom& g, const vo
     directions |= sl.s[i].l > 0;
     weighted |= sl.s[i].m > 0;
   }
+  // unit of the coordinates: the power of two at or below the farthest grid point's distance along an axis
+  double far = 0.0;
+  for (int a = 0; a < 3; ++a) far = std::max(far, std::fabs(g.o[a] - g.obs[a]) + g.h * N);
+  const double unit = std::ldexp(1.0, -std::ilogb(far));
+  const T near = (T)std::ldexp(1.0, std::ilogb(0.5 * g.h * unit));
   T* coords = nullptr;
   if (directions) {
     NPC_TRY(ws_get(ctx, "fwd.coords", sizeof(T) * 6 * N, (void**)&coords));
-    k_axis_coords<T><<<(6 * N + 255) / 256, 256, 0, ctx->stream>>>(g, coords);
+    k_axis_coords<T><<<(6 * N + 255) / 256, 256, 0, ctx->stream>>>(g, unit, coords);
     NPC_LAUNCH(ctx);
   }
   if (single) {
@@ -1022,14 +1101,14 @@ npc_status fwd_impl(npc_ctx* ctx, const PowerPlan& plan, const Geom& g, const vo
     auto kern = k_fwd_z<T, N>;
     NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
     kern<<<dim3(N / TX, N), ColCfg<N>::THREADS, smem, ctx->stream>>>((const T*)mesh_a, (const T*)mesh_b, (C*)half, sl,
-                                                                     coords, (T)(g.h * (N / 8)), nrm, tw, KZ);
+                                                                     coords, (T)(g.h * (N / 8) * unit), near, nrm, tw, KZ);
   }
   NPC_LAUNCH(ctx);
   NPC_TRY(stage_mark(ctx, "fft_z_weighted"));
   const int n2max = plan.row_n2max > 0 ? plan.row_n2max : (1 << 30);
   // planes (f, kz) are contiguous N*N blocks; y rows have stride N
   if (weighted)
-    NPC_TRY((y_pass_weighted<T, N>(ctx, (C*)half, sl, coords, nrm, tw, ytx_for(ctx, N, sizeof(T) == 8), KZ, n2max)));
+    NPC_TRY((y_pass_weighted<T, N>(ctx, (C*)half, sl, coords, near, nrm, tw, ytx_for(ctx, N, sizeof(T) == 8), KZ, n2max)));
   else
     NPC_TRY((y_pass<T, N>(ctx, (C*)half, plan.fl.nf * KZ, tw, ytx_for(ctx, N, sizeof(T) == 8), KZ, n2max)));
   NPC_TRY(stage_mark(ctx, "fft_y"));
