@@ -157,7 +157,9 @@ struct SignalList {
 // power of two of at most half a cell (`near` columns: the one or few at the observer's x and y) take out of
 // r^-m a power of two f^m <= 1 that their column factor puts back.  f = 2^floor(log2(max(|px|, |py|))) / near
 // comes from the bits of px and py, so both passes form the same one; it is at most r / near, which leaves
-// the signal no larger than its neighbours'.  Every other column has r >= near.
+// the signal no larger than its neighbours'.  Every other column has r >= near.  Few meshes have near columns,
+// and the code for them would cost all others (512^3: z pass 4.51 -> 4.78 ms, y pass 6.00 -> 6.23), so it is
+// a variant (NEAR) of the passes that the host launches for meshes with near columns.
 __device__ __forceinline__ float pow2_floor(float x) { return __uint_as_float(__float_as_uint(x) & 0x7f800000u); }
 __device__ __forceinline__ double pow2_floor(double x) {
   return __longlong_as_double(__double_as_longlong(x) & 0x7ff0000000000000ll);
@@ -232,13 +234,13 @@ __device__ __forceinline__ void column_signal(T (&sv)[8], const T* tile, int c, 
   }
 }
 
-template <typename T, int N, int TX>
+template <typename T, int N, int TX, bool NEAR>
 __device__ __forceinline__ void any_signal(T (&sv)[8], const Signal& sg, const T* tileA, const T* tileB, int c, int t,
                                            const T (&pxy2)[2], const T (&pz0)[2], T dz, const YNorm& nrm,
                                            bool norm_in, int near_phases, const T* __restrict__ coords, int x, int y,
                                            T near) {
   const T* tile = sg.phase ? tileB : tileA;
-  if (near_phases & (1 << sg.phase)) {
+  if (NEAR && (near_phases & (1 << sg.phase))) {
     const int lm = sg.l * (sg.l + 1) / 2 + sg.m;
     near_signal<T, N, TX>(sv, sg.l, sg.m, tile, c, t, coords, sg.phase, x, y, near,
                           sg.l > 0 && (sg.m == 0 || norm_in) ? ynorm<T>(nrm, lm) : T(1));
@@ -275,7 +277,7 @@ __global__ void k_axis_coords(const Geom g, double unit, T* __restrict__ tab) {
 }
 
 // First pass: the signals' half spectra along z, S[slot][kz][y][x].
-template <typename T, int N>
+template <typename T, int N, bool NEAR>
 __global__ void __launch_bounds__(ColCfg<N>::THREADS, zpass_min_blocks<T, N>())
 k_fwd_z(const T* __restrict__ mesh_a, const T* __restrict__ mesh_b, cplx<T>* __restrict__ half,
         const __grid_constant__ SignalList sl, const T* __restrict__ coords, const T dz, const T near, const YNorm nrm,
@@ -306,7 +308,7 @@ k_fwd_z(const T* __restrict__ mesh_a, const T* __restrict__ mesh_b, cplx<T>* __r
       const T px = coords[ph * N + x0 + c], py = coords[(2 + ph) * N + y];
       pxy2[ph] = px * px + py * py;
       pz0[ph] = coords[(4 + ph) * N + t];
-      near_phases |= absmax(px, py) < near ? 1 << ph : 0;
+      if (NEAR) near_phases |= absmax(px, py) < near ? 1 << ph : 0;
     }
   }
   __syncthreads();
@@ -317,11 +319,11 @@ k_fwd_z(const T* __restrict__ mesh_a, const T* __restrict__ mesh_b, cplx<T>* __r
     C v[8];
     {
       T a[8], b[8];
-      any_signal<T, N, TX>(a, s0, tileA, tileB, c, t, pxy2, pz0, dz, nrm, sl.norm_in_signal, near_phases, coords,
-                           x0 + c, y, near);
+      any_signal<T, N, TX, NEAR>(a, s0, tileA, tileB, c, t, pxy2, pz0, dz, nrm, sl.norm_in_signal, near_phases, coords,
+                                 x0 + c, y, near);
       if (s1.re >= 0) {
-        any_signal<T, N, TX>(b, s1, tileA, tileB, c, t, pxy2, pz0, dz, nrm, sl.norm_in_signal, near_phases, coords,
-                             x0 + c, y, near);
+        any_signal<T, N, TX, NEAR>(b, s1, tileA, tileB, c, t, pxy2, pz0, dz, nrm, sl.norm_in_signal, near_phases,
+                                   coords, x0 + c, y, near);
       } else {
 #pragma unroll
         for (int q = 0; q < 8; ++q) b[q] = T(0);
@@ -391,7 +393,7 @@ static SignalList make_signals(const FieldList& fl) {
 }
 
 // v = S norm Re (px + i py)^M and keep = S norm Im (px + i py)^M at the thread's elements
-template <typename T, int N, int TX, int M>
+template <typename T, int N, int TX, int M, bool NEAR>
 __device__ __forceinline__ void column_factors(cplx<T> (&v)[8], cplx<T>* keep, const T* __restrict__ pys, T px, T near,
                                                T norm, int c, int t) {
   constexpr int TPF = N / 8;
@@ -399,7 +401,7 @@ __device__ __forceinline__ void column_factors(cplx<T> (&v)[8], cplx<T>* keep, c
   for (int q = 0; q < 8; ++q) {
     T fx = px, fy = pys[t + q * TPF];
     const T own = absmax(fx, fy);
-    if (own < near) {
+    if (NEAR && own < near) {
       const T back = near * pow2_inv(own);
       fx *= back;
       fy *= back;
@@ -418,7 +420,7 @@ __device__ __forceinline__ void column_factors(cplx<T> (&v)[8], cplx<T>* keep, c
 
 // y pass with the column factors: plane (signal, kz) = blockIdx.y; the transforms of S times the
 // real and the imaginary part of norm (px + i py)^m go to the two parts' fields (m = 0: S itself, in place).
-template <typename T, int N, int TX>
+template <typename T, int N, int TX, bool NEAR>
 __global__ void __launch_bounds__(TX * N / 8, (sizeof(T) == 4 && TX * N / 8 <= 512 ? 1536 / (TX * N / 8) : 1))
 k_fft_cols_weighted(cplx<T>* __restrict__ half, const __grid_constant__ SignalList sl, const T* __restrict__ coords,
                     const T near, const YNorm nrm, const cplx<T>* __restrict__ tw_g, int KZ, int row_n2max) {
@@ -447,10 +449,10 @@ k_fft_cols_weighted(cplx<T>* __restrict__ half, const __grid_constant__ SignalLi
     const T* __restrict__ pys = coords + (2 + sg.phase) * N;
     const T norm = sl.norm_in_signal ? T(1) : ynorm<T>(nrm, sg.l * (sg.l + 1) / 2 + sg.m);
     switch (sg.m) {
-      case 1: column_factors<T, N, TX, 1>(v, keep, pys, px, near, norm, c, t); break;
-      case 2: column_factors<T, N, TX, 2>(v, keep, pys, px, near, norm, c, t); break;
-      case 3: column_factors<T, N, TX, 3>(v, keep, pys, px, near, norm, c, t); break;
-      default: column_factors<T, N, TX, 4>(v, keep, pys, px, near, norm, c, t);
+      case 1: column_factors<T, N, TX, 1, NEAR>(v, keep, pys, px, near, norm, c, t); break;
+      case 2: column_factors<T, N, TX, 2, NEAR>(v, keep, pys, px, near, norm, c, t); break;
+      case 3: column_factors<T, N, TX, 3, NEAR>(v, keep, pys, px, near, norm, c, t); break;
+      default: column_factors<T, N, TX, 4, NEAR>(v, keep, pys, px, near, norm, c, t);
     }
   }
   __syncthreads();
@@ -953,10 +955,12 @@ k_power_finalize(const double* __restrict__ part, const FinalParams F, const dou
 // ---------------------------------------------------------------------------------------------
 template <int N> constexpr bool ytx_ok(int tx) { return tx <= N && N % tx == 0 && tx * N / 8 <= 1024; }
 
+constexpr int default_ytx(int n) { return n >= 1024 ? 4 : (n >= 512 ? 8 : 16); }
+
 int ytx_for(const npc_ctx* ctx, int n, bool fp64) {
   auto it = ctx->ytx.find(n * 2 + (fp64 ? 1 : 0));
   if (it != ctx->ytx.end()) return it->second;
-  return n >= 1024 ? 4 : (n >= 512 ? 8 : 16);
+  return default_ytx(n);
 }
 
 template <typename T, int N, int TX>
@@ -990,7 +994,7 @@ npc_status y_pass(npc_ctx* ctx, cplx<T>* data, int nplanes, const cplx<T>* tw, i
   return set_err(ctx, NPC_ERR_INVALID_ARG, "y pass: unsupported columns per CTA %d", tx);
 }
 
-template <typename T, int N, int TX>
+template <typename T, int N, int TX, bool NEAR = false>
 npc_status y_pass_weighted_tx(npc_ctx* ctx, cplx<T>* half, const SignalList& sl, const T* coords, T near,
                               const YNorm& nrm, const cplx<T>* tw, int KZ, int row_n2max) {
   using C = cplx<T>;
@@ -998,7 +1002,7 @@ npc_status y_pass_weighted_tx(npc_ctx* ctx, cplx<T>* half, const SignalList& sl,
     return set_err(ctx, NPC_ERR_INVALID_ARG, "y pass: %d columns per CTA not valid at n = %d", TX, N);
   } else {
     const size_t smem = sizeof(C) * (N + col_rows<N, TX>() * TX + N * TX);
-    auto kern = k_fft_cols_weighted<T, N, TX>;
+    auto kern = k_fft_cols_weighted<T, N, TX, NEAR>;
     NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
     const int nplanes = sl.n * KZ;   // at most 32 x 512
     kern<<<dim3(N / TX, nplanes), TX * N / 8, smem, ctx->stream>>>(half, sl, coords, near, nrm, tw, KZ, row_n2max);
@@ -1009,7 +1013,9 @@ npc_status y_pass_weighted_tx(npc_ctx* ctx, cplx<T>* half, const SignalList& sl,
 
 template <typename T, int N>
 npc_status y_pass_weighted(npc_ctx* ctx, cplx<T>* half, const SignalList& sl, const T* coords, T near,
-                           const YNorm& nrm, const cplx<T>* tw, int tx, int KZ, int row_n2max) {
+                           bool near_columns, const YNorm& nrm, const cplx<T>* tw, int tx, int KZ, int row_n2max) {
+  if (near_columns)
+    return y_pass_weighted_tx<T, N, default_ytx(N), true>(ctx, half, sl, coords, near, nrm, tw, KZ, row_n2max);
   // 32 columns of the longest FP64 lines and their copy would not fit an SM's shared memory
   if (sizeof(cplx<T>) * N * tx * 2 > 150 * 1024) tx = 16;
   switch (tx) {
@@ -1083,8 +1089,15 @@ npc_status fwd_impl(npc_ctx* ctx, const PowerPlan& plan, const Geom& g, const vo
   for (int a = 0; a < 3; ++a) far = std::max(far, std::fabs(g.o[a] - g.obs[a]) + g.h * N);
   const double unit = std::ldexp(1.0, -std::ilogb(far));
   const T near = (T)std::ldexp(1.0, std::ilogb(0.5 * g.h * unit));
+  bool near_columns = false;
   T* coords = nullptr;
   if (directions) {
+    bool close[2] = {false, false};   // k_axis_coords has a value below `near` on the x, on the y axis
+    for (int a = 0; a < 2; ++a)
+      for (int j = 0; j < N; ++j)
+        for (double shift : {0.0, 0.5})
+          close[a] |= std::fabs((T)((g.o[a] + ((double)j - shift) * g.h - g.obs[a]) * unit)) < near;
+    near_columns = close[0] && close[1];
     NPC_TRY(ws_get(ctx, "fwd.coords", sizeof(T) * 6 * N, (void**)&coords));
     k_axis_coords<T><<<(6 * N + 255) / 256, 256, 0, ctx->stream>>>(g, unit, coords);
     NPC_LAUNCH(ctx);
@@ -1098,7 +1111,7 @@ npc_status fwd_impl(npc_ctx* ctx, const PowerPlan& plan, const Geom& g, const vo
     kern<<<dim3(N / (2 * STX), N), SingleCfg<N>::THREADS, ssmem, ctx->stream>>>((const T*)mesh_a, (C*)half, tw, KZ);
   } else {
     const size_t smem = sizeof(C) * (N + col_rows<N, TX>() * TX) + sizeof(T) * (mesh_b ? 2 : 1) * N * TX;
-    auto kern = k_fwd_z<T, N>;
+    auto kern = near_columns ? k_fwd_z<T, N, true> : k_fwd_z<T, N, false>;
     NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
     kern<<<dim3(N / TX, N), ColCfg<N>::THREADS, smem, ctx->stream>>>((const T*)mesh_a, (const T*)mesh_b, (C*)half, sl,
                                                                      coords, (T)(g.h * (N / 8) * unit), near, nrm, tw, KZ);
@@ -1108,7 +1121,8 @@ npc_status fwd_impl(npc_ctx* ctx, const PowerPlan& plan, const Geom& g, const vo
   const int n2max = plan.row_n2max > 0 ? plan.row_n2max : (1 << 30);
   // planes (f, kz) are contiguous N*N blocks; y rows have stride N
   if (weighted)
-    NPC_TRY((y_pass_weighted<T, N>(ctx, (C*)half, sl, coords, near, nrm, tw, ytx_for(ctx, N, sizeof(T) == 8), KZ, n2max)));
+    NPC_TRY((y_pass_weighted<T, N>(ctx, (C*)half, sl, coords, near, near_columns, nrm, tw,
+                                   ytx_for(ctx, N, sizeof(T) == 8), KZ, n2max)));
   else
     NPC_TRY((y_pass<T, N>(ctx, (C*)half, plan.fl.nf * KZ, tw, ytx_for(ctx, N, sizeof(T) == 8), KZ, n2max)));
   NPC_TRY(stage_mark(ctx, "fft_y"));

@@ -53,6 +53,8 @@ def _spec(n, box, origin, observer, interlace, **kw):
     (32, 1000.0, (12.7,) * 3, (NEXT,) * 3),                   # a grid point 1e-13 off on every axis
     (32, 1000.0, (12.7,) * 3, (NEXT, 512.7, 300.0)),          # grid lines along y and z through the observer
     (32, 1000.0, (-484.375, -484.375, -900.0), (0.0,) * 3),   # a column of the shifted phase through the observer
+    (32, 1000.0, (-507.99, -507.99, -500.0), (0.0,) * 3),     # a column within the 8 that count as near ...
+    (32, 1000.0, (-508.01, -507.99, -500.0), (0.0,) * 3),     # ... and none
 ])
 def test_multipoles_with_the_observer_on_a_grid_line(api, n, box, origin, observer, interlace, prec, tol):
     g, r = _around(observer, origin, box, box / n, np.float64 if prec == "fp64" else np.float32)
