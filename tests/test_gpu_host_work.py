@@ -1,0 +1,31 @@
+"""Host work of a small measurement: nothing between the passes grows with the fields' number."""
+import time
+
+import pytest
+
+pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from synthetic import make_survey_catalogs  # noqa: E402
+from helpers import ensure_built  # noqa: E402
+
+
+def test_call_time_of_more_harmonics():
+    """At 16^3 the 20 additional fields of l = 1, 3 cost the device some tens of microseconds.  A search for
+    the fields' float32 coefficients in every call took 8 us each, 160 us together; half of that separates
+    the two."""
+    ensure_built()
+    from paper_2605_04864_gb300 import api
+
+    g, r, origin = make_survey_catalogs(500, 2_000, 500.0, 900.0, 16, seed=3, fkp_p0=1e4)
+
+    def best(ells):
+        times = []
+        for _ in range(60):
+            t = time.perf_counter()
+            api.power_multipoles(g, r, n=16, box=500.0, origin=origin, kbins=(0.0, 0.02, 4), ells=ells, precision="mixed")
+            times.append(time.perf_counter() - t)
+        return min(times)
+
+    best((0, 2, 4))
+    assert best((0, 1, 2, 3, 4)) - best((0, 2, 4)) <= 80e-6
