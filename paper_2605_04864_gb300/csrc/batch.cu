@@ -210,6 +210,7 @@ npc_status batch_exec(npc_ctx* ctx, int nitems, const npc_batch_item* items, uin
   NPC_TRY(ensure_branches(ctx, nb));
   for (int b = 0; b < nb; ++b) {
     ctx->subs[b]->ytx = ctx->ytx;
+    ctx->subs[b]->ytxw = ctx->ytxw;
     ctx->subs[b]->use_tcgen05 = ctx->use_tcgen05;
     ctx->subs[b]->wait_limit = ctx->wait_limit;
   }

@@ -215,6 +215,7 @@ struct npc_ctx {
   std::map<std::string, struct BatchGraph*> graphs;
   int batch_branches = 0;              // 0: not tuned (default 4)
   std::map<int, int> ytx;              // tuned columns per CTA of the y pass, per (n * 2 + fp64)
+  std::map<int, int> ytxw;             // the same with column factors
   cudaStream_t batch_hub = nullptr;    // stream the batch graphs are captured on and launched from
   std::map<const void*, size_t> kernel_smem;                            // allow_smem: limit given per kernel
   std::map<std::tuple<const void*, int, size_t>, int> kernel_ctas;      // ctas_per_sm answers
@@ -345,7 +346,7 @@ npc_status power_core(npc_ctx* ctx, const npc_mesh_spec& ms, const DevCatalog& d
                       const npc_kbins& kb, uint32_t ell_mask, uint32_t modified_mask, int prec, const double* sc,
                       double* dev_out);
 
-// Autotuner of the y pass (columns per CTA) for mesh size n; the choice is kept in ctx->ytx.
+// Autotuner of the y pass (columns per CTA) for mesh size n; the choices are kept in ctx->ytx and ctx->ytxw.
 npc_status tune_y_pass(npc_ctx* ctx, int n, int prec, int nplanes);
 
 npc_status run_forward_transforms(npc_ctx* ctx, int prec, const PowerPlan& plan, const Geom& g,

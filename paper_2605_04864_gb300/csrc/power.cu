@@ -977,12 +977,23 @@ k_power_finalize(const double* __restrict__ part, const FinalParams F, const dou
 // ---------------------------------------------------------------------------------------------
 template <int N> constexpr bool ytx_ok(int tx) { return tx <= N && N % tx == 0 && tx * N / 8 <= 1024; }
 
-constexpr int default_ytx(int n) { return n >= 1024 ? 4 : (n >= 512 ? 8 : 16); }
+// with column factors: a second copy of the columns has to fit an SM's shared memory as well
+template <typename T, int N> constexpr size_t ytxw_smem(int tx) {
+  return sizeof(cplx<T>) * (N + (size_t)(tx < 16 ? N + N / 8 : N) * tx + (size_t)N * tx);
+}
+template <typename T, int N> constexpr bool ytxw_ok(int tx) { return ytx_ok<N>(tx) && ytxw_smem<T, N>(tx) <= 227 * 1024; }
 
+constexpr int default_ytx(int n) { return n >= 1024 ? 4 : (n >= 512 ? 8 : 16); }
+template <typename T, int N> constexpr int default_ytxw() { return default_ytx(N); }
+
+// the tuned width of the plain y pass, else the default
 int ytx_for(const npc_ctx* ctx, int n, bool fp64) {
   auto it = ctx->ytx.find(n * 2 + (fp64 ? 1 : 0));
-  if (it != ctx->ytx.end()) return it->second;
-  return default_ytx(n);
+  return it != ctx->ytx.end() ? it->second : default_ytx(n);
+}
+template <typename T, int N> int ytxw_for(const npc_ctx* ctx) {
+  auto it = ctx->ytxw.find(N * 2 + (sizeof(T) == 8 ? 1 : 0));
+  return it != ctx->ytxw.end() ? it->second : default_ytxw<T, N>();
 }
 
 template <typename T, int N, int TX>
@@ -1020,10 +1031,11 @@ template <typename T, int N, int TX, bool NEAR = false>
 npc_status y_pass_weighted_tx(npc_ctx* ctx, cplx<T>* half, const SignalList& sl, const T* coords, T near,
                               const YNorm& nrm, const cplx<T>* tw, int KZ, int row_n2max) {
   using C = cplx<T>;
-  if constexpr (!ytx_ok<N>(TX)) {
+  if constexpr (!ytxw_ok<T, N>(TX)) {
     return set_err(ctx, NPC_ERR_INVALID_ARG, "y pass: %d columns per CTA not valid at n = %d", TX, N);
   } else {
-    const size_t smem = sizeof(C) * (N + col_rows<N, TX>() * TX + N * TX);
+    constexpr size_t smem = ytxw_smem<T, N>(TX);
+    static_assert(smem == sizeof(C) * (N + col_rows<N, TX>() * TX + N * TX), "shared memory of the kernel");
     auto kern = k_fft_cols_weighted<T, N, TX, NEAR>;
     NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
     const int nplanes = sl.n * KZ;   // at most 32 x 512
@@ -1037,9 +1049,7 @@ template <typename T, int N>
 npc_status y_pass_weighted(npc_ctx* ctx, cplx<T>* half, const SignalList& sl, const T* coords, T near,
                            bool near_columns, const YNorm& nrm, const cplx<T>* tw, int tx, int KZ, int row_n2max) {
   if (near_columns)
-    return y_pass_weighted_tx<T, N, default_ytx(N), true>(ctx, half, sl, coords, near, nrm, tw, KZ, row_n2max);
-  // 32 columns of the longest FP64 lines and their copy would not fit an SM's shared memory
-  if (sizeof(cplx<T>) * N * tx * 2 > 150 * 1024) tx = 16;
+    return y_pass_weighted_tx<T, N, default_ytxw<T, N>(), true>(ctx, half, sl, coords, near, nrm, tw, KZ, row_n2max);
   switch (tx) {
     case 4: return y_pass_weighted_tx<T, N, 4>(ctx, half, sl, coords, near, nrm, tw, KZ, row_n2max);
     case 8: return y_pass_weighted_tx<T, N, 8>(ctx, half, sl, coords, near, nrm, tw, KZ, row_n2max);
@@ -1049,28 +1059,21 @@ npc_status y_pass_weighted(npc_ctx* ctx, cplx<T>* half, const SignalList& sl, co
   return set_err(ctx, NPC_ERR_INVALID_ARG, "y pass: unsupported columns per CTA %d", tx);
 }
 
-// Autotuner for the y pass: times every valid columns-per-CTA choice on a scratch buffer of
-// `nplanes` planes (values irrelevant to the timing) and keeps the fastest for (n, precision).
-template <typename T, int N>
-npc_status tune_y_impl(npc_ctx* ctx, int nplanes) {
-  using C = cplx<T>;
-  const void* twp;
-  NPC_TRY(get_twiddles(ctx, N, sizeof(T) == 8 ? NPC_PREC_FP64 : NPC_PREC_MIXED, &twp));
-  C* buf;
-  NPC_TRY(ws_get(ctx, "tune.y", sizeof(C) * (size_t)nplanes * N * N, (void**)&buf));
-  NPC_CUDA(ctx, cudaMemsetAsync(buf, 0, sizeof(C) * (size_t)nplanes * N * N, ctx->stream));
+// Autotuner for the y pass: times every valid columns-per-CTA choice of both forms (plain and with column
+// factors, which needs twice the shared memory per column) on a scratch buffer of `nplanes` planes (values
+// irrelevant to the timing) and keeps the fastest of each for (n, precision).
+template <typename Run>
+npc_status fastest_width(npc_ctx* ctx, const std::vector<int>& widths, Run&& run, int* best_tx) {
   cudaEvent_t e0, e1;
   NPC_CUDA(ctx, cudaEventCreate(&e0));
   NPC_CUDA(ctx, cudaEventCreate(&e1));
   float best = 1e30f;
-  int best_tx = ytx_for(ctx, N, sizeof(T) == 8);
   npc_status st = NPC_OK;
-  for (int tx : {4, 8, 16, 32}) {
-    if (!(tx <= N && N % tx == 0 && tx * N / 8 <= 1024)) continue;
-    st = y_pass<T, N>(ctx, buf, nplanes, (const C*)twp, tx);  // warm-up
+  for (int tx : widths) {
+    st = run(tx);  // warm-up
     if (st != NPC_OK) break;
     cudaEventRecord(e0, ctx->stream);
-    for (int rep = 0; rep < 3 && st == NPC_OK; ++rep) st = y_pass<T, N>(ctx, buf, nplanes, (const C*)twp, tx);
+    for (int rep = 0; rep < 3 && st == NPC_OK; ++rep) st = run(tx);
     cudaEventRecord(e1, ctx->stream);
     if (st != NPC_OK) break;
     cudaEventSynchronize(e1);
@@ -1078,13 +1081,45 @@ npc_status tune_y_impl(npc_ctx* ctx, int nplanes) {
     cudaEventElapsedTime(&ms, e0, e1);
     if (ms < best) {
       best = ms;
-      best_tx = tx;
+      *best_tx = tx;
     }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (st != NPC_OK) return st;
-  ctx->ytx[N * 2 + (sizeof(T) == 8 ? 1 : 0)] = best_tx;
+  return st;
+}
+
+template <typename T, int N>
+npc_status tune_y_impl(npc_ctx* ctx, int nplanes) {
+  using C = cplx<T>;
+  constexpr bool fp64 = sizeof(T) == 8;
+  const void* twp;
+  NPC_TRY(get_twiddles(ctx, N, fp64 ? NPC_PREC_FP64 : NPC_PREC_MIXED, &twp));
+  const C* tw = (const C*)twp;
+  C* buf;
+  T* coords;
+  NPC_TRY(ws_get(ctx, "tune.y", sizeof(C) * (size_t)nplanes * N * N, (void**)&buf));
+  NPC_TRY(ws_get(ctx, "tune.coords", sizeof(T) * 6 * N, (void**)&coords));
+  NPC_CUDA(ctx, cudaMemsetAsync(buf, 0, sizeof(C) * (size_t)nplanes * N * N, ctx->stream));
+  NPC_CUDA(ctx, cudaMemsetAsync(coords, 0, sizeof(T) * 6 * N, ctx->stream));
+  std::vector<int> plain, weighted;
+  for (int tx : {4, 8, 16, 32}) {
+    if (ytx_ok<N>(tx)) plain.push_back(tx);
+    if (ytxw_ok<T, N>(tx)) weighted.push_back(tx);
+  }
+  int tx = default_ytx(N), txw = default_ytxw<T, N>();
+  NPC_TRY(fastest_width(ctx, plain, [&](int w) { return y_pass<T, N>(ctx, buf, nplanes, tw, w); }, &tx));
+  SignalList sl{};   // phases a and b of Y_21: two signals read, four fields written
+  sl.n = 2;
+  for (int8_t ph = 0; ph < 2; ++ph) sl.s[ph] = Signal{ph, 2, 1, (int8_t)(2 * ph), (int8_t)(2 * ph + 1)};
+  const YNorm nrm = ylm_norm_table();
+  const int kz = std::max(1, std::min(nplanes / 4, N / 2));
+  if (nplanes >= 4)
+    NPC_TRY(fastest_width(ctx, weighted, [&](int w) {
+      return y_pass_weighted<T, N>(ctx, buf, sl, coords, T(0), false, nrm, tw, w, kz, 1 << 30);
+    }, &txw));
+  ctx->ytx[N * 2 + fp64] = tx;
+  ctx->ytxw[N * 2 + fp64] = txw;
   return NPC_OK;
 }
 
@@ -1144,7 +1179,7 @@ npc_status fwd_impl(npc_ctx* ctx, const PowerPlan& plan, const Geom& g, const vo
   // planes (f, kz) are contiguous N*N blocks; y rows have stride N
   if (weighted)
     NPC_TRY((y_pass_weighted<T, N>(ctx, (C*)half, sl, coords, near, near_columns, nrm, tw,
-                                   ytx_for(ctx, N, sizeof(T) == 8), KZ, n2max)));
+                                   ytxw_for<T, N>(ctx), KZ, n2max)));
   else
     NPC_TRY((y_pass<T, N>(ctx, (C*)half, plan.fl.nf * KZ, tw, ytx_for(ctx, N, sizeof(T) == 8), KZ, n2max)));
   NPC_TRY(stage_mark(ctx, "fft_y"));
