@@ -567,7 +567,7 @@ __device__ __forceinline__ double from_fixed(long long q, double inv) { return (
 //     a return value; no word can overflow (1023 * 2^21 < 2^31).  10 cycles at 671 objects.
 //   float, more objects: the adds return the old word, so that an overflow of l is carried into h
 //     (2^32 = 1024 * 2^22) and one of h into the cell's signed byte of a third array (the whole sum is
-//     below 2^60, so h overflows at most 2^38 / 2^32 = 64 times either way).  9 cycles at 20,000
+//     at most 127/128 of 2^61, so h overflows at most 127 times either way).  9 cycles at 20,000
 //     objects, where the tile's clearing and writing no longer count.
 //   double: low and high halves of the 64-bit integer, the high add taking the carry of the low one.
 constexpr int NARROW_MAX = 1023;
@@ -702,13 +702,14 @@ k_paint_brick(const typename RecOf<T>::type* __restrict__ rec, const uint32_t* _
     // fixed-point scale 2^e with cnt * max|w| * 2^e < 2^61 (no overflow of the tile sums)
     const double bound = (double)cnt * sc[maxw_slot];
     int ex = 0;
-    if (bound > 0) frexp(bound, &ex);
+    double mant = 0.0;
+    if (bound > 0) mant = frexp(bound, &ex);
     int e = 61 - ex;
     if constexpr (sizeof(T) == 4) {
-      // float: below 2^60 (the words' range) and every tap |w W| 2^e < 2^43 (that of fixed_parts)
+      // float: at most 127/128 of 2^61 (the words' range) and every tap |w W| 2^e < 2^43 (that of fixed_parts)
       int exw = 0;
       if (sc[maxw_slot] > 0) frexp(sc[maxw_slot], &exw);
-      e = max(-126, min(126, min(e - 1, 43 - exw)));
+      e = max(-126, min(126, min(mant > 127.0 / 128.0 ? e - 1 : e, 43 - exw)));
     }
     s_exp = e;
   }

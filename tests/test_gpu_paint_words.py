@@ -14,7 +14,8 @@ EPS = 2.0**-24
 
 def _parts(w, cnt):
     """The kernel's split of a whole tap: w 2^e = 2^22 h + l with both |h|, |l| <= 2^21."""
-    e = min(60 - np.frexp(float(cnt) * float(np.abs(w).max()))[1], 43 - np.frexp(float(np.abs(w).max()))[1])
+    mant, ex = np.frexp(float(cnt) * float(np.abs(w).max()))
+    e = min((60 if mant > 127 / 128 else 61) - ex, 43 - np.frexp(float(np.abs(w).max()))[1])
     v = w.astype(np.float64) * 2.0**e
     h = np.rint(v / 2.0**22)
     return h, v - h * 2.0**22
@@ -72,3 +73,23 @@ def test_high_word_of_both_signs():
     cells, weights, counts = [(33, 34, 35), (33, 34, 35), (36, 34, 35)], [w, -w, w], [20_000, 16_000, 3_000]
     pos, wt = _objects(cells, weights, counts)
     _check(pos, wt, cells, weights, counts)
+
+
+def test_smallest_unit_of_a_full_brick():
+    """300,000 objects of weights +1 and -1 in a brick (2^18 < 300,000 < 2^19) leave 2^-42 as the unit of the
+    tile's sums: a lone weight of 2^-42 keeps its value.  With a unit of 2^-41 it is a tie and rounds to 0."""
+    cells, weights, counts = [(2, 2, 2), (5, 2, 2), (9, 9, 9)], [1.0, -1.0, 2.0**-42], [150_000, 150_000, 1]
+    pos, wt = _objects(cells, weights, counts)
+    got = _paint(pos, wt, N, float(N), 2)
+    assert abs(got[9, 9, 9] - 2.0**-42) <= 2.0**-42 * 2.0**-10
+
+
+@pytest.mark.parametrize("cells,count", [([(3, 3, 3)], 262_144), ([(3, 3, 3), (4, 3, 3)], 131_072), ([(3, 3, 3)], 260_000)])
+@pytest.mark.parametrize("sign", [1, -1])
+def test_fullest_cells(cells, count, sign):
+    """Weights just below 2 on one or two points, bounds on either side of 127/128 of a power of two: the digits
+    of the high word come to +-64 and +-127."""
+    w = sign * (2.0 - 2.0**-22)
+    weights = [w, -w][: len(cells)]
+    pos, wt = _objects(cells, weights, [count] * len(cells))
+    _check(pos, wt, cells, weights, [count] * len(cells))
