@@ -170,9 +170,9 @@ npc_status npc_catalog_scalars(npc_ctx* ctx, const npc_catalog* data, const npc_
  * synchronisation).  It computes out[0..7] as npc_catalog_scalars defines them, but needs no
  * context and allocates nothing: its scratch (per-block partial sums) is a static device array of
  * 786,560 bytes that every device which loads the library holds until the process exits.  Its
- * reduction tree depends on n (one block per 4,096 objects, where the context call always sums
- * 1,024 fixed blocks), so the two calls agree to rounding (about 1e-12 relative), not bit for
- * bit; repeated calls on the same inputs are bitwise identical.
+ * reduction tree depends on n (one block per 4,096 objects, where the context call stops at four
+ * blocks per SM), so the two calls agree to rounding (about 1e-12 relative), not bit for bit;
+ * repeated calls on the same inputs are bitwise identical.
  *   - data / randoms: device pointers only (on_device = 1), at most 33,554,432 objects each,
  *     otherwise NPC_ERR_INVALID_ARG with a message in `err`; randoms == NULL means a periodic box.
  *   - out_device: 8 doubles of device memory; the call is asynchronous on `cuda_stream` (NULL:

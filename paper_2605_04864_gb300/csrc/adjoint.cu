@@ -506,7 +506,9 @@ k_adj_z(cplx<T>* __restrict__ T2, const AFieldTable* __restrict__ ftp, const int
   }
 }
 
-template <int N> struct AWrite {   // column pairs per CTA
+// Column pairs per CTA: 16 where 32 divides the mesh (256^3: 26.6 us, 28.7 with 8) and 8 from 512 on (512^3: 0.195
+// ms, as with 16; 0.280 with 4; 1024^3: 2.1 ms, 3.1 with 4).
+template <int N> struct AWrite {
   static constexpr int TX = N >= 512 || N % 32 ? 8 : 16;
   static constexpr int THREADS = TX * N / 8;
 };

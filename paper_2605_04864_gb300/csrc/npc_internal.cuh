@@ -51,10 +51,6 @@ __device__ __forceinline__ double2 csub_packed(double2 a, double2 b) { return cs
 template <int SIGN, typename C> __device__ __forceinline__ C csub_i(C a, C b) {
   return SIGN < 0 ? cmk(a.y - b.y, b.x - a.x) : cmk(b.y - a.y, a.x - b.x);
 }
-// multiply by (sign * i): sign = -1 gives -i, +1 gives +i
-template <int SIGN, typename C> __host__ __device__ __forceinline__ C cmul_i(C a) {
-  return SIGN < 0 ? cmk(a.y, -a.x) : cmk(-a.y, a.x);
-}
 
 // ---------------------------------------------------------------------------------------------
 // Spherical harmonics Y_l^m (m >= 0, Condon-Shortley phase) at a unit vector, l <= 8.
@@ -100,56 +96,15 @@ __device__ __forceinline__ void ylm_eval(int l, int m, T x, T y, T z, const YNor
   im = c * pim;
 }
 
-// Closed forms of Q_lm for l in {2, 4} (expanded from the recurrence above), falling back to
-// the recurrence otherwise.  (x, y, z) is a unit vector.
-template <typename T>
-__device__ __forceinline__ void ylm_fast(int l, int m, T x, T y, T z, const YNorm& nrm, T& re, T& im) {
-  const T z2 = z * z;
-  T q;
-  switch (l * 16 + m) {
-    case 0x00: re = ynorm<T>(nrm, 0); im = T(0); return;
-    case 0x20: q = T(1.5) * z2 - T(0.5); break;
-    case 0x21: q = T(-3) * z; break;
-    case 0x22: q = T(3); break;
-    case 0x40: q = (T(35) * z2 * z2 - T(30) * z2 + T(3)) * T(0.125); break;
-    case 0x41: q = T(-2.5) * z * (T(7) * z2 - T(3)); break;
-    case 0x42: q = T(7.5) * (T(7) * z2 - T(1)); break;
-    case 0x43: q = T(-105) * z; break;
-    case 0x44: q = T(105); break;
-    default: ylm_eval<T>(l, m, x, y, z, nrm, re, im); return;
-  }
-  T pr = T(1), pim = T(0);
-  for (int j = 0; j < m; ++j) {
-    const T nr = pr * x - pim * y;
-    pim = pr * y + pim * x;
-    pr = nr;
-  }
-  const T c = ynorm<T>(nrm, l * (l + 1) / 2 + m) * q;
-  re = c * pr;
-  im = c * pim;
-}
-
-// Legendre polynomial L_l(mu), l <= 8 (Bonnet recurrence).
-template <typename T> __device__ __forceinline__ T legendre_p(int l, T mu) {
-  if (l == 0) return T(1);
-  T p0 = T(1), p1 = mu;
-  for (int ll = 2; ll <= l; ++ll) {
-    const T p2 = (T(2 * ll - 1) * mu * p1 - T(ll - 1) * p0) / T(ll);
-    p0 = p1;
-    p1 = p2;
-  }
-  return p1;
-}
-
 // ---------------------------------------------------------------------------------------------
 // Field descriptors for the forward transforms
 // ---------------------------------------------------------------------------------------------
-enum : int8_t { PART_RE = 0, PART_IM = 1, PART_ONE = 2, PART_ZERO = 3 };
+enum : int8_t { PART_RE = 0, PART_IM = 1, PART_ONE = 2 };
 
 struct Comp {          // one real field: mesh phase x weight function
   int8_t phase;        // 0 or 1
   int8_t ell, m;       // Y_l^m (m >= 0)
-  int8_t part;         // PART_RE / PART_IM of Y_l^m, PART_ONE (global LOS), PART_ZERO
+  int8_t part;         // PART_RE / PART_IM of Y_l^m, PART_ONE (no weight: F_0, global LOS)
   int8_t tracer = 0;   // 1: F_0 of the first tracer A of a cross spectrum (the others are B's)
 };
 
@@ -157,7 +112,7 @@ constexpr int NPC_MAX_FIELDS = 56;  // real fields per call (2 phases x 25 for l
 
 struct FieldList {
   int nf;                     // number of real fields
-  Comp f[NPC_MAX_FIELDS];     // real field f; forward pairs are (2p, 2p+1)
+  Comp f[NPC_MAX_FIELDS];     // real field f, at half spectrum f after the forward passes
 };
 
 // Geometry needed to evaluate xhat at a grid point.

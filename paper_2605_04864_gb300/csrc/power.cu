@@ -59,7 +59,7 @@ template <int N> struct SingleCfg {   // column pairs per CTA: 2 TX divides N, T
 
 // The two columns' values are neighbours in memory: one 8-byte load when the mesh is aligned to it (VEC).
 template <typename T, int N, bool VEC>
-__global__ void __launch_bounds__(SingleCfg<N>::THREADS, (sizeof(T) == 4 && SingleCfg<N>::THREADS == 512 ? 2 : 1))
+__global__ void __launch_bounds__(SingleCfg<N>::THREADS, 1)
 k_fwd_z_single(const T* __restrict__ mesh, cplx<T>* __restrict__ half, const cplx<T>* __restrict__ tw_g, int KZ) {
   using C = cplx<T>;
   constexpr int TX = SingleCfg<N>::TX;
@@ -583,7 +583,6 @@ struct ContractParams {
   SumDesc sum[MAX_PRODS];
   int global_los;
   double los[3];
-  int assign;
   double kf;
 };
 
@@ -604,7 +603,6 @@ template <typename T> __device__ __forceinline__ T legendre_0to4(int l, T mu) {
 template <int N> struct XTeam {
   static constexpr int TPF = N / 8;
   static constexpr bool BLOCK = !(TPF % 32 == 0 || 32 % TPF == 0);
-  static constexpr int SIZE = TPF > 32 ? TPF : 32;   // of a team, unless BLOCK
   // exchange buffers per row: two where every exchange of the transform writes the other one, which
   // leaves one barrier per exchange
   static constexpr int XBUF = BLOCK ? 1 : 2;
@@ -613,6 +611,7 @@ template <int N> struct XTeam {
   static constexpr int ROW = XBUF * row_pad_len<N>() + (TPF < 16 ? TPF : 0);
   // threads per CTA: whole warps of whole rows for the lengths 3 * 2^k
   static constexpr int THREADS = BLOCK ? 96 : CONTRACT_THREADS;
+  static_assert(THREADS % TPF == 0, "whole rows");
 };
 
 // v[q] (mode kx = t + q TPF) times the step's scale * the part of Q_LM(uz) (ux + i uy)^M, added to acc.
@@ -645,7 +644,7 @@ __device__ __forceinline__ void add_weighted(cplx<T> (&acc)[8], const cplx<T> (&
 // wait for each other.  The modes (kx, ky) with either sign of each have one |k|, hence one bin: all four
 // (the two signs of kx where rows are not paired) are added before the warp-segmented scan.
 template <typename T, int N, int MINB>
-__global__ void __launch_bounds__(CONTRACT_THREADS, MINB)
+__global__ void __launch_bounds__(XTeam<N>::THREADS, MINB)
 k_fft_x_contract(const cplx<T>* __restrict__ half, const __grid_constant__ ContractParams P,
                  const int16_t* __restrict__ bintab, const cplx<T>* __restrict__ tw_g,
                  const cplx<T>* __restrict__ factors, double* __restrict__ part) {
@@ -655,12 +654,11 @@ k_fft_x_contract(const cplx<T>* __restrict__ half, const __grid_constant__ Contr
   constexpr int NP = row_pad_len<N>();
   const int G = blockDim.x / TPF;             // rows in flight
   const int nw = blockDim.x >> 5;
-  const int nbuf = G + (Team::BLOCK && blockDim.x % TPF ? 1 : 0);   // threads left over transform zeros
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* phs = tw + N;                            // e^{i pi m/N}, m = -N .. N-1
-  C* rowbuf = phs + 2 * N;                    // [nbuf][ROW]
-  C* fsm = rowbuf + (size_t)nbuf * Team::ROW;   // [G][1 or 2 rows][nacc][N]
+  C* rowbuf = phs + 2 * N;                    // [G][ROW]
+  C* fsm = rowbuf + (size_t)G * Team::ROW;   // [G][1 or 2 rows][nacc][N]
   const int nslot = P.pair_rows ? 2 : 1;
   T* winv = reinterpret_cast<T*>(fsm + (size_t)G * nslot * P.nacc * N);   // 1/sinc^p, a = 0..N/2
   double* spart = reinterpret_cast<double*>(smem_raw + (((reinterpret_cast<unsigned char*>(winv + N / 2 + 2) - smem_raw) + 15) & ~(size_t)15));
@@ -674,7 +672,6 @@ k_fft_x_contract(const cplx<T>* __restrict__ half, const __grid_constant__ Contr
   __syncthreads();
   double* mypart = P.shared_part ? spart + (size_t)warp * nent : part + ((size_t)blockIdx.x * nw + warp) * nent;
   const int g = tid / TPF, t = tid % TPF;
-  const bool ingroup = g < G;
   const size_t fstride = (size_t)P.KZ * N * N;
   const T half_or_one = P.nphase == 2 ? T(0.5) : T(1);
   // items (kz, |ky|), ky >= 0 before -ky
@@ -693,10 +690,10 @@ k_fft_x_contract(const cplx<T>* __restrict__ half, const __grid_constant__ Contr
     return half + ((size_t)kz * N + (sgn && ay ? N - ay : ay)) * N;
   };
   // team-uniform loop: a team's groups (rows of one warp, or of the block) go on until none has an item
-  int item = ingroup ? blockIdx.x * G + g : nitems;
+  int item = blockIdx.x * G + g;
   if (!Team::BLOCK) item = seek(item);
   int pass = 0, flip = 0;
-  C* bufs = rowbuf + (size_t)(ingroup ? g : G) * Team::ROW;
+  C* bufs = rowbuf + (size_t)g * Team::ROW;
   C v[8], vn[8];
   if (in_bins(item)) {
     const C* src = row_of(item, 0) + (size_t)P.step[0].field * fstride;
@@ -783,12 +780,12 @@ k_fft_x_contract(const cplx<T>* __restrict__ half, const __grid_constant__ Contr
               }
             }
             if (c.flags & STEP_STORE) {
-              C* f = fsm + (((size_t)(ingroup ? g : 0) * nslot + (P.pair_rows ? sgn : 0)) * P.nacc + c.acc) * N;
+              C* f = fsm + (((size_t)g * nslot + (P.pair_rows ? sgn : 0)) * P.nacc + c.acc) * N;
               const T wr = half_or_one * winv[ay] * winv[kz];
 #pragma unroll
               for (int q = 0; q < 8; ++q) {
                 const int ai = q < 4 ? t + q * TPF : (8 - q) * TPF - t;
-                if (ingroup) f[t + q * TPF] = cscale(racc[q], wr * winv[ai]);
+                f[t + q * TPF] = cscale(racc[q], wr * winv[ai]);
                 racc[q] = cmk(T(0), T(0));
               }
             }
@@ -855,7 +852,9 @@ k_fft_x_contract(const cplx<T>* __restrict__ half, const __grid_constant__ Contr
           const unsigned heads = __ballot_sync(0xffffffffu, head);
           const int first = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));   // lane of the run's head
           const bool last = (lane == 31) || ((heads >> (lane + 1)) & 1u);
-          // run sums over at most 32 lanes stay in T; only run ends convert to float64
+          // run sums (of at most 32 lanes, 2 modes each, or 4 with ky and -ky) stay in T; only run ends convert to
+          // float64.  Runs cut to 32 modes have the same errors against 64 bits to three digits (128^3, 96
+          // catalogues; 256^3, 16) and cost 6 % of the pass at 128^3, 36 % with ky and -ky at 256^3.
 #pragma unroll
           for (int e = 0; e < MAX_SUMS; ++e) {
             if (e < MAX_PRODS && e >= P.nprod) continue;
@@ -983,6 +982,8 @@ template <typename T, int N> constexpr size_t ytxw_smem(int tx) {
 }
 template <typename T, int N> constexpr bool ytxw_ok(int tx) { return ytx_ok<N>(tx) && ytxw_smem<T, N>(tx) <= 227 * 1024; }
 
+// Columns per CTA that are not tuned: the fastest of both forms or within 4 % of it in float32 (1024^3: 7 % with
+// column factors), in float64 within 3 % plain and 12 % with column factors (192: 576 us with 4, 646 with 16).
 constexpr int default_ytx(int n) { return n >= 1024 ? 4 : (n >= 512 ? 8 : 16); }
 template <typename T, int N> constexpr int default_ytxw() { return default_ytx(N); }
 
@@ -1267,7 +1268,6 @@ npc_status contract_impl(npc_ctx* ctx, const PowerPlan& plan, const npc_mesh_spe
   P.KZ = plan.kz_keep > 0 ? std::min(plan.kz_keep, N / 2) : N / 2;
   P.global_los = plan.global_los;
   for (int a = 0; a < 3; ++a) P.los[a] = plan.los[a];
-  P.assign = plan.assign;
   P.kf = 2.0 * M_PI / m.box;
   {
     // a mode is binned only if k_f |q| < kmin + nbins dk; its row has ky^2 + kz^2 <= |q|^2
@@ -1280,14 +1280,16 @@ npc_status contract_impl(npc_ctx* ctx, const PowerPlan& plan, const npc_mesh_spe
   // rows ky and -ky), the warps' partial sums where they are small
   auto smem_of = [&](int threads) {
     const int G = threads / XTeam<N>::TPF;
-    const int nbuf = G + (XTeam<N>::BLOCK && threads % XTeam<N>::TPF ? 1 : 0);
-    size_t b = sizeof(C) * ((size_t)3 * N + (size_t)nbuf * XTeam<N>::ROW +
+    size_t b = sizeof(C) * ((size_t)3 * N + (size_t)G * XTeam<N>::ROW +
                             (size_t)G * (P.pair_rows ? 2 : 1) * P.nacc * N) + sizeof(T) * (N / 2 + 2);
     b = (b + 15) & ~(size_t)15;
     if (P.shared_part) b += sizeof(double) * (threads / 32) * P.nbins * P.nsum;
     return b;
   };
   P.pair_rows = P.nacc == 1 ? 1 : 0;
+  // Shared sums save the clearing of the partials and leave the finalize one set per CTA: 10 us of 128^3, 18 of
+  // a 256^3 box (the pass itself is up to 3 % slower); at 512^3 14 us of 7 ms, not taken.  Above 32 KB they
+  // would take the second CTA's shared memory.
   P.shared_part = N <= 256 && sizeof(double) * (CONTRACT_THREADS / 32) * P.nbins * P.nsum <= 32768 ? 1 : 0;
   // fewer threads per CTA where the rows would not fill the SMs four times over (a CTA of 256 threads
   // holds 32 rows at n = 64), or where the shared memory asks for it (FP64 at 256^3 with odd multipoles)
@@ -1297,7 +1299,8 @@ npc_status contract_impl(npc_ctx* ctx, const PowerPlan& plan, const npc_mesh_spe
          (smem_of(threads) > 227 * 1024 || nitems < 4 * ctx->num_sms * (threads / XTeam<N>::TPF)))
     threads /= 2;
   const size_t smem = smem_of(threads);
-  auto kern = k_fft_x_contract<T, N, (sizeof(T) == 4 ? 2 : 1)>;
+  // float32: as many CTAs as 128 registers a thread allow (five of 96 threads: up to 136 without a spill)
+  auto kern = k_fft_x_contract<T, N, (sizeof(T) == 8 ? 1 : (XTeam<N>::BLOCK ? 5 : 2))>;
   NPC_TRY(allow_smem(ctx, (const void*)kern, smem));
   int per_sm = 0;
   NPC_TRY(ctas_per_sm(ctx, (const void*)kern, threads, smem, &per_sm));
