@@ -65,7 +65,8 @@ typedef struct {
   int32_t periodic;    /* 1: periodic box, no randoms (delta = n - mean); 0: survey with randoms */
   int32_t los;         /* 0: endpoint line of sight xhat from `observer`; 1: global `los_dir` */
   double los_dir[3];   /* used when los == 1 (need not be normalised) */
-  double observer[3];  /* used when los == 0 */
+  double observer[3];  /* used when los == 0; anywhere, in the box too: a mesh point exactly at it has the
+                          direction of the z axis */
 } npc_mesh_spec;
 
 /* A catalogue: positions [n][3] (x,y,z interleaved), weights [n], number densities [n]. */
